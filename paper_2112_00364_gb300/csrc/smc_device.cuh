@@ -40,6 +40,22 @@ __device__ __forceinline__ double pow2i(int n) {
 // exact factors 2^(k_t - k_max) instead of exponentials.
 __device__ __forceinline__ int tile_exponent(double M) { return (int)ceil(M * kInvLn2); }
 
+__device__ __forceinline__ float trunc_f32(unsigned hi, unsigned lo);
+
+// tile_exponent off the FP64 pipe (three operations of 16 issue cycles a warp
+// there): in single precision wherever M / ln 2 lies further from an integer than
+// the error of that (below 2.5e-7 relative), else as above.
+__device__ __forceinline__ int tile_exponent_fast(double M) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(M);
+  const unsigned hi = (unsigned)(b >> 32);
+  if ((hi & 0x7fffffffu) < 0x40a00000u) {  // |M| < 2^11
+    const float y = trunc_f32(hi, (unsigned)b) * 1.44269504f;
+    const float c = ceilf(y), band = fabsf(y) * 5e-7f;
+    if (c - y > band && y - (c - 1.0f) > band && y != 0.0f) return (int)c;
+  }
+  return tile_exponent(M);
+}
+
 struct Block4 {
   uint32_t w0, w1, w2, w3;
 };
@@ -85,12 +101,14 @@ __host__ __device__ __forceinline__ Block4 philox(uint32_t c0, uint32_t c1, uint
 // rounded result; special and extreme arguments go to the library functions.
 constexpr int kRsExpN = 36 * 256;      // table points of e^(-j/256), j < kRsExpN
 constexpr int kRsExpPad = kRsExpN + 4;  // then zeros (whole 16-byte pairs)
+constexpr int kExp32N = 1233;           // table points of e^(-j/32): arguments below 38.5 (38.53)
 struct MathTab {
   double log_f[192];    // log(j/128), j = 90..181 used
   double inv_f[192];    // 128 / j, j = 90..181 used
   double inv_f52[192];  // (128 / j) 2^-52 (exact scaling of inv_f)
   double inv_f53[192];  // (128 / j) 2^-53
-  unsigned long long exp2_neg_q63[128];  // round(2^(-j/128) 2^63)
+  unsigned long long exp_neg32_q63[kExp32N];   // round(e^(-j/32) 2^63), the weights' exponential
+  unsigned long long exp_neg2048_q63[64];      // round(e^(-j/2048) 2^63)
   unsigned long long inv_f_q62[192];        // round((128 / j) 2^62), j = 90..181 used
   unsigned long long exp2_neg64_q63[64];    // round(2^(-j/64) 2^63)
   unsigned long long exp2_neg4096_q63[64];  // round(2^(-j/4096) 2^63)
@@ -214,41 +232,38 @@ __device__ __forceinline__ double tang_exp(double x, const MathTab* __restrict__
 // round(e^d 2^B) for d <= 0 (B = 54 for the segment kernel's tiles of at most
 // 256 weights, 50 for the standalone resampler's tiles of 4096, so that a
 // tile's sum stays below 2^62), the weight of a particle relative to a
-// power-of-two reference as a 2^-B fixed-point integer, on the integer pipes
-// (only the argument split is FP64).  e^d = 2^-y with y = -d / ln 2 = n + j/128
-// + r, r < 2^-7: e^d = 2^-n 2^(-j/128) e^(-r ln 2), the last factor by its
-// Taylor series to degree 6 (Horner; all partial sums positive), in 2^-63 fixed
-// point with 64-bit multiply-high products.  Within one unit of the exact
-// rounding; below e^-38.5 (less than half a unit) it returns 0.  A d slightly
-// above 0 (rounding of the reference) is taken as 0.
+// power-of-two reference as a 2^-B fixed-point integer, on the integer pipes.
+// The argument X = -d in 2^-58 units splits by its bits, with no reduction
+// product: X = j1/32 + j2/2048 + r, r < 2^-11, e^-X = T1[j1] T2[j2] (1 - q)
+// with q = 1 - e^-r = r - r^2/2 + r^3/6 - r^4/24 in 2^-64 units (the dropped
+// r^5/120 is below 2^-61), r^2 from the top 32 bits of r and one cross term.
+// Only the absolute error counts (the result is a multiple of 2^-54), so T1
+// holds e^(-j/32) itself in 2^-63 units: two 64-bit multiply-highs, no shift by
+// a power of two; at most 0.02 units of 2^-54 before the one rounding, beside
+// the 2^-58 of the argument.  Bound: issue.  About 60 instructions against about
+// 130 for a power-of-two reduction with a degree-6 series in 64-bit products.
+// Below e^-38.5 (less than half a unit) the weight is 0.  A d slightly above 0
+// (rounding of the reference) is taken as 0.
 constexpr unsigned long long kInvLn2Q63 = 0xb8aa3b295c17f0bcull;  // round(2^63 / ln 2)
 constexpr unsigned long long kLn2Q64 = 0xb17217f7d1cf79acull;     // round(ln 2 2^64)
-
-__device__ __forceinline__ unsigned long long mulhi64(unsigned long long a, unsigned long long b) {
-  return __umul64hi(a, b);
-}
 
 // The core from X = -d 2^58 (an unsigned integer, -d < 38.5).
 template <int B>
 __device__ __forceinline__ long long exp_fix_x(unsigned long long X, const MathTab* __restrict__ T) {
   static_assert(B >= 40 && B <= 54, "fixed-point bits");
-  // Y = X / ln 2 in units of 2^-58: floor(X kInvLn2Q63 / 2^63)
-  const unsigned long long Y = (mulhi64(X, kInvLn2Q63) << 1) | ((X * kInvLn2Q63) >> 63);
-  const int n = (int)(Y >> 58);
-  if (n >= B + 1) return 0;  // at most half a unit
-  const int j = (int)((Y >> 51) & 127);
-  const unsigned long long r = Y & ((1ull << 51) - 1);  // r 2^58, r < 2^-7
-  const unsigned long long t2 = mulhi64(r << 5, kLn2Q64) << 1;  // 2 t 2^63 with t = r ln 2
-  unsigned long long p = 0x2d82d82d82d82eull;                   // 2^63 / 720
-  p = 0x111111111111111ull - mulhi64(t2, p);                     // 2^63 / 120 - t p
-  p = 0x555555555555555ull - mulhi64(t2, p);                     // 2^63 / 24
-  p = 0x1555555555555555ull - mulhi64(t2, p);                    // 2^63 / 6
-  p = 0x4000000000000000ull - mulhi64(t2, p);                    // 2^63 / 2
-  p = 0x8000000000000000ull - mulhi64(t2, p);                    // 2^63
-  p = 0x8000000000000000ull - mulhi64(t2, p);                    // e^-t 2^63
-  const unsigned long long q = mulhi64(p, __ldg(&T->exp2_neg_q63[j])) << 1;  // e^-(j/128 + r) ln 2 2^63
-  const int s = 63 - B + n;  // to 2^-B units and the factor 2^-n
-  return (long long)((q + (1ull << (s - 1))) >> s);
+  const unsigned long long t = __umul64hi(__ldg(&T->exp_neg32_q63[X >> 53]),
+                                          __ldg(&T->exp_neg2048_q63[(X >> 47) & 63]));  // 2^62
+  const unsigned long long r = X & ((1ull << 47) - 1);  // r 2^58
+  const unsigned rh = (unsigned)(r >> 15);              // r 2^43
+  const unsigned rl = (unsigned)(r & 0x7fffu) << 17;    // the rest, r 2^75
+  const unsigned long long rr = (unsigned long long)rh * rh;  // r^2 2^86
+  const unsigned r2 = (unsigned)(rr >> 32);                    // r^2 2^54
+  const unsigned long long a2 = (rr >> 23) + (__umulhi(rh, rl) >> 22);  // r^2/2 2^64
+  const unsigned a3 = __umulhi(__umulhi(r2, rh), 2863311531u) >> 3;     // r^3/6 2^64
+  const unsigned a4 = __umulhi(__umulhi(r2, r2), 178956971u) >> 12;     // r^4/24 2^64
+  const unsigned long long q = (r << 6) - a2 + a3 - a4;
+  const unsigned long long w = t - __umul64hi(t, q);  // e^-X 2^62
+  return (long long)((w + (1ull << (61 - B))) >> (62 - B));
 }
 
 // 2^-(Y 2^-57 - n) in 2^-61 fixed point (in (2^60, 2^61]) for Y = y 2^57 and
@@ -338,43 +353,67 @@ __device__ __forceinline__ long long exp_fix2(double d, const unsigned long long
 // ---- the argument k ln 2 - x in 2^-58 fixed point, on the integer pipes ----
 // For a power-of-two reference 2^k (|k| < 2^11) and a log-weight x <= k ln 2
 // (up to rounding): K = k ln 2 2^58 from ln 2 to 2^-116, and x 2^58 from the
-// bits of x, both in 128-bit integers, so X = K - x 2^58 is within two units
-// of (k ln 2 - x) 2^58 whatever the magnitudes of k and x.
+// bits of x, so X = K - x 2^58 is within two units of (k ln 2 - x) 2^58
+// whatever the magnitudes of k and x.
 constexpr unsigned long long kLn2Q116Hi = 0xb17217f7d1cf7ull;               // round(ln 2 2^116) >> 64
 constexpr unsigned long long kLn2Q116Lo = 0x9abc9e3b39803f2full;           // its low 64 bits
 constexpr unsigned long long kExpCutQ58 = 0x9a00000000000000ull;           // 38.5 2^58
+static_assert((kExpCutQ58 >> 53) < kExp32N, "the table covers every weight above the cut");
 
 __device__ __forceinline__ __int128 ref_q58(int k) {
   const __int128 l = ((__int128)kLn2Q116Hi << 64) | (__int128)kLn2Q116Lo;
   return ((__int128)k * l) >> 58;
 }
 
-// floor-toward-zero of x 2^58 as a signed 128-bit integer (|x| < 2^69)
-__device__ __forceinline__ __int128 fix_q58(double x) {
-  const long long b = __double_as_longlong(x);
-  const int e = (int)((b >> 52) & 0x7ff);
-  if (e == 0) return 0;
-  const unsigned long long m = (unsigned long long)((b & 0x000FFFFFFFFFFFFFll) | 0x0010000000000000ll);
-  const int sh = e - 1017;
-  __int128 v;
-  if (sh >= 74)
-    v = (__int128)1 << 126;
-  else if (sh >= 0)
-    v = (__int128)m << sh;
-  else
-    v = -sh < 64 ? (__int128)(m >> -sh) : 0;
-  return b < 0 ? -v : v;
+// The low 64 bits of ref_q58(k) (k ln 2 2^58 rounded down), |k| < 2^11.
+__device__ __forceinline__ unsigned long long ref_q58_lo(int k) {
+  const unsigned long long ks = (unsigned long long)(long long)k;
+  const unsigned long long lo = ks * kLn2Q116Lo;
+  const unsigned long long hi =
+      __umul64hi(ks, kLn2Q116Lo) - (k < 0 ? kLn2Q116Lo : 0ull) + ks * kLn2Q116Hi;
+  return (lo >> 58) | (hi << 6);
 }
 
-// round(e^(x - k ln 2) 2^B) for a log-weight x (-inf allowed) and the
-// reference K = ref_q58(k), |k| < 2^11: integer pipes only.
-template <int B>
-__device__ __forceinline__ long long weight_fix(double x, __int128 K, const MathTab* __restrict__ T) {
-  if (__double_as_longlong(x) == (long long)0xFFF0000000000000ull) return 0;  // -inf
-  __int128 X = K - fix_q58(x);
-  if (X < 0) X = 0;  // x above the reference by rounding: weight 1
-  if (X >= (__int128)kExpCutQ58) return 0;
-  return exp_fix_x<B>((unsigned long long)X, T);
+// Shifts that give 0 for a count of 64 or more.
+__device__ __forceinline__ unsigned long long shl64(unsigned long long x, unsigned n) {
+  unsigned long long r;
+  asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(n));
+  return r;
+}
+__device__ __forceinline__ unsigned long long shr64(unsigned long long x, unsigned n) {
+  unsigned long long r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(n));
+  return r;
+}
+
+// A double of magnitude below 2^127 as a float, truncated (below 2^-126: 0),
+// from its bits on the integer pipes (a conversion runs at the FP64 pipe's rate).
+__device__ __forceinline__ float trunc_f32(unsigned hi, unsigned lo) {
+  const unsigned mag = hi & 0x7fffffffu;
+  if (mag < 0x38100000u) return 0.0f;
+  return __uint_as_float(__funnelshift_l(lo, mag - 0x38000000u, 3) | (hi & 0x80000000u));
+}
+
+// round(e^(x - k ln 2) 2^54) for a log-weight x (-inf allowed), the reference
+// exponent k, |k| < 2^11, k ln 2 >= x up to rounding, K = ref_q58_lo(k): integer
+// pipes only.  X = k ln 2 2^58 - x 2^58 is formed modulo 2^64, which is its value
+// whenever k ln 2 - x < 64; a float comparison (error below 2^-10) settles the
+// rest, whose weight is 0.
+__device__ __forceinline__ long long weight_fix54(double x, int k, unsigned long long K,
+                                                  const MathTab* __restrict__ T) {
+  const long long b = __double_as_longlong(x);
+  const unsigned hi = (unsigned)((unsigned long long)b >> 32), lo = (unsigned)b;
+  const int e = (int)((hi >> 20) & 0x7ffu);
+  if (e >= 1034) return b < 0 ? 0 : 1ll << 54;  // |x| >= 2^11 or not finite
+  if (fmaf((float)k, kLn2f, -trunc_f32(hi, lo)) > 60.0f) return 0;
+  const unsigned long long m =
+      ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
+  const int sh = e - 1017;  // x 2^58 = m 2^sh
+  const unsigned long long v = sh >= 0 ? shl64(m, (unsigned)sh) : shr64(m, (unsigned)-sh);
+  unsigned long long X = b < 0 ? K + v : K - v;
+  if (X > ~15ull) X = 0;  // x above the reference by rounding: weight 1
+  if (X >= kExpCutQ58) return 0;
+  return exp_fix_x<54>(X, T);
 }
 
 // The argument in 2^-52 units, in 64-bit integers: for a reference k with
@@ -1018,12 +1057,15 @@ __device__ __forceinline__ double from_order_key(long long k) {
   return __longlong_as_double(k >= 0 ? k : k ^ 0x7FFFFFFFFFFFFFFFll);
 }
 
-// Warp max of doubles through their order keys (integer shuffles only).
+// Warp max of doubles through their order keys: the high words by one integer
+// warp reduction, the low words among the lanes that hold it by another (two
+// instructions against five rounds of two shuffles and a 64-bit maximum).
 __device__ __forceinline__ double warp_max_key(double x) {
-  long long v = order_key(x);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return from_order_key(v);
+  const long long v = order_key(x);
+  const int h = (int)(v >> 32);
+  const int mh = __reduce_max_sync(0xffffffffu, h);
+  const unsigned ml = __reduce_max_sync(0xffffffffu, h == mh ? (unsigned)v : 0u);
+  return from_order_key(((long long)mh << 32) | (long long)ml);
 }
 
 // ---- fixed-point weights: w * 2^54 as int64 (tile-local scans) ----

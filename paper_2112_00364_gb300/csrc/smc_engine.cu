@@ -185,7 +185,13 @@ smc_status math_table(const MathTab** out) {
       if (j == 0) return 1ull << 63;
       return (unsigned long long)std::llroundl(std::ldexp(std::exp2l(-(long double)j / m), 63));
     };
-    for (int j = 0; j < 128; ++j) h.exp2_neg_q63[j] = q63(j, 128);
+    // e^-(j/m) 2^63 rounded; j = 0 is 2^63 itself
+    auto e63 = [](int j, int m) -> unsigned long long {
+      if (j == 0) return 1ull << 63;
+      return (unsigned long long)std::llroundl(std::ldexp(std::exp(-(long double)j / m), 63));
+    };
+    for (int j = 0; j < kExp32N; ++j) h.exp_neg32_q63[j] = e63(j, 32);
+    for (int j = 0; j < 64; ++j) h.exp_neg2048_q63[j] = e63(j, 2048);
     for (int j = 0; j < 64; ++j) {
       h.exp2_neg64_q63[j] = q63(j, 64);
       h.exp2_neg4096_q63[j] = q63(j, 4096);

@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(TPB, 1) small_run_kernel(const RunDev* __restr
   // ends segment k, where it overlaps the other CTAs' arrival
   Combined c_close;
   bool resample_close = false;
-  double u = 0.0;  // the uniform of the next search, drawn in the barrier's shadow
+  unsigned long long uf = 0;  // the uniform of the next search, drawn in the barrier's shadow
   // the run's counters, summed per lane over the segments and added once
   unsigned long long n_near = 0, n_overflow = 0, n_limit = 0, n_draws = 0, n_blocks = 0;
   for (int k = 0;; ++k) {
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(TPB, 1) small_run_kernel(const RunDev* __restr
       if (resample && lane == 0) {
         Q64 d, z0;
         long long tolZ;
-        search_scalars(c, N, A.recip_n, u, &d, &z0, &tolZ);
+        search_scalars(c, N, A.recip_n, uf, &d, &z0, &tolZ);
         q5[0] = d.hi;
         q5[1] = d.lo;
         q5[2] = z0.hi;
@@ -320,10 +320,10 @@ __global__ void __launch_bounds__(TPB, 1) small_run_kernel(const RunDev* __restr
     // the tile's weights: a warp is a tile, so its reference is the warp's
     long long ef = 0;
     const double Mw = warp_max_key(lw);
-    const int kt = Mw == -INFINITY ? kDeadTile : tile_exponent(Mw);
+    const int kt = Mw == -INFINITY ? kDeadTile : tile_exponent_fast(Mw);
     if (valid && kt != kDeadTile) {
       if (kt > -2048 && kt < 2048) {
-        ef = weight_fix<54>(lw, ref_q58(kt), A.md.tab);
+        ef = weight_fix54(lw, kt, ref_q58_lo(kt), A.md.tab);
       } else {
         const double kd = (double)kt;
         const double dd = fma(-kd, kLn2Lo, fma(-kd, kLn2Hi, lw));
@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(TPB, 1) small_run_kernel(const RunDev* __restr
     // the segment's records, running sums and states, for the next combine
     if (CL) cluster_arrive();
     if (k > 0 && lead && threadIdx.x == 0) finish_segment(A, k, c_close, resample_close);
-    if (lane == 0) u = Unif<double>::first(philox(0u, (uint32_t)k, 0u, 1u, A.k0, A.k1));
+    if (lane == 0) uf = search_uniform(A, k);
     if (CL)
       cluster_wait();
     else

@@ -78,6 +78,11 @@ __device__ __forceinline__ bool finish_segment(const RunDev& A, int k, const Com
   return go_on;
 }
 
+// u 2^64 of the uniform of the search after checkpoint k.
+__device__ __forceinline__ unsigned long long search_uniform(const RunDev& A, int k) {
+  return frac64(Unif<double>::first(philox(0u, (uint32_t)k, 0u, 1u, A.k0, A.k1)));
+}
+
 // What the search of segment k needs about segment k-1's weights.
 struct SearchCtx {
   const long long* O;  // offsets in units U, O[T] = S
@@ -88,11 +93,12 @@ struct SearchCtx {
   long long tolZ;      // 1e-12 N on the q scale, in units U
 };
 
-// The run's search scalars from its combined total (one thread).
+// The run's search scalars from its combined total (one thread); uf = u 2^64.
 __device__ __forceinline__ void search_scalars(const Combined& c, int N, unsigned long long recip_n,
-                                               double u, Q64* d, Q64* z0, long long* tolZ) {
+                                               unsigned long long uf, Q64* d, Q64* z0,
+                                               long long* tolZ) {
   *d = q_ratio((unsigned long long)c.S, (unsigned long long)N, recip_n);
-  *z0 = q_scale(frac64(u), *d);
+  *z0 = q_scale(uf, *d);
   *tolZ = floor_i64(kBoundaryEps * (double)c.S);
 }
 
@@ -225,15 +231,29 @@ __device__ __forceinline__ void prefetch_neighbours(const RunDev& A, int t, int 
   for (int f = 0; f < M::N_INT; ++f) prefetch_range<TPB>(&S.inf_(f, 0, A.N), lo, hi, 4);
 }
 
+// A CTA's shared memory.
+template <int TPB>
+struct StepShared {
+  double red[4 * (TPB / 32) + 1];  // combine_offsets' reductions
+  unsigned long long scal[5];      // the search scalars
+  unsigned long long uf;           // u 2^64 of the search they are for
+  long long sum[TPB / 32], sq[TPB / 32];  // the warps' weight sums (and of their squares)
+  unsigned draws[TPB / 32], execs[TPB / 32];
+  int kw[TPB / 32], last;
+  long long O[redundant_cap(TPB)];  // the offsets of a run combined in every CTA
+  int ks[redundant_cap(TPB)];       // and its tiles' reference exponents
+};
+
 // One tile of one run for segment k (the whole per-CTA body of a wave).
 template <class M, int TPB>
-__device__ __forceinline__ void step_tile(const RunDev& A, const int t, const int k, double* sh,
-                                          int* sh_last, int* sh_kw, long long* sh_O, int* sh_ks) {
+__device__ __forceinline__ void step_tile(const RunDev& A, const int t, const int k,
+                                          StepShared<TPB>& S) {
   using R = typename M::R;
   RunState* rs = A.rs;
   const int N = A.N;
   const int i = t * A.tile + threadIdx.x;
   const bool valid = (int)threadIdx.x < A.tile && i < N;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int nb = k & 1, cb = nb ^ 1;
   const StateView Sc = A.state[cb];
   const StateView Sn = A.state[nb];
@@ -253,33 +273,32 @@ __device__ __forceinline__ void step_tile(const RunDev& A, const int t, const in
     X.rec = A.rec[cb];
     bool resample;
     if (redundant) {
-      const Combined c = combine_offsets<TPB>(A.rec[cb], A.n_tiles, sh_O, sh_ks, sh,
+      const Combined c = combine_offsets<TPB>(A.rec[cb], A.n_tiles, S.O, S.ks, S.red,
                                               A.ess ? A.tq[cb] : nullptr);
       const bool go_on = c.kmax != kDeadTile && c.alive && k < A.max_segments;
       resample = decide_resample(A, c);
-      if (t == 0 && threadIdx.x == 0) finish_segment(A, k, c, resample);
+      // (by the tile's last thread: its warp is the one most often without particles)
+      if (t == 0 && threadIdx.x == TPB - 1) finish_segment(A, k, c, resample);
       if (!go_on) return;
       // the run's search scalars by one thread, shared through shared memory
-      unsigned long long* shq = reinterpret_cast<unsigned long long*>(sh + TPB / 32 + 1);
       if (resample && threadIdx.x == 0) {
         Q64 d, z0;
         long long tolZ;
-        search_scalars(c, N, A.recip_n, Unif<double>::first(philox(0u, (uint32_t)(k - 1), 0u, 1u, A.k0, A.k1)),
-                       &d, &z0, &tolZ);
-        shq[0] = d.hi;
-        shq[1] = d.lo;
-        shq[2] = z0.hi;
-        shq[3] = z0.lo;
-        shq[4] = (unsigned long long)tolZ;
+        search_scalars(c, N, A.recip_n, S.uf, &d, &z0, &tolZ);
+        S.scal[0] = d.hi;
+        S.scal[1] = d.lo;
+        S.scal[2] = z0.hi;
+        S.scal[3] = z0.lo;
+        S.scal[4] = (unsigned long long)tolZ;
       }
       __syncthreads();
-      X.O = sh_O;
-      X.ks = sh_ks;
+      X.O = S.O;
+      X.ks = S.ks;
       X.kmax = c.kmax;
       X.G = c.G;
-      X.d = Q64{shq[0], shq[1]};
-      X.z0 = Q64{shq[2], shq[3]};
-      X.tolZ = (long long)shq[4];
+      X.d = Q64{S.scal[0], S.scal[1]};
+      X.z0 = Q64{S.scal[2], S.scal[3]};
+      X.tolZ = (long long)S.scal[4];
     } else {
       resample = rs->resample != 0;
       X.O = A.tile_O;
@@ -339,87 +358,117 @@ __device__ __forceinline__ void step_tile(const RunDev& A, const int t, const in
     A.logw[i] = lw;
     alive = L.pc != PC_STOP;
   }
-  warp_add_u64(&rs->n_overflow, active ? (unsigned long long)L.overflow : 0ull);
-  warp_add_u64(&rs->n_limit, active ? (unsigned long long)L.limited : 0ull);
-  // work counters: Philox blocks of the model's draw stream and blocks executed
-  warp_add_u64(&rs->n_draws, valid ? (unsigned long long)s.d : 0ull);
-  warp_add_u64(&rs->n_blocks, (unsigned long long)n_exec);
   // Weights, first per warp as soon as the warp's particles reached the
   // checkpoint (overlapping the tile's slower warps): the warp's max M_w, its
   // power-of-two reference k_w = ceil(M_w / ln 2), and e_j = exp(logw_j - k_w
   // ln 2) 2^54 rounded to an integer on the integer pipes.  Then, after the tile barrier, the tile
   // reference k_t = max k_w, the exact shift of each weight to it, and the
   // tile's integer running sum E_j (the next segment's search keys).
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   long long ef = 0;
   const double Mw = warp_max_key(lw);
-  const int kw = Mw == -INFINITY ? kDeadTile : tile_exponent(Mw);
+  const int kw = Mw == -INFINITY ? kDeadTile : tile_exponent_fast(Mw);
   if (valid && kw != kDeadTile) {
     // (an FP32 log-weight is exact as a double, so both precisions share the
     // normaliser's integer-pipe exponential)
     if (kw > -2048 && kw < 2048) {
-      ef = weight_fix<54>(lw, ref_q58(kw), A.md.tab);  // integer pipes only
+      ef = weight_fix54(lw, kw, ref_q58_lo(kw), A.md.tab);  // integer pipes only
     } else {
       const double kd = (double)kw;
       const double d = fma(-kd, kLn2Lo, fma(-kd, kLn2Hi, lw));  // lw - kw ln 2, two-part ln 2
       ef = exp_fix54(d, A.md.tab);
     }
   }
-  if (lane == 0) sh_kw[wid] = kw;
+  // work counters: Philox blocks of the model's draw stream and blocks executed,
+  // summed over the CTA: one atomic a CTA and counter.  (With one a warp, 65,536
+  // of them fell on two words in a wave of 2^20 particles; that, a fence by every
+  // thread and two more barriers took 20 of the rate-shift model's 178 us a wave.)
+  // Kills are rare.
+  const unsigned draws = __reduce_add_sync(0xffffffffu, valid ? s.d : 0u);
+  const unsigned execs = __reduce_add_sync(0xffffffffu, (unsigned)n_exec);
+  const unsigned kills = __reduce_add_sync(
+      0xffffffffu, active ? (unsigned)L.overflow | ((unsigned)L.limited << 16) : 0u);
+  if (lane == 0) {
+    if (kills & 0xffffu) atomicAdd(&rs->n_overflow, (unsigned long long)(kills & 0xffffu));
+    if (kills >> 16) atomicAdd(&rs->n_limit, (unsigned long long)(kills >> 16));
+    S.kw[wid] = kw;
+    S.draws[wid] = draws;
+    S.execs[wid] = execs;
+  }
   alive = __syncthreads_or(alive);
-  int kt = sh_kw[0];
+  int kt = S.kw[0];
 #pragma unroll
-  for (int w = 1; w < TPB / 32; ++w) kt = max(kt, sh_kw[w]);
+  for (int w = 1; w < TPB / 32; ++w) kt = max(kt, S.kw[w]);
   const int shift = kw == kDeadTile ? 64 : kt - kw;
   if (shift >= 63)
     ef = 0;
   else if (shift > 0)
     ef = (ef + (1ll << (shift - 1))) >> shift;
-  const long long E = block_incl_scan_i64<TPB>(ef, reinterpret_cast<long long*>(sh));
-  if (valid) A.E[nb][i] = E;
-  if (A.ess) {  // the tile's sum of squared weights, units 2^-54 of 2^(2 k_t)
+  long long E = block_incl_scan_i64<32>(ef, nullptr);  // the warp's running sums
+  if (A.ess) {  // the warp's sum of squared weights, units 2^-54 of 2^(2 k_t)
     const unsigned long long u = (unsigned long long)ef;
-    const long long sq = (long long)((__umul64hi(u, u) << 10) | ((u * u) >> 54));
-    __syncthreads();
-    const long long Q = block_incl_scan_i64<TPB>(sq, reinterpret_cast<long long*>(sh));
-    if (threadIdx.x == TPB - 1) A.tq[nb][t] = Q;
+    unsigned long long sq = (__umul64hi(u, u) << 10) | ((u * u) >> 54);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    if (lane == 0) S.sq[wid] = (long long)sq;
   }
-  if (threadIdx.x == TPB - 1) {
-    TileRec r;
-    r.s = E;
-    r.k = kt;
-    r.alive = alive;
-    A.rec[nb][t] = r;
+  if (lane == 31) S.sum[wid] = E;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < TPB / 32 - 1; ++w) E += w < wid ? S.sum[w] : 0;
+  if (valid) A.E[nb][i] = E;
+  if (wid == TPB / 32 - 1) {  // the last warp closes the tile
+    unsigned long long d = lane < TPB / 32 ? S.draws[lane] : 0u, x = lane < TPB / 32 ? S.execs[lane] : 0u;
+    long long Q = A.ess && lane < TPB / 32 ? S.sq[lane] : 0;
+#pragma unroll
+    for (int o = TPB / 64; o > 0; o >>= 1) {
+      d += __shfl_xor_sync(0xffffffffu, d, o);
+      x += __shfl_xor_sync(0xffffffffu, x, o);
+      Q += __shfl_xor_sync(0xffffffffu, Q, o);
+    }
+    if (lane == 0) {
+      if (d) atomicAdd(&rs->n_draws, d);
+      if (x) atomicAdd(&rs->n_blocks, x);
+      if (A.ess) A.tq[nb][t] = Q;
+    }
+    __syncwarp();  // tq before the arrival
+    if (lane == 31) {
+      TileRec r;
+      r.s = E;
+      r.k = kt;
+      r.alive = alive;
+      A.rec[nb][t] = r;
+      if (!redundant) {  // the run's last tile of the segment combines for the next wave
+        __threadfence();
+        const unsigned prev = atomicAdd(&rs->arrive, 1u);
+        S.last = (prev == (unsigned)A.n_tiles - 1u);
+      }
+    }
   }
   if (redundant) return;  // the next wave combines
-  __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) {
-    const unsigned prev = atomicAdd(&rs->arrive, 1u);
-    *sh_last = (prev == (unsigned)A.n_tiles - 1u);
-  }
-  __syncthreads();
-  if (*sh_last) {  // the run's last tile of segment k: combine for the next wave
+  if (S.last) {  // the run's last tile of segment k: combine for the next wave
     __threadfence();
-    const Combined c = combine_offsets<TPB>(A.rec[nb], A.n_tiles, A.tile_O, nullptr, sh,
+    const Combined c = combine_offsets<TPB>(A.rec[nb], A.n_tiles, A.tile_O, nullptr, S.red,
                                             A.ess ? A.tq[nb] : nullptr);
-    if (threadIdx.x == 0) {
-      const bool resample = decide_resample(A, c);
+    // closing the segment (log Z, its records) and the next search's scalars, by a
+    // thread each
+    const bool resample = decide_resample(A, c);
+    if (threadIdx.x == TPB - 1) {
       rs->resample = resample ? 1 : 0;
-      if (finish_segment(A, k + 1, c, resample) && resample) {
-        Q64 d, z0;
-        long long tolZ;
-        search_scalars(c, N, A.recip_n, Unif<double>::first(philox(0u, (uint32_t)k, 0u, 1u, A.k0, A.k1)), &d,
-                       &z0, &tolZ);
-        rs->kmax = c.kmax;
-        rs->G = c.G;
-        rs->d_hi = d.hi;
-        rs->d_lo = d.lo;
-        rs->z0_hi = z0.hi;
-        rs->z0_lo = z0.lo;
-        rs->tolZ = tolZ;
-      }
+      finish_segment(A, k + 1, c, resample);
       rs->arrive = 0;
+    }
+    if (threadIdx.x == 0 && resample && c.kmax != kDeadTile) {
+      Q64 d, z0;
+      long long tolZ;
+      search_scalars(c, N, A.recip_n, S.uf, &d, &z0, &tolZ);
+      rs->kmax = c.kmax;
+      rs->G = c.G;
+      rs->d_hi = d.hi;
+      rs->d_lo = d.lo;
+      rs->z0_hi = z0.hi;
+      rs->z0_lo = z0.lo;
+      rs->tolZ = tolZ;
     }
   }
 }
@@ -434,11 +483,7 @@ template <typename R, int TPB, int KIND>
 __global__ void __launch_bounds__(TPB, (sizeof(R) == 4 ? 1024 : 768) / TPB) wave_kernel(const RunDev* __restrict__ runs,
                                                    const int2* __restrict__ cta_map, unsigned wave) {
   __shared__ __align__(16) RunDev sr;
-  __shared__ double sh[TPB / 32 + 2 + TPB + 1];
-  __shared__ int sh_last;
-  __shared__ int sh_kw[TPB / 32];
-  __shared__ long long sh_O[redundant_cap(TPB)];
-  __shared__ int sh_ks[redundant_cap(TPB)];
+  __shared__ StepShared<TPB> S;
   const int2 rt = cta_map[blockIdx.x];
   {
     const int* src = reinterpret_cast<const int*>(runs + rt.x);
@@ -451,26 +496,28 @@ __global__ void __launch_bounds__(TPB, (sizeof(R) == 4 ? 1024 : 768) / TPB) wave
   // this wave's last CTAs still run; everything below reads what the previous
   // wave wrote, so it waits for that wave's completion first.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int k = (int)(wave - sr.start_wave);  // wraps correctly past 2^32 waves
+  // the uniform of the search whose scalars this CTA may form, from the counter
+  // alone: in the wait's shadow
+  if (threadIdx.x == 0) S.uf = search_uniform(sr, sr.redundant ? k - 1 : k);
   asm volatile("griddepcontrol.wait;" ::: "memory");
   RunState* rs = sr.rs;
-  if (*(volatile int32_t*)&rs->done) return;
-  const int k = (int)(wave - sr.start_wave);  // wraps correctly past 2^32 waves
-  if (k < 0) return;
+  if (*(volatile int32_t*)&rs->done || k < 0) return;
   if (KIND == SMC_MODEL_LG) {
-    step_tile<LgModel<R>, TPB>(sr, rt.y, k, sh, &sh_last, sh_kw, sh_O, sh_ks);
+    step_tile<LgModel<R>, TPB>(sr, rt.y, k, S);
     return;
   }
   if (KIND == SMC_MODEL_CRBD) {
-    step_tile<TreeModel<R, false>, TPB>(sr, rt.y, k, sh, &sh_last, sh_kw, sh_O, sh_ks);
+    step_tile<TreeModel<R, false>, TPB>(sr, rt.y, k, S);
     return;
   }
   switch (sr.md.kind) {
-    case SMC_MODEL_LG: step_tile<LgModel<R>, TPB>(sr, rt.y, k, sh, &sh_last, sh_kw, sh_O, sh_ks); break;
-    case SMC_MODEL_SEIR: step_tile<SeirModel<R>, TPB>(sr, rt.y, k, sh, &sh_last, sh_kw, sh_O, sh_ks); break;
-    case SMC_MODEL_CRBD: step_tile<TreeModel<R, false>, TPB>(sr, rt.y, k, sh, &sh_last, sh_kw, sh_O, sh_ks); break;
-    case SMC_MODEL_RATESHIFT: step_tile<TreeModel<R, true>, TPB>(sr, rt.y, k, sh, &sh_last, sh_kw, sh_O, sh_ks); break;
-    case SMC_MODEL_CRBD_DS: step_tile<TreeDsModel<R>, TPB>(sr, rt.y, k, sh, &sh_last, sh_kw, sh_O, sh_ks); break;
-    default: step_tile<GeoModel<R>, TPB>(sr, rt.y, k, sh, &sh_last, sh_kw, sh_O, sh_ks); break;
+    case SMC_MODEL_LG: step_tile<LgModel<R>, TPB>(sr, rt.y, k, S); break;
+    case SMC_MODEL_SEIR: step_tile<SeirModel<R>, TPB>(sr, rt.y, k, S); break;
+    case SMC_MODEL_CRBD: step_tile<TreeModel<R, false>, TPB>(sr, rt.y, k, S); break;
+    case SMC_MODEL_RATESHIFT: step_tile<TreeModel<R, true>, TPB>(sr, rt.y, k, S); break;
+    case SMC_MODEL_CRBD_DS: step_tile<TreeDsModel<R>, TPB>(sr, rt.y, k, S); break;
+    default: step_tile<GeoModel<R>, TPB>(sr, rt.y, k, S); break;
   }
 }
 
