@@ -301,6 +301,7 @@ Layout make_layout(const smc_model_s* m, const smc_run_cfg* c) {
   const size_t rb = c->precision == SMC_PREC_FP32 ? 4 : 8;
   L.tile = tile_for((int64_t)N);
   L.n_tiles = (int)((N + L.tile - 1) / L.tile);
+  L.pad = (L.tile + 31) / 32 * 32;
   L.max_segments = c->max_segments > 0 ? c->max_segments
                    : (m->n_segments_known > 0 ? m->n_segments_known : kUnboundedSegments);
   const int max_res = std::max(1, L.max_segments - 1);
@@ -320,8 +321,10 @@ Layout make_layout(const smc_model_s* m, const smc_run_cfg* c) {
     L.stack[b] = take(rb * N * (size_t)m->stack_cap);
   }
   L.logw = take(8 * N);
-  L.E[0] = take(8 * N);
-  L.E[1] = take(8 * N);
+  for (int b = 0; b < 2; ++b) {
+    L.E[b] = take(8 * (size_t)L.n_tiles * (size_t)L.pad);
+    L.ends[b] = take(L.pad > 32 ? 64 * (size_t)L.n_tiles : 0);
+  }
   L.rec[0] = take(sizeof(TileRec) * (size_t)L.n_tiles);
   L.rec[1] = take(sizeof(TileRec) * (size_t)L.n_tiles);
   L.tq[0] = take(8 * (size_t)L.n_tiles);
@@ -352,6 +355,7 @@ RunDev make_rundev(const smc_model_s* m, const smc_run_cfg* c, const Layout& Ly,
     A.state[b].ints = (int32_t*)(ws + Ly.ints[b]);
     A.state[b].stack = ws + Ly.stack[b];
     A.E[b] = (long long*)(ws + Ly.E[b]);
+    A.ends[b] = (long long*)(ws + Ly.ends[b]);
   }
   A.logw = (double*)(ws + Ly.logw);
   A.rec[0] = (TileRec*)(ws + Ly.rec[0]);
@@ -371,6 +375,7 @@ RunDev make_rundev(const smc_model_s* m, const smc_run_cfg* c, const Layout& Ly,
   A.recip_n = ~0ull / (unsigned long long)c->n_particles;
   A.n_tiles = Ly.n_tiles;
   A.tile = Ly.tile;
+  A.pad = Ly.pad;
   A.max_segments = Ly.max_segments;
   A.record_all = c->record_all_ancestors ? 1 : 0;
   A.anc_rows = Ly.anc_rows;

@@ -44,7 +44,11 @@ struct RunDev {
   ModelDev md;
   StateView state[2];
   double* logw;       // [N] log-weights of the latest segment (f64; FP32 values widened)
-  long long* E[2];    // [N] tile-local running sums of the weights x 2^54 (int64), double-buffered by segment parity
+  // [n_tiles][pad] running sums of the weights x 2^54 (int64) within each warp of a tile
+  // (pad: the tile in whole warps), double-buffered by segment parity, and, for
+  // tiles of more than one warp, [n_tiles][8] the warps' ends in the tile's running sum
+  long long* E[2];
+  long long* ends[2];
   TileRec* rec[2];    // [n_tiles] tile reductions, double-buffered by segment parity
   long long* tq[2];   // [n_tiles] ESS mode: the tiles' sums of squared weights (units 2^-54 of 2^(2 k_t))
   int32_t* dec;       // [max_segments] 1 where the population was resampled after checkpoint k
@@ -56,7 +60,7 @@ struct RunDev {
   unsigned long long recip_n;  // floor((2^64 - 1) / N), the search scalars' divisor
   double ess_tau;       // 0: resample after every checkpoint; > 0: only when ESS < ess_tau N
   double ess_target;    // ess_tau N
-  int N, n_tiles, tile, max_segments, record_all, anc_rows;
+  int N, n_tiles, tile, pad, max_segments, record_all, anc_rows;
   unsigned start_wave;  // wave index of the run's segment 0 (segment k runs in wave start_wave + k)
   int redundant;        // combine a segment's tiles in every CTA of the next wave (else in the last CTA)
   int ess;              // ess_tau > 0 (an integer flag for the kernel's branches)
@@ -70,9 +74,9 @@ struct RunDev {
 };
 
 struct Layout {
-  size_t real[2], ints[2], stack[2], logw, E[2], rec[2], tq[2], dec, tO, rs, anc, incr,
+  size_t real[2], ints[2], stack[2], logw, E[2], ends[2], rec[2], tq[2], dec, tO, rs, anc, incr,
       fin_real, fin_int, fin_stack, snap, total;
-  int n_tiles, tile, anc_rows, max_segments;
+  int n_tiles, tile, pad, anc_rows, max_segments;
 };
 
 // Device addresses of one wave's run table and per-bucket CTA maps.

@@ -102,91 +102,171 @@ __device__ __forceinline__ void search_scalars(const Combined& c, int N, unsigne
   *tolZ = floor_i64(kBoundaryEps * (double)c.S);
 }
 
+// The tile of an offset: t = max{ t : O_t <= Z } in [0, T], and O_t.  Every lane
+// of the warp calls it; the lanes' Z are non-decreasing.  The warp's 32
+// consecutive offsets span few tiles, so one window of 32 tile offsets, one
+// load a lane, holds them all: around the CTA's own tile when the offsets are in
+// global memory (systematic ancestors lie near their particle: the window holds
+// them but for a population whose weights are very uneven across its tiles), by
+// one 32-way step through shared memory when they are there; a 32-way descent
+// finds the window otherwise.  One or two rounds of loads against the log2 T
+// dependent ones of a binary search per lane (12 L2 round trips at 4,096 tiles).
+// kShared: O is in shared memory and T < 1024.
+__device__ __forceinline__ int find_tile(long long Z, const long long* O, int T, bool shared_O,
+                                         int near_t, long long* Ot) {
+  constexpr unsigned kAll = 0xffffffffu;
+  constexpr long long kTop = 0x7FFFFFFFFFFFFFFFll;
+  const int lane = threadIdx.x & 31;
+  const long long Zf = __shfl_sync(kAll, Z, 0);
+  const long long Zl = __shfl_sync(kAll, Z, 31);
+  int w0 = shared_O ? 0 : max(0, min(near_t - 15, T - 31));
+  long long val = kTop;
+  bool have = false;
+  if (!shared_O) {
+    if (w0 + lane <= T) val = O[w0 + lane];
+    const unsigned le = __ballot_sync(kAll, val <= Zf);
+    have = le != 0u && le != kAll;
+  }
+  if (!have) {  // 32-way descent to the window that holds the first lane's tile
+    int span = T + 1;
+    w0 = 0;
+    while (span > 32) {
+      const int step = (span + 31) >> 5, at = lane * step;
+      const long long v = at < span ? O[w0 + at] : kTop;
+      const int s = __popc(__ballot_sync(kAll, v <= Zf)) - 1;  // O_w0 <= Zf
+      w0 += s * step;
+      span = min(step, span - s * step);
+    }
+    val = w0 + lane <= T ? O[w0 + lane] : kTop;
+  }
+  const int cf = __popc(__ballot_sync(kAll, val <= Zf)) - 1;
+  const int cl = __popc(__ballot_sync(kAll, val <= Zl)) - 1;
+  int p = cf;
+  if (cl != cf) {  // the lanes lie in different tiles
+    p = 0;
+#pragma unroll
+    for (int step = 16; step >= 1; step >>= 1) {
+      const long long v = __shfl_sync(kAll, val, p + step);
+      if (v <= Z) p += step;
+    }
+  }
+  *Ot = __shfl_sync(kAll, val, p);
+  int t = w0 + p;
+  if (cl == 31 && p == 31 && t < T) {  // beyond the window: a binary search
+    int hi = T;
+    while (t < hi) {
+      const int mid = (t + hi + 1) >> 1;
+      if (O[mid] <= Z)
+        t = mid;
+      else
+        hi = mid - 1;
+    }
+    *Ot = O[t];
+  }
+  return t;
+}
+
 // a_i = min{ j : q_j > y } for y = i + u, with q_j = P_j N / S and P_j the
 // running sum of the weights; on the P scale in units U the offset is
 // z_i = z_0 + i S / N (64.64 fixed point, exact and non-decreasing in i).  The
 // tile is t = max{ t : O_t <= z } (N - 1 if z lies above every offset); inside
 // it P_j = O_t + E_j 2^-(k_max - k_t + G), so P_j > z <=> E_j > floor((z - O_t)
-// 2^(k_max - k_t + G)) (E_j is an integer): one threshold per particle, then an
-// 8-ary search with integer compares (three rounds of independent loads for a
-// 256-particle tile).  If no element of tile t qualifies, the first element of
-// tile t+1 does.  The offset is flagged when it lies within 1e-12 N of q_a or
-// q_{a-1}, measured in the same units.  Integer arithmetic only.  kL2: the
-// running sums were written by other CTAs of the same launch (a cluster's run),
-// so they are read at L2, past this SM's L1.
-template <bool kL2>
-__device__ __forceinline__ long long load_sum(const long long* p) {
-  if (kL2) return __ldcg(p);
-  return *p;
-}
-
-template <bool kL2 = false>
-__device__ __forceinline__ int systematic_search(int i, const RunDev& A, const SearchCtx& X,
-                                                 const long long* __restrict__ E, bool* near) {
+// 2^(k_max - k_t + G)) (E_j is an integer): one threshold F per particle.  The
+// tile's running sums are kept as its warps' own (E_j = C_{c-1} + e_j for warp c of
+// the tile) with the warps' ends C_c in one 64-byte row a tile, so the search is
+// the row (which warp: the first C_c > F), eight of the warp's 32 sums and the
+// four between two of those: two rounds of loads, the third from lines the second
+// brought.  Bound: the latency of those rounds and issue; with a binary search per
+// lane over the tiles and an 8-ary search over a whole tile's sums (12 + 3 rounds
+// at 4,096 tiles) a wave of 2^20 particles took 105 us instead of 77 with the
+// linear-Gaussian model, 158 instead of 144 with the rate-shift model.  If no
+// element of tile t qualifies, the first element of tile t+1 does.  The offset is
+// flagged when it lies within 1e-12 N of q_a or q_{a-1}, measured in the same
+// units.  Integer arithmetic only.  Every lane of the warp calls it (i of the
+// lanes past the last particle repeats that particle).
+__device__ __forceinline__ int systematic_search(int i, int near_t, const RunDev& A,
+                                                 const SearchCtx& X,
+                                                 const long long* __restrict__ E,
+                                                 const long long* __restrict__ ends, bool* near) {
   const int N = A.N, T = A.n_tiles;
   const Q64 z = q_add(X.z0, q_mul_u32((unsigned)i, X.d));
   const long long Z = (long long)z.hi;
-  int lo = 0, hi = T;  // O_0 = 0 <= z
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (X.O[mid] <= Z)
-      lo = mid;
-    else
-      hi = mid - 1;
-  }
-  if (lo >= T) {  // above the last offset (rounding at the top)
-    *near = Z - X.O[T] < X.tolZ;
+  long long Ot;
+  const int t = find_tile(Z, X.O, T, X.ks != nullptr, near_t, &Ot);
+  if (t >= T) {  // above the last offset (rounding at the top)
+    *near = Z - Ot < X.tolZ;
     return N - 1;
   }
-  const int t = lo;
-  const int j0 = t * A.tile, j1 = min(N, j0 + A.tile);
-  const int kt = X.ks ? X.ks[t] : load_rec(X.rec + t).k;
-  const int sh = X.kmax - kt + X.G;
-  const long long F = q_threshold(z, X.O[t], sh);
-  const long long tolF = shl_sat(X.tolZ, sh);
-  // first j in [j0, j1) with E_j > F
-  long long Eb = 0;  // E_{b-1} for the current bracket start b (0 before the tile)
-  int b = j0, len = j1 - j0;
-  while (len > 8) {
-    const int w = (len + 7) >> 3;
-    long long v[8];
+  const int kt = X.ks ? X.ks[t] : __ldcg(&X.rec[t].k);
+  const int pad = A.pad;
+  long long base = 0;  // the sum before the warp's first element
+  int c = 0;
+  long long C[8];
+  if (pad > 32) {
+    const longlong2* p = reinterpret_cast<const longlong2*>(ends + (size_t)t * 8);
 #pragma unroll
-    for (int m = 0; m < 8; ++m) v[m] = load_sum<kL2>(E + b + min((m + 1) * w, len) - 1);
-    int m = 8;
-#pragma unroll
-    for (int q = 7; q >= 0; --q)
-      if (v[q] > F) m = q;
-    if (m == 8) {  // nothing in the tile qualifies
-      Eb = v[7];
-      b += len;
-      len = 0;
-      break;
+    for (int q = 0; q < 4; ++q) {
+      const longlong2 v = p[q];
+      C[2 * q] = v.x;
+      C[2 * q + 1] = v.y;
     }
-    if (m > 0) Eb = v[m - 1];
-    len = min((m + 1) * w, len) - m * w;
-    b += m * w;
   }
-  int l = b + len;  // none found yet
+  const int sh = X.kmax - kt + X.G;
+  const long long F = q_threshold(z, Ot, sh);
+  const long long tolF = shl_sat(X.tolZ, sh);
+  if (pad > 32) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      if (C[q] <= F) {
+        base = C[q];
+        c = q + 1;
+      }
+  }
+  const int j0 = t * A.tile, j1 = min(N, j0 + A.tile);
+  int a = -1;
+  long long Eb = base;  // E_{a-1}, or the tile's total when no element qualifies
   long long El = 0;
-  if (len > 0) {
+  if (c < 8) {
+    const long long* e = E + ((size_t)t * pad + (size_t)c * 32);
+    const long long f = F - base;
     long long v[8];
 #pragma unroll
-    for (int m = 0; m < 8; ++m) v[m] = m < len ? load_sum<kL2>(E + b + m) : 0x7FFFFFFFFFFFFFFFll;
-    int m = 8;
+    for (int q = 0; q < 8; ++q) v[q] = e[4 * q + 3];
+    int m = 0;
+    long long b = 0;
 #pragma unroll
-    for (int q = 7; q >= 0; --q)
-      if (v[q] > F) m = q;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      if (q == m) El = v[q];
-      if (q < m && q < len) Eb = v[q];
+    for (int q = 0; q < 8; ++q)
+      if (v[q] <= f) {
+        b = v[q];
+        m = q + 1;
+      }
+    if (m < 8) {
+      const longlong2* p = reinterpret_cast<const longlong2*>(e + 4 * m);
+      const longlong2 v0 = p[0], v1 = p[1];
+      int l = 4 * m;
+      El = v0.x;
+      if (v0.x <= f) {
+        b = v0.x;
+        El = v0.y;
+        l += 1;
+        if (v0.y <= f) {
+          b = v0.y;
+          El = v1.x;
+          l += 1;
+          if (v1.x <= f) {
+            b = v1.x;
+            El = v1.y;
+            l += 1;
+          }
+        }
+      }
+      a = j0 + c * 32 + l;
+      El += base;
     }
-    if (m < len) l = b + m;
+    Eb += b;
   }
   bool nr = F - Eb < tolF;
-  int a;
-  if (l < j1) {
-    a = l;
+  if (a >= 0) {
     nr = nr || El - F <= tolF;
   } else if (j1 < N) {  // the first element of the next tile
     a = j1;
@@ -196,39 +276,6 @@ __device__ __forceinline__ int systematic_search(int i, const RunDev& A, const S
   }
   *near = nr;
   return a;
-}
-
-// One L2 line into this SM's L1 ahead of its use (a hint: nothing waits on it).
-__device__ __forceinline__ void prefetch_l1(const void* p) {
-  asm volatile("{\n\t.reg .u64 g;\n\tcvta.to.global.u64 g, %0;\n\tprefetch.global.L1 [g];\n\t}"
-               :: "l"(p));
-}
-
-// The lines of particles [lo, hi) of one array of elements of esz bytes.
-template <int TPB>
-__device__ __forceinline__ void prefetch_range(const void* base, int lo, int hi, int esz) {
-  const char* b = static_cast<const char*>(base) + (size_t)lo * esz;
-  const int lines = ((hi - lo) * esz + 127) >> 7;
-  for (int j = threadIdx.x; j < lines; j += TPB) prefetch_l1(b + (size_t)j * 128);
-}
-
-// Before the offsets are read, pull into L1 what this tile's search and gather
-// will most likely need: systematic ancestors of a tile's
-// particles lie mostly in the tiles t - 1 .. t + 1, so the previous segment's
-// running sums and PSTATE rows of those particles (written by the previous
-// wave).  Their loads then overlap the combine instead of following it.
-template <class M, int TPB>
-__device__ __forceinline__ void prefetch_neighbours(const RunDev& A, int t, int cb) {
-  using R = typename M::R;
-  const int lo = max(0, (t - 1) * A.tile);
-  const int hi = (int)min((long long)A.N, (long long)(t + 2) * A.tile);  // N may be near 2^31
-  if (lo >= hi) return;
-  const StateView& S = A.state[cb];
-  prefetch_range<TPB>(A.E[cb], lo, hi, 8);
-#pragma unroll
-  for (int f = 0; f < M::N_REAL; ++f) prefetch_range<TPB>(&S.rf<R>(f, 0, A.N), lo, hi, (int)sizeof(R));
-#pragma unroll
-  for (int f = 0; f < M::N_INT; ++f) prefetch_range<TPB>(&S.inf_(f, 0, A.N), lo, hi, 4);
 }
 
 // A CTA's shared memory.
@@ -266,9 +313,6 @@ __device__ __forceinline__ void step_tile(const RunDev& A, const int t, const in
   if (load) {
     if (valid) M::load(L, Sn, SnapView{A.snap_logw, A.snap_real, A.snap_int, A.snap_stack}, i, N, s);
   } else if (k > 0) {
-    // (a run combined in every CTA keeps its offsets in shared memory and its
-    // combine short: there the prefetch measured no gain)
-    if (!redundant) prefetch_neighbours<M, TPB>(A, t, cb);
     SearchCtx X;
     X.rec = A.rec[cb];
     bool resample;
@@ -309,9 +353,15 @@ __device__ __forceinline__ void step_tile(const RunDev& A, const int t, const in
       X.z0 = Q64{rs->z0_hi, rs->z0_lo};
       X.tolZ = rs->tolZ;
     }
+    int a_s = i;
+    if (resample && i - lane < N && (int)threadIdx.x - lane < A.tile) {  // (whole warps)
+      const int i_last = min(N, (t + 1) * A.tile) - 1;
+      a_s = systematic_search(min(i, i_last), t, A, X, A.E[cb], A.ends[cb], &near);
+      near = near && valid;
+    }
     if (valid) {
       const int row = A.record_all ? k - 1 : 0;
-      int a = resample ? systematic_search(i, A, X, A.E[cb], &near) : i;
+      int a = a_s;
       bool bad = false;
       if (SMC_DEBUG_CHECKS) {
         if (!(a >= 0 && a < N)) {
@@ -403,7 +453,8 @@ __device__ __forceinline__ void step_tile(const RunDev& A, const int t, const in
     ef = 0;
   else if (shift > 0)
     ef = (ef + (1ll << (shift - 1))) >> shift;
-  long long E = block_incl_scan_i64<32>(ef, nullptr);  // the warp's running sums
+  const long long E = block_incl_scan_i64<32>(ef, nullptr);  // the warp's running sums
+  if ((int)threadIdx.x < A.pad) A.E[nb][(size_t)t * A.pad + threadIdx.x] = E;
   if (A.ess) {  // the warp's sum of squared weights, units 2^-54 of 2^(2 k_t)
     const unsigned long long u = (unsigned long long)ef;
     unsigned long long sq = (__umul64hi(u, u) << 10) | ((u * u) >> 54);
@@ -413,9 +464,6 @@ __device__ __forceinline__ void step_tile(const RunDev& A, const int t, const in
   }
   if (lane == 31) S.sum[wid] = E;
   __syncthreads();
-#pragma unroll
-  for (int w = 0; w < TPB / 32 - 1; ++w) E += w < wid ? S.sum[w] : 0;
-  if (valid) A.E[nb][i] = E;
   if (wid == TPB / 32 - 1) {  // the last warp closes the tile
     unsigned long long d = lane < TPB / 32 ? S.draws[lane] : 0u, x = lane < TPB / 32 ? S.execs[lane] : 0u;
     long long Q = A.ess && lane < TPB / 32 ? S.sq[lane] : 0;
@@ -425,6 +473,15 @@ __device__ __forceinline__ void step_tile(const RunDev& A, const int t, const in
       x += __shfl_xor_sync(0xffffffffu, x, o);
       Q += __shfl_xor_sync(0xffffffffu, Q, o);
     }
+    // the warps' ends C_c (past the last warp: the tile's total) and the total
+    long long C = lane < TPB / 32 ? S.sum[lane] : 0;
+#pragma unroll
+    for (int o = 1; o < TPB / 32; o <<= 1) {
+      const long long y = __shfl_up_sync(0xffffffffu, C, o);
+      if (lane >= o) C += y;
+    }
+    const long long total = __shfl_sync(0xffffffffu, C, TPB / 32 - 1);
+    if (TPB > 32 && lane < 8) A.ends[nb][(size_t)t * 8 + lane] = lane < TPB / 32 ? C : total;
     if (lane == 0) {
       if (d) atomicAdd(&rs->n_draws, d);
       if (x) atomicAdd(&rs->n_blocks, x);
@@ -433,7 +490,7 @@ __device__ __forceinline__ void step_tile(const RunDev& A, const int t, const in
     __syncwarp();  // tq before the arrival
     if (lane == 31) {
       TileRec r;
-      r.s = E;
+      r.s = total;
       r.k = kt;
       r.alive = alive;
       A.rec[nb][t] = r;
