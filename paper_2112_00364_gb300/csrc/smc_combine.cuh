@@ -83,22 +83,56 @@ __device__ __forceinline__ long long magnitude(long long s, int kt, int kmax) {
   return (sh >= 63 ? 0 : (s >> sh)) + 1;
 }
 
+// The same through the L1: after an acquire (a fence, or the start of the kernel)
+// that followed the records' writes.
+__device__ __forceinline__ TileRec load_rec_l1(const TileRec* p) {
+  const longlong2 v = *reinterpret_cast<const longlong2*>(p);
+  TileRec r;
+  r.s = v.x;
+  r.k = (int32_t)(v.y & 0xffffffffll);
+  r.alive = (int32_t)(v.y >> 32);
+  return r;
+}
+
 struct Combined {
   long long S;  // total in units U
   int kmax, G, alive;
-  double ess;   // (sum w)^2 / sum w^2 when the squared sums were given, else 0
+  double ess;   // (sum w)^2 / sum w^2 when the squared sums were given (thread ess_thread()), else 0
 };
 
-// Combine n_tiles tile records into the offsets O[0..nt] (O[nt] = S).  With
-// `ks` non-NULL the records are first staged in shared memory (k_t into ks,
-// s_t into O, which the offsets then overwrite); otherwise they are read from
-// `rec` on each pass.  Every thread of the CTA calls it; all integer work.
-// With `q` (the tiles' sums of squared weights) non-NULL the effective sample
-// size is formed too, in FP64 by the first warp: sum w^2 relative to 2^(2 k_max).
-template <int TPB>
-__device__ Combined combine_offsets(const TileRec* rec, int nt, long long* O, int* ks, double* sh,
-                                    const long long* q = nullptr) {
-  constexpr int P = 4;  // consecutive tiles per thread per chunk
+// The thread that forms the effective sample size (thread 0 forms other scalars).
+__host__ __device__ constexpr int ess_thread(int tpb) { return tpb > 32 ? 32 : 0; }
+// 64-bit words of shared scratch that combine_offsets uses.
+__host__ __device__ constexpr int combine_scratch(int tpb) { return 6 * (tpb / 32); }
+
+// q 2^-d for a tile's sum of squared weights q and d >= 0, in 32.32-bit pieces
+// (bits below 2^-32 dropped), added to f (fraction), l and h (the value's halves).
+__device__ __forceinline__ void add_scaled(unsigned long long q, int d, unsigned long long* f,
+                                           unsigned long long* l, unsigned long long* h) {
+  const unsigned long long v = d < 64 ? q >> d : 0ull;
+  const unsigned long long frac =
+      d < 32 ? (q << (32 - d)) & 0xffffffffull : d < 96 ? (q >> (d - 32)) & 0xffffffffull : 0ull;
+  *f += frac;
+  *l += v & 0xffffffffull;
+  *h += v >> 32;
+}
+
+// Combine n_tiles tile records into the offsets O[0..nt] (O[nt] = S); ks non-NULL
+// receives the tiles' reference exponents.  Every thread of the CTA calls it; integer work only.  Up to four
+// tiles a thread (1,024 with 256 threads: every run combined in each of its CTAs)
+// the records are read once and stay in registers; larger populations read them
+// four at a time, from L2 once and from L1 afterwards.  Bound: latency (the
+// round of loads and four barriers: one each for k_max, the unit, the scan and the
+// result).  (Contiguous runs of 16 tiles a thread at 4,096 tiles, uncoalesced,
+// made a rate-shift wave of 2^20 particles 160 us instead of 144.)  With `q` (the tiles' sums of squared weights) non-NULL the effective
+// sample size is formed too, its sum exact to 2^-32 of a unit whatever the order.
+// `after(c)` is called by every thread before the last barrier: what it writes to
+// shared memory is there for all when combine_offsets returns (not called when
+// every weight is zero).
+template <int TPB, class F>
+__device__ __forceinline__ Combined combine_offsets(const TileRec* rec, int nt, long long* O, int* ks, double* sh,
+                                    const long long* q, F after) {
+  constexpr int P = 4;
   constexpr int W = TPB / 32;
   constexpr unsigned kAll = 0xffffffffu;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -106,17 +140,38 @@ __device__ Combined combine_offsets(const TileRec* rec, int nt, long long* O, in
   int* sk = reinterpret_cast<int*>(sh);                     // [2W] warps' (k max, alive)
   long long* sm = reinterpret_cast<long long*>(sh) + W;     // [W] warps' magnitude sums
   long long* ss = reinterpret_cast<long long*>(sh) + 2 * W;  // [W] warps' unit totals
-  double* qs = sh + 3 * W;                                   // [1] effective sample size
-  int kl = kDeadTile, al = 0;
-  for (int t = threadIdx.x; t < nt; t += TPB) {
-    const TileRec r = load_rec(rec + t);
-    if (ks) {
-      ks[t] = r.k;
-      O[t] = r.s;
+  unsigned long long* es = reinterpret_cast<unsigned long long*>(sh) + 3 * W;  // [3W] squares
+  const bool regs = nt <= P * TPB;
+  const int per = (nt + TPB - 1) / TPB;
+  const int t0 = regs ? min(nt, (int)threadIdx.x * per) : 0, t1 = regs ? min(nt, t0 + per) : 0;
+  TileRec r[P];
+  auto each = [&](auto f) {  // f(t, record) over this thread's tiles
+    if (regs) {
+#pragma unroll
+      for (int p = 0; p < P; ++p)
+        if (t0 + p < t1) f(t0 + p, r[p]);
+    } else {
+      for (int t = threadIdx.x; t < nt; t += P * TPB) {
+        TileRec b[P];
+#pragma unroll
+        for (int p = 0; p < P; ++p) b[p] = load_rec_l1(rec + min(t + p * TPB, nt - 1));
+#pragma unroll
+        for (int p = 0; p < P; ++p)
+          if (t + p * TPB < nt) f(t + p * TPB, b[p]);
+      }
     }
-    kl = max(kl, r.k);
-    al |= r.alive;
+  };
+  if (regs) {
+#pragma unroll
+    for (int p = 0; p < P; ++p)
+      if (t0 + p < t1) r[p] = load_rec(rec + t0 + p);
   }
+  int kl = kDeadTile, al = 0;
+  each([&](int t, const TileRec& x) {
+    if (ks) ks[t] = x.k;
+    kl = max(kl, x.k);
+    al |= x.alive;
+  });
   kl = __reduce_max_sync(kAll, kl);
   al = (int)__reduce_or_sync(kAll, (unsigned)al);
   if (lane == 0) {
@@ -143,48 +198,54 @@ __device__ Combined combine_offsets(const TileRec* rec, int nt, long long* O, in
   // G from b = sum over live tiles of (floor(s_t 2^-(k_max - k_t + 20)) + 1),
   // which lies between the exact sum T of the totals in units of 2^20 U (at
   // G = 0) and T + n_tiles: G = bitlen(b) - 42 gives 2^(41+G) <= b < 2^(42+G),
-  // so S = sum v_t is within [2^61 - n_tiles 2^(20-G), 2^62 + n_tiles].  (With
-  // ks each thread reads back the tiles it staged itself.)
+  // so S = sum v_t is within [2^61 - n_tiles 2^(20-G), 2^62 + n_tiles].
   long long bl = 0;
-  for (int t = threadIdx.x; t < nt; t += TPB) {
-    if (ks)
-      bl += magnitude(O[t], ks[t], c.kmax);
-    else {
-      const TileRec r = load_rec(rec + t);
-      bl += magnitude(r.s, r.k, c.kmax);
+  unsigned long long qf = 0, ql = 0, qh = 0;
+  each([&](int t, const TileRec& x) {
+    bl += magnitude(x.s, x.k, c.kmax);
+    if (q && x.k != kDeadTile) {  // sum w^2 relative to 2^(2 k_max)
+      const int d = c.kmax - x.k;
+      if (d < 48) add_scaled((unsigned long long)__ldcg(q + t), 2 * d, &qf, &ql, &qh);
     }
-  }
+  });
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) bl += __shfl_xor_sync(kAll, bl, o);
-  if (lane == 0) sm[wid] = bl;
+  if (q) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      qf += __shfl_xor_sync(kAll, qf, o);
+      ql += __shfl_xor_sync(kAll, ql, o);
+      qh += __shfl_xor_sync(kAll, qh, o);
+    }
+  }
+  if (lane == 0) {
+    sm[wid] = bl;
+    if (q) {
+      es[3 * wid] = qf;
+      es[3 * wid + 1] = ql;
+      es[3 * wid + 2] = qh;
+    }
+  }
   __syncthreads();
   long long bnd = sm[0];
 #pragma unroll
   for (int w = 1; w < W; ++w) bnd += sm[w];
   c.G = (64 - __clzll(bnd)) + 20 - 62;
-  // the totals in units U and their exclusive prefix sums, P consecutive tiles
-  // a thread, chunk by chunk
-  long long carry = 0;
-  for (int base = 0; base < nt; base += TPB * P) {
+  // the totals in units U and their exclusive prefix sums, up to P consecutive
+  // tiles a thread (chunk by chunk when there are more)
+  for (int base = 0; base < nt; base += P * TPB) {
+    const int u0 = regs ? t0 : base + (int)threadIdx.x * P;
+    const int u1 = regs ? t1 : min(nt, u0 + P);
+    if (!regs) {
+#pragma unroll
+      for (int p = 0; p < P; ++p)
+        if (u0 + p < u1) r[p] = load_rec_l1(rec + u0 + p);
+    }
     long long v[P];
     long long tot = 0;
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-      const int t = base + threadIdx.x * P + p;
-      v[p] = 0;
-      if (t < nt) {
-        long long st;
-        int kt;
-        if (ks) {
-          st = O[t];
-          kt = ks[t];
-        } else {
-          const TileRec r = load_rec(rec + t);
-          st = r.s;
-          kt = r.k;
-        }
-        v[p] = to_run_units(st, kt, c.kmax, c.G);
-      }
+      v[p] = u0 + p < u1 ? to_run_units(r[p].s, r[p].k, c.kmax, c.G) : 0;
       tot += v[p];
     }
     long long inc = tot;
@@ -195,42 +256,36 @@ __device__ Combined combine_offsets(const TileRec* rec, int nt, long long* O, in
     }
     if (lane == 31) ss[wid] = inc;
     __syncthreads();
-    long long off = carry + (inc - tot), all = 0;
+    long long off = c.S + inc - tot;
 #pragma unroll
     for (int w = 0; w < W; ++w) {
       const long long x = ss[w];
       if (w < wid) off += x;
-      all += x;
+      c.S += x;
     }
 #pragma unroll
     for (int p = 0; p < P; ++p) {
-      const int t = base + threadIdx.x * P + p;
-      if (t < nt) O[t] = off;
+      if (u0 + p < u1) O[u0 + p] = off;
       off += v[p];
     }
-    carry += all;
-    if (base + TPB * P < nt) __syncthreads();  // every thread has read ss
+    if (base + P * TPB < nt) __syncthreads();  // every thread has read ss
   }
-  c.S = carry;
-  if (threadIdx.x == 0) O[nt] = carry;
-  if (q && wid == 0) {  // sum w^2 relative to 2^(2 k_max), in FP64, by the first warp
-    double acc = 0.0;
-    for (int t = lane; t < nt; t += 32) {
-      const int kt = ks ? ks[t] : load_rec(rec + t).k;
-      if (kt != kDeadTile) {
-        const int d2 = 2 * (c.kmax - kt);
-        if (d2 < 900) acc = acc + (double)__ldcg(q + t) * pow2i(-54 - d2);
-      }
-    }
+  if (threadIdx.x == 0) O[nt] = c.S;
+  if (q && threadIdx.x == ess_thread(TPB)) {
+    unsigned long long f = es[0], l = es[1], h = es[2];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc = acc + __shfl_xor_sync(kAll, acc, o);
-    if (lane == 0) {
-      const double sd = (double)carry * pow2i(c.G - 54);
-      qs[0] = acc > 0.0 ? (sd * sd) / acc : 0.0;
+    for (int w = 1; w < W; ++w) {
+      f += es[3 * w];
+      l += es[3 * w + 1];
+      h += es[3 * w + 2];
     }
+    const double acc =
+        ((double)h * 4294967296.0 + ((double)l + (double)f * 0x1p-32)) * pow2i(-54);
+    const double sd = (double)c.S * pow2i(c.G - 54);
+    c.ess = acc > 0.0 ? (sd * sd) / acc : 0.0;
   }
-  __syncthreads();  // the offsets (and the ESS) for every thread
-  if (q) c.ess = qs[0];
+  after(c);
+  __syncthreads();  // the offsets and after()'s results for every thread
   return c;
 }
 

@@ -402,62 +402,104 @@ RunDev make_rundev(const smc_model_s* m, const smc_run_cfg* c, const Layout& Ly,
   return A;
 }
 
-cudaError_t launch_wave(const WavePlan& W, int precision, cudaStream_t st, unsigned wave) {
-  // waves whose runs all run the linear-Gaussian or the CRBD model launch that
-  // model's own kernel (smc_waves_kind.cu); others dispatch per run
-  if (W.kind == SMC_MODEL_LG || W.kind == SMC_MODEL_CRBD)
-    return launch_wave_kind(W, precision, st, wave);
-  for (int b = 0; b < 4; ++b) {
-    if (!W.n_ctas[b]) continue;
-    cudaError_t e = precision == SMC_PREC_FP32
-                        ? launch_bucket<float, 0>(b, W.runs, W.maps[b], W.n_ctas[b], st, wave)
-                        : launch_bucket<double, 0>(b, W.runs, W.maps[b], W.n_ctas[b], st, wave);
+ChainStreams::~ChainStreams() {
+  for (cudaEvent_t e : done_) cudaEventDestroy(e);
+  if (ready_) cudaEventDestroy(ready_);
+  for (cudaStream_t s : s_) cudaStreamDestroy(s);
+}
+
+cudaError_t ChainStreams::init(int n) {
+  cudaError_t e = cudaEventCreateWithFlags(&ready_, cudaEventDisableTiming);
+  for (int i = 0; i < n && e == cudaSuccess; ++i) {
+    cudaStream_t s;
+    if ((e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking)) != cudaSuccess) break;
+    s_.push_back(s);
+    cudaEvent_t ev;
+    if ((e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) != cudaSuccess) break;
+    done_.push_back(ev);
+  }
+  return e;
+}
+
+cudaError_t ChainStreams::fork(cudaStream_t main, int chains) {
+  cudaError_t e = cudaEventRecord(ready_, main);
+  for (int i = 0; i < std::min(chains, size()) && e == cudaSuccess; ++i)
+    e = cudaStreamWaitEvent(s_[(size_t)i], ready_, 0);
+  return e;
+}
+
+cudaError_t ChainStreams::join(cudaStream_t main, int chains) {
+  cudaError_t e = cudaSuccess;
+  for (int i = 0; i < std::min(chains, size()) && e == cudaSuccess; ++i) {
+    e = cudaEventRecord(done_[(size_t)i], s_[(size_t)i]);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(main, done_[(size_t)i], 0);
+  }
+  return e;
+}
+
+namespace {
+cudaError_t launch_chain(const WavePlan& W, const WaveChain& c, int precision, cudaStream_t st,
+                         unsigned wave) {
+  switch (c.kind) {
+    case SMC_MODEL_LG: return launch_kind<SMC_MODEL_LG>(c, W.runs, precision, st, wave);
+    case SMC_MODEL_CRBD: return launch_kind<SMC_MODEL_CRBD>(c, W.runs, precision, st, wave);
+    case SMC_MODEL_RATESHIFT: return launch_kind<SMC_MODEL_RATESHIFT>(c, W.runs, precision, st, wave);
+    case SMC_MODEL_SEIR: return launch_kind<SMC_MODEL_SEIR>(c, W.runs, precision, st, wave);
+    case SMC_MODEL_CRBD_DS: return launch_kind<SMC_MODEL_CRBD_DS>(c, W.runs, precision, st, wave);
+    default: return launch_kind<SMC_MODEL_GEOMETRIC>(c, W.runs, precision, st, wave);
+  }
+}
+}  // namespace
+
+cudaError_t launch_wave(const WavePlan& W, int precision, cudaStream_t st, unsigned wave,
+                        const ChainStreams* streams) {
+  for (size_t i = 0; i < W.chains.size(); ++i) {
+    const cudaError_t e = launch_chain(W, W.chains[i], precision,
+                                       streams ? streams->at((int)i) : st, wave);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
 
-// The model kind shared by every run of a wave plan (0 when they differ).
-int uniform_kind(const std::vector<RunDev>& runs) {
-  if (runs.empty()) return 0;
-  const int k = runs[0].md.kind;
-  for (const RunDev& r : runs)
-    if (r.md.kind != k) return 0;
-  return k;
-}
-
 size_t wave_meta_bytes(const std::vector<RunDev>& runs) {
   size_t n_ctas = 0;
   for (const RunDev& r : runs) n_ctas += (size_t)r.n_tiles;
-  return align_up(sizeof(RunDev) * runs.size(), 256) + align_up(sizeof(int2) * n_ctas, 256) + 4 * 256;
+  return align_up(sizeof(RunDev) * runs.size(), 256) + align_up(sizeof(int2) * n_ctas, 256) +
+         kMaxChains * 256;
 }
 
-// Copies the run table and the per-bucket CTA maps to `meta` (device) and
-// fills W with their device addresses.
+size_t fill_plan(const std::vector<RunDev>& runs, char* host, void* dev, WavePlan* W) {
+  std::vector<int2> maps[kMaxChains];
+  for (size_t r = 0; r < runs.size(); ++r) {
+    std::vector<int2>& m = maps[(runs[r].md.kind - 1) * 4 + bucket_for(runs[r].tile)];
+    for (int t = 0; t < runs[r].n_tiles; ++t) m.push_back(make_int2((int)r, t));
+  }
+  std::memcpy(host, runs.data(), sizeof(RunDev) * runs.size());
+  size_t off = align_up(sizeof(RunDev) * runs.size(), 256);
+  W->runs = (const RunDev*)dev;
+  W->chains.clear();
+  for (int c = 0; c < kMaxChains; ++c) {
+    if (maps[c].empty()) continue;
+    WaveChain w;
+    w.kind = c / 4 + 1;
+    w.bucket = c % 4;
+    w.n_ctas = (int)maps[c].size();
+    w.map = (const int2*)((char*)dev + off);
+    W->chains.push_back(w);
+    std::memcpy(host + off, maps[c].data(), sizeof(int2) * maps[c].size());
+    off = align_up(off + sizeof(int2) * maps[c].size(), 256);
+  }
+  return off;
+}
+
 // The run table and CTA maps to device memory at `meta`.  From pageable
 // staging the call waits for the copy; from `pinned` (at least
 // wave_meta_bytes(runs), not rewritten before the copy has run) it does not.
 smc_status upload_wave(const std::vector<RunDev>& runs, void* meta, cudaStream_t st, WavePlan* W,
                        std::vector<char>* staging, char* pinned) {
-  const size_t run_bytes = align_up(sizeof(RunDev) * runs.size(), 256);
-  std::vector<int2> maps[4];
-  for (size_t r = 0; r < runs.size(); ++r) {
-    const int b = bucket_for(runs[r].tile);
-    for (int t = 0; t < runs[r].n_tiles; ++t) maps[b].push_back(make_int2((int)r, t));
-  }
-  staging->assign(wave_meta_bytes(runs), 0);
-  std::memcpy(staging->data(), runs.data(), sizeof(RunDev) * runs.size());
-  size_t off = run_bytes;
-  W->runs = (const RunDev*)meta;
-  for (int b = 0; b < 4; ++b) {
-    W->n_ctas[b] = (int)maps[b].size();
-    W->maps[b] = (const int2*)((char*)meta + off);
-    if (!maps[b].empty()) std::memcpy(staging->data() + off, maps[b].data(), sizeof(int2) * maps[b].size());
-    off = align_up(off + sizeof(int2) * maps[b].size(), 256);
-  }
-  W->kind = uniform_kind(runs);
+  if (!pinned) staging->assign(wave_meta_bytes(runs), 0);
+  const size_t off = fill_plan(runs, pinned ? pinned : staging->data(), meta, W);
   if (pinned) {
-    std::memcpy(pinned, staging->data(), off);
     SMC_CUDA_TRY(cudaMemcpyAsync(meta, pinned, off, cudaMemcpyHostToDevice, st));
     return SMC_OK;
   }
@@ -474,11 +516,8 @@ namespace {
 // index, so a graph captured for the same addresses, CTA counts, precision and
 // number of waves is reusable once the run table (device memory) is uploaded.
 bool graph_matches(const GraphCache* g, const WavePlan& W, int precision, int max_waves) {
-  if (!g->exec || g->runs != W.runs || g->precision != precision || g->waves != max_waves)
-    return false;
-  for (int b = 0; b < 4; ++b)
-    if (g->maps[b] != W.maps[b] || g->n_ctas[b] != W.n_ctas[b]) return false;
-  return true;
+  return g->exec && g->plan.runs == W.runs && g->precision == precision && g->waves == max_waves &&
+         g->plan.chains == W.chains;
 }
 
 // Capture max_waves waves on `st` into a graph and instantiate it into g.
@@ -500,29 +539,26 @@ smc_status capture_waves(GraphCache* g, const WavePlan& W, int precision, int ma
     g->exec = nullptr;
     return cuda_fail(e, "cudaGraphInstantiate(waves)");
   }
-  g->runs = W.runs;
+  g->plan = W;
   g->precision = precision;
   g->waves = max_waves;
-  for (int b = 0; b < 4; ++b) {
-    g->maps[b] = W.maps[b];
-    g->n_ctas[b] = W.n_ctas[b];
-  }
   return SMC_OK;
 }
 
 // Runs waves until every run is done or `max_waves` waves ran.  Known-length
 // batches launch exactly max_waves waves without reading anything back (as one
-// CUDA graph when `graph` is given and the stream can be captured); otherwise
+// CUDA graph when `graph` is given and the stream can be captured; on the chains'
+// own streams when `streams` is given); otherwise
 // the run states are polled every 16 waves.  A run of S segments needs S + 1
 // waves: the wave after its last segment combines that segment.
 smc_status drive_waves(const WavePlan& W, int precision, const std::vector<RunState*>& states,
                        int max_waves, bool known, cudaStream_t st, std::vector<cudaEvent_t>* evs,
-                       bool timed, int* launched, double* kernel_ms, GraphCache* graph = nullptr) {
+                       bool timed, int* launched, double* kernel_ms, GraphCache* graph = nullptr,
+                       ChainStreams* streams = nullptr) {
   *launched = 0;
   *kernel_ms = 0.0;
   timed = timed && evs;
-  int kernels_per_wave = 0;
-  for (int b = 0; b < 4; ++b) kernels_per_wave += W.n_ctas[b] ? 1 : 0;
+  const int kernels_per_wave = (int)W.chains.size();
   if (known && graph && !timed && st != nullptr && st != cudaStreamLegacy) {
     if (!graph_matches(graph, W, precision, max_waves)) {
       smc_status s = capture_waves(graph, W, precision, max_waves, st);
@@ -542,17 +578,21 @@ smc_status drive_waves(const WavePlan& W, int precision, const std::vector<RunSt
       }
       SMC_CUDA_TRY(cudaEventRecord((*evs)[2 * waves], st));
     }
-    SMC_CUDA_TRY(launch_wave(W, precision, st, (unsigned)waves));
+    SMC_CUDA_TRY(launch_wave(W, precision, st, (unsigned)waves, streams));
     if (timed) SMC_CUDA_TRY(cudaEventRecord((*evs)[2 * waves + 1], st));
     ++waves;
     *launched += kernels_per_wave;
     return SMC_OK;
   };
   if (known) {
-    for (int k = 0; k < max_waves; ++k) {
-      smc_status s = one();
-      if (s) return s;
+    smc_status s = SMC_OK;
+    if (streams) SMC_CUDA_TRY(streams->fork(st, kernels_per_wave));
+    for (int k = 0; k < max_waves && !s; ++k) s = one();
+    if (streams) {  // after an error too: what was launched still uses the workspace
+      const cudaError_t e = streams->join(st, kernels_per_wave);
+      if (!s && e != cudaSuccess) s = cuda_fail(e, "joining the chains' streams");
     }
+    if (s) return s;
   } else {
     const int chunk = 16;
     const size_t n_runs = states.size();
@@ -1127,8 +1167,12 @@ extern "C" smc_status smc_run_batch(const smc_model_t* ms, const smc_run_cfg* cf
   int launched = 0;
   double kms = 0.0;
   GraphCache graph;
+  const bool graphed = cfgs[0].launch_mode == SMC_LAUNCH_GRAPH;
+  ChainStreams streams;
+  const bool fan = known && !graphed && W.chains.size() > 1;
+  if (fan) SMC_CUDA_TRY(streams.init(std::min((int)W.chains.size(), kChainStreams)));
   st = drive_waves(W, prec, states, max_waves + 1, known, cs, nullptr, false, &launched, &kms,
-                   cfgs[0].launch_mode == SMC_LAUNCH_GRAPH ? &graph : nullptr);
+                   graphed ? &graph : nullptr, fan ? &streams : nullptr);
   if (st) {
     graph_cache_clear(&graph);
     cudaEventDestroy(e0);

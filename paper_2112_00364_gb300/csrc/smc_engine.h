@@ -79,21 +79,55 @@ struct Layout {
   int n_tiles, tile, pad, anc_rows, max_segments;
 };
 
-// Device addresses of one wave's run table and per-bucket CTA maps.
+// One model and CTA size among the runs of a set: a wave of the set is one launch
+// per chain, and a chain's launches depend on one another only (every run belongs
+// to one chain).
+struct WaveChain {
+  int kind = 0, bucket = 0, n_ctas = 0;
+  const int2* map = nullptr;  // CTA -> (run, tile)
+  bool operator==(const WaveChain& o) const {
+    return kind == o.kind && bucket == o.bucket && n_ctas == o.n_ctas && map == o.map;
+  }
+};
+constexpr int kMaxChains = 6 * 4;
+constexpr int kChainStreams = 8;  // two models in four CTA sizes have a stream each
+
+// Device addresses of one set's run table and its chains.
 struct WavePlan {
   const RunDev* runs = nullptr;
-  const int2* maps[4] = {nullptr, nullptr, nullptr, nullptr};
-  int n_ctas[4] = {0, 0, 0, 0};
-  int kind = 0;  // the model of every run of the plan (SMC_MODEL_*), 0 when they differ
+  std::vector<WaveChain> chains;
+};
+
+// Streams for a set's chains beside the stream its caller works on, so that a
+// chain's waves need not wait for the slowest CTAs of the others' (on one stream
+// every launch waits for the launch before it).  fork(): the chains' work waits for
+// what `main` holds so far; join(): `main` waits for the chains' work so far.
+// Chain i runs on stream i modulo the number of streams.  Owned by one batch call
+// or one server; its streams are idle when it is destroyed (after a join that the
+// owner has waited for).
+class ChainStreams {
+ public:
+  ChainStreams() = default;
+  ChainStreams(const ChainStreams&) = delete;
+  ChainStreams& operator=(const ChainStreams&) = delete;
+  ~ChainStreams();
+  cudaError_t init(int n);
+  cudaError_t fork(cudaStream_t main, int chains);
+  cudaError_t join(cudaStream_t main, int chains);
+  cudaStream_t at(int chain) const { return s_[(size_t)chain % s_.size()]; }
+  int size() const { return (int)s_.size(); }
+
+ private:
+  std::vector<cudaStream_t> s_;
+  std::vector<cudaEvent_t> done_;
+  cudaEvent_t ready_ = nullptr;
 };
 
 // An instantiated CUDA graph of a known-length sequence of waves and the wave
 // plan it was captured for.
 struct GraphCache {
   cudaGraphExec_t exec = nullptr;
-  const RunDev* runs = nullptr;
-  const int2* maps[4] = {nullptr, nullptr, nullptr, nullptr};
-  int n_ctas[4] = {0, 0, 0, 0};
+  WavePlan plan;
   int precision = -1, waves = 0;
 };
 void graph_cache_clear(GraphCache* g);
@@ -147,10 +181,16 @@ RunDev make_rundev(const smc_model_s* m, const smc_run_cfg* c, const Layout& Ly,
 size_t wave_meta_bytes(const std::vector<RunDev>& runs);
 smc_status upload_wave(const std::vector<RunDev>& runs, void* meta, cudaStream_t st, WavePlan* W,
                        std::vector<char>* staging, char* pinned = nullptr);
-cudaError_t launch_wave(const WavePlan& W, int precision, cudaStream_t st, unsigned wave);
-// the waves of a plan whose runs all run the linear-Gaussian or the CRBD model
-cudaError_t launch_wave_kind(const WavePlan& W, int precision, cudaStream_t st, unsigned wave);
-int uniform_kind(const std::vector<RunDev>& runs);
+// The run table and CTA maps of a set of runs into `host` (at least
+// wave_meta_bytes(runs)), the plan for them at the device address `dev`; returns
+// the bytes to copy.
+size_t fill_plan(const std::vector<RunDev>& runs, char* host, void* dev, WavePlan* W);
+// One wave: every chain's launch, on `st`, or each on its own stream with `streams`.
+cudaError_t launch_wave(const WavePlan& W, int precision, cudaStream_t st, unsigned wave,
+                        const ChainStreams* streams = nullptr);
+template <int KIND>
+cudaError_t launch_kind(const WaveChain& c, const RunDev* runs, int precision, cudaStream_t st,
+                        unsigned wave);
 smc_status collect_run(const smc_model_s* m, const smc_run_cfg* c, const Layout& Ly, char* ws,
                        const RunDev& A, const RunState& hrs, smc_result* r, cudaStream_t cs);
 smc_status check_cfg(const smc_model_s* m, const smc_run_cfg* c);

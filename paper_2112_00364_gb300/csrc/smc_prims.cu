@@ -427,7 +427,8 @@ __global__ void __launch_bounds__(RS_COMBINE_TPB) rs_combine(const TileRec* __re
   const Combined c = nt <= 4 * RS_COMBINE_TPB
                          ? combine_small(rec, nt, O, reinterpret_cast<long long*>(sh),
                                          reinterpret_cast<int*>(sh + 64))
-                         : combine_offsets<RS_COMBINE_TPB>(rec, nt, O, nullptr, sh);
+                         : combine_offsets<RS_COMBINE_TPB>(rec, nt, O, nullptr, sh, nullptr,
+                                                           [](const Combined&) {});
   // the log-Z increment (thread 0) and the search scalars (thread 32) in parallel
   if (c.kmax == kDeadTile) {
     if (threadIdx.x == 0) {

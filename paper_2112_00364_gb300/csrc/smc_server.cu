@@ -97,6 +97,7 @@ struct Server {
   size_t budget;
   int device = 0;
   cudaStream_t stream = nullptr;
+  ChainStreams chains;
   std::thread worker;
   std::mutex mu;
   std::condition_variable cv_work, cv_done;
@@ -171,22 +172,7 @@ smc_status upload_table(Server* S) {
     SMC_CUDA_TRY(cudaMallocHost(&S->pinned_meta, sz));
     S->pinned_meta_bytes = sz;
   }
-  // same layout as upload_wave, written into pinned staging
-  std::vector<int2> maps[4];
-  for (size_t r = 0; r < runs.size(); ++r) {
-    const int b = bucket_for(runs[r].tile);
-    for (int t = 0; t < runs[r].n_tiles; ++t) maps[b].push_back(make_int2((int)r, t));
-  }
-  std::memcpy(S->pinned_meta, runs.data(), sizeof(RunDev) * runs.size());
-  size_t off = align_up(sizeof(RunDev) * runs.size(), 256);
-  S->plan.runs = (const RunDev*)S->meta;
-  for (int b = 0; b < 4; ++b) {
-    S->plan.n_ctas[b] = (int)maps[b].size();
-    S->plan.maps[b] = (const int2*)((char*)S->meta + off);
-    if (!maps[b].empty()) std::memcpy(S->pinned_meta + off, maps[b].data(), sizeof(int2) * maps[b].size());
-    off = align_up(off + sizeof(int2) * maps[b].size(), 256);
-  }
-  S->plan.kind = uniform_kind(runs);
+  const size_t off = fill_plan(runs, S->pinned_meta, S->meta, &S->plan);
   SMC_CUDA_TRY(cudaMemcpyAsync(S->meta, S->pinned_meta, off, cudaMemcpyHostToDevice, S->stream));
   SMC_CUDA_TRY(cudaEventRecord(S->meta_ev, S->stream));
   S->table_dirty = false;
@@ -382,12 +368,23 @@ void worker_main(Server* S) {
     if (S->table_dirty && (err = upload_table(S))) break;
     const int per_poll = std::max(1, S->cfg.poll_waves);
     NvtxRange nv_waves("smc_server/waves");
-    for (int w = 0; w < per_poll && !err; ++w) {
-      cudaError_t e = launch_wave(S->plan, S->cfg.precision, S->stream, (unsigned)S->waves.load());
-      if (e != cudaSuccess) err = cuda_fail(e, "wave launch");
+    // the chains (models and CTA sizes) side by side on their own streams
+    const int n_chains = (int)S->plan.chains.size();
+    const bool fan = n_chains > 1;
+    cudaError_t we = fan ? S->chains.fork(S->stream, n_chains) : cudaSuccess;
+    for (int w = 0; w < per_poll && we == cudaSuccess; ++w) {
+      we = launch_wave(S->plan, S->cfg.precision, S->stream, (unsigned)S->waves.load(),
+                       fan ? &S->chains : nullptr);
       S->waves += 1;
     }
-    if (err) break;
+    if (fan) {  // after an error too: the drain below waits for S->stream alone
+      const cudaError_t je = S->chains.join(S->stream, n_chains);
+      if (we == cudaSuccess) we = je;
+    }
+    if (we != cudaSuccess) {
+      err = cuda_fail(we, "wave launch");
+      break;
+    }
     // flags of this wave into buffer `parity`
     const int n = (int)S->resident.size();
     gather_flags_kernel<<<(n + 127) / 128, 128, 0, S->stream>>>(S->plan.runs, n, S->flags_dev);
@@ -453,6 +450,7 @@ extern "C" smc_status smc_server_create(size_t device_mem_budget, const smc_serv
   S->budget = device_mem_budget;
   cudaError_t e = cudaGetDevice(&S->device);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&S->stream, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = S->chains.init(kChainStreams);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&S->meta_ev, cudaEventDisableTiming);
   for (int b = 0; b < 2 && e == cudaSuccess; ++b)
     e = cudaEventCreateWithFlags(&S->flags_ev[b], cudaEventDisableTiming);

@@ -281,14 +281,69 @@ __device__ __forceinline__ int systematic_search(int i, int near_t, const RunDev
 // A CTA's shared memory.
 template <int TPB>
 struct StepShared {
-  double red[4 * (TPB / 32) + 1];  // combine_offsets' reductions
+  double red[combine_scratch(TPB)];  // combine_offsets' reductions
+  double ess;                      // its effective sample size
   unsigned long long scal[5];      // the search scalars
   unsigned long long uf;           // u 2^64 of the search they are for
   long long sum[TPB / 32], sq[TPB / 32];  // the warps' weight sums (and of their squares)
   unsigned draws[TPB / 32], execs[TPB / 32];
-  int kw[TPB / 32], last;
+  int kw[TPB / 32], last, resample;
   long long O[redundant_cap(TPB)];  // the offsets of a run combined in every CTA
   int ks[redundant_cap(TPB)];       // and its tiles' reference exponents
+};
+
+// What the combine's threads publish: for a run combined in every CTA, the
+// decision and the search scalars in shared memory, a thread each.
+template <int TPB>
+struct PublishShared {
+  const RunDev* A;
+  StepShared<TPB>* S;
+  __device__ __forceinline__ void operator()(const Combined& x) const {
+    if (threadIdx.x == ess_thread(TPB)) {
+      S->ess = x.ess;
+      S->resample = decide_resample(*A, x);
+    }
+    if (threadIdx.x == 0) {
+      Q64 d, z0;
+      long long tolZ;
+      search_scalars(x, A->N, A->recip_n, S->uf, &d, &z0, &tolZ);
+      S->scal[0] = d.hi;
+      S->scal[1] = d.lo;
+      S->scal[2] = z0.hi;
+      S->scal[3] = z0.lo;
+      S->scal[4] = (unsigned long long)tolZ;
+    }
+  }
+};
+
+// For a run combined in the last CTA of segment k: the decision and the closing
+// (log Z, its records), and the next search's scalars, a thread each.
+template <int TPB>
+struct PublishRun {
+  const RunDev* A;
+  StepShared<TPB>* S;
+  int k;
+  __device__ __forceinline__ void operator()(const Combined& x) const {
+    RunState* rs = A->rs;
+    if (threadIdx.x == ess_thread(TPB)) {
+      const bool resample = decide_resample(*A, x);
+      rs->resample = resample ? 1 : 0;
+      finish_segment(*A, k + 1, x, resample);
+      rs->arrive = 0;
+    }
+    if (threadIdx.x == 0 && x.kmax != kDeadTile) {
+      Q64 d, z0;
+      long long tolZ;
+      search_scalars(x, A->N, A->recip_n, S->uf, &d, &z0, &tolZ);
+      rs->kmax = x.kmax;
+      rs->G = x.G;
+      rs->d_hi = d.hi;
+      rs->d_lo = d.lo;
+      rs->z0_hi = z0.hi;
+      rs->z0_lo = z0.lo;
+      rs->tolZ = tolZ;
+    }
+  }
 };
 
 // One tile of one run for segment k (the whole per-CTA body of a wave).
@@ -317,25 +372,19 @@ __device__ __forceinline__ void step_tile(const RunDev& A, const int t, const in
     X.rec = A.rec[cb];
     bool resample;
     if (redundant) {
-      const Combined c = combine_offsets<TPB>(A.rec[cb], A.n_tiles, S.O, S.ks, S.red,
-                                              A.ess ? A.tq[cb] : nullptr);
+      // two threads form the decision and the search scalars, for all to read
+      const Combined c = combine_offsets<TPB>(
+          A.rec[cb], A.n_tiles, S.O, S.ks, S.red, A.ess ? A.tq[cb] : nullptr,
+          PublishShared<TPB>{&A, &S});
       const bool go_on = c.kmax != kDeadTile && c.alive && k < A.max_segments;
-      resample = decide_resample(A, c);
-      // (by the tile's last thread: its warp is the one most often without particles)
-      if (t == 0 && threadIdx.x == TPB - 1) finish_segment(A, k, c, resample);
-      if (!go_on) return;
-      // the run's search scalars by one thread, shared through shared memory
-      if (resample && threadIdx.x == 0) {
-        Q64 d, z0;
-        long long tolZ;
-        search_scalars(c, N, A.recip_n, S.uf, &d, &z0, &tolZ);
-        S.scal[0] = d.hi;
-        S.scal[1] = d.lo;
-        S.scal[2] = z0.hi;
-        S.scal[3] = z0.lo;
-        S.scal[4] = (unsigned long long)tolZ;
+      resample = S.resample != 0;
+      // (closed by the tile's last thread: its warp is the one most often without particles)
+      if (t == 0 && threadIdx.x == TPB - 1) {
+        Combined x = c;
+        x.ess = S.ess;
+        finish_segment(A, k, x, resample);
       }
-      __syncthreads();
+      if (!go_on) return;
       X.O = S.O;
       X.ks = S.ks;
       X.kmax = c.kmax;
@@ -444,6 +493,12 @@ __device__ __forceinline__ void step_tile(const RunDev& A, const int t, const in
     S.draws[wid] = draws;
     S.execs[wid] = execs;
   }
+  // The next wave's CTAs may start now (this one's particles are done): earlier
+  // they would hold places on the SMs that other chains' CTAs can use, later their
+  // start is not hidden.  At the CTA's start / here / at its end: batch of 512
+  // 142.9 / 140.3 / 139.9 ms, CRBD 64k 24.2 / 24.0 / 24.5 us a wave, delayed
+  // sampling 68.6 / 67.9 / 66.8, linear-Gaussian 23k 9.71 / 9.76 / 9.95.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   alive = __syncthreads_or(alive);
   int kt = S.kw[0];
 #pragma unroll
@@ -505,37 +560,34 @@ __device__ __forceinline__ void step_tile(const RunDev& A, const int t, const in
   __syncthreads();
   if (S.last) {  // the run's last tile of segment k: combine for the next wave
     __threadfence();
+    const PublishRun<TPB> close{&A, &S, k};
     const Combined c = combine_offsets<TPB>(A.rec[nb], A.n_tiles, A.tile_O, nullptr, S.red,
-                                            A.ess ? A.tq[nb] : nullptr);
-    // closing the segment (log Z, its records) and the next search's scalars, by a
-    // thread each
-    const bool resample = decide_resample(A, c);
-    if (threadIdx.x == TPB - 1) {
-      rs->resample = resample ? 1 : 0;
-      finish_segment(A, k + 1, c, resample);
-      rs->arrive = 0;
-    }
-    if (threadIdx.x == 0 && resample && c.kmax != kDeadTile) {
-      Q64 d, z0;
-      long long tolZ;
-      search_scalars(c, N, A.recip_n, S.uf, &d, &z0, &tolZ);
-      rs->kmax = c.kmax;
-      rs->G = c.G;
-      rs->d_hi = d.hi;
-      rs->d_lo = d.lo;
-      rs->z0_hi = z0.hi;
-      rs->z0_lo = z0.lo;
-      rs->tolZ = tolZ;
-    }
+                                            A.ess ? A.tq[nb] : nullptr, close);
+    if (c.kmax == kDeadTile) close(c);
   }
 }
+
+// The block table of a model kind.
+template <int KIND, typename R>
+struct ModelOf;
+template <typename R>
+struct ModelOf<SMC_MODEL_LG, R> { using type = LgModel<R>; };
+template <typename R>
+struct ModelOf<SMC_MODEL_CRBD, R> { using type = TreeModel<R, false>; };
+template <typename R>
+struct ModelOf<SMC_MODEL_RATESHIFT, R> { using type = TreeModel<R, true>; };
+template <typename R>
+struct ModelOf<SMC_MODEL_GEOMETRIC, R> { using type = GeoModel<R>; };
+template <typename R>
+struct ModelOf<SMC_MODEL_SEIR, R> { using type = SeirModel<R>; };
+template <typename R>
+struct ModelOf<SMC_MODEL_CRBD_DS, R> { using type = TreeDsModel<R>; };
 
 // One wave: CTA b runs tile cta_map[b].y of run cta_map[b].x, segment
 // k = wave - start_wave of that run.
 // 768 resident threads per SM (three 256-thread CTAs: the grid sizing of
 // tile_for) bounds the kernel to 85 registers per thread.
-// KIND 0 dispatches on each run's model; a KIND of SMC_MODEL_* is the kernel of
-// waves whose runs all run that model (only its block table is compiled in).
+// KIND: the model (SMC_MODEL_*) that every run of the launch runs.
 template <typename R, int TPB, int KIND>
 __global__ void __launch_bounds__(TPB, (sizeof(R) == 4 ? 1024 : 768) / TPB) wave_kernel(const RunDev* __restrict__ runs,
                                                    const int2* __restrict__ cta_map, unsigned wave) {
@@ -548,11 +600,10 @@ __global__ void __launch_bounds__(TPB, (sizeof(R) == 4 ? 1024 : 768) / TPB) wave
     for (int w = threadIdx.x; w < (int)(sizeof(RunDev) / 4); w += TPB) dst[w] = src[w];
   }
   __syncthreads();
-  // Waves are launched with programmatic stream serialisation: the next wave's
-  // CTAs may start (and copy their run table, which no kernel writes) while
-  // this wave's last CTAs still run; everything below reads what the previous
-  // wave wrote, so it waits for that wave's completion first.
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // Waves are launched with programmatic stream serialisation: a wave's CTAs may
+  // start (and copy their run table, which no kernel writes) while the last CTAs
+  // of the previous one still run; everything below reads what that wave wrote, so
+  // it waits for its completion first.
   const int k = (int)(wave - sr.start_wave);  // wraps correctly past 2^32 waves
   // the uniform of the search whose scalars this CTA may form, from the counter
   // alone: in the wait's shadow
@@ -560,22 +611,7 @@ __global__ void __launch_bounds__(TPB, (sizeof(R) == 4 ? 1024 : 768) / TPB) wave
   asm volatile("griddepcontrol.wait;" ::: "memory");
   RunState* rs = sr.rs;
   if (*(volatile int32_t*)&rs->done || k < 0) return;
-  if (KIND == SMC_MODEL_LG) {
-    step_tile<LgModel<R>, TPB>(sr, rt.y, k, S);
-    return;
-  }
-  if (KIND == SMC_MODEL_CRBD) {
-    step_tile<TreeModel<R, false>, TPB>(sr, rt.y, k, S);
-    return;
-  }
-  switch (sr.md.kind) {
-    case SMC_MODEL_LG: step_tile<LgModel<R>, TPB>(sr, rt.y, k, S); break;
-    case SMC_MODEL_SEIR: step_tile<SeirModel<R>, TPB>(sr, rt.y, k, S); break;
-    case SMC_MODEL_CRBD: step_tile<TreeModel<R, false>, TPB>(sr, rt.y, k, S); break;
-    case SMC_MODEL_RATESHIFT: step_tile<TreeModel<R, true>, TPB>(sr, rt.y, k, S); break;
-    case SMC_MODEL_CRBD_DS: step_tile<TreeDsModel<R>, TPB>(sr, rt.y, k, S); break;
-    default: step_tile<GeoModel<R>, TPB>(sr, rt.y, k, S); break;
-  }
+  step_tile<typename ModelOf<KIND, R>::type, TPB>(sr, rt.y, k, S);
 }
 
 // One bucket of a wave, launched so that it may begin before the kernel ahead

@@ -1,0 +1,23 @@
+// smc_waves.cuh -- launching the wave kernels of one model.  A wave of a set of
+// runs is one launch per model and CTA size among them (a chain of such launches,
+// wave after wave): each kernel holds one model's block table only, so its code
+// and registers (one kernel dispatching on each run's model spilled 250 bytes a
+// thread at the 64 registers of FP32 particles: 150 us instead of 143 a rate-shift
+// wave of 2^20).  Each model is compiled in a translation unit of its own.
+#pragma once
+#include <cuda_runtime.h>
+
+#include "smc_engine.h"
+#include "smc_step.cuh"
+
+namespace smc {
+
+template <int KIND>
+cudaError_t launch_kind(const WaveChain& c, const RunDev* runs, int precision, cudaStream_t st,
+                        unsigned wave) {
+  return precision == SMC_PREC_FP32
+             ? launch_bucket<float, KIND>(c.bucket, runs, c.map, c.n_ctas, st, wave)
+             : launch_bucket<double, KIND>(c.bucket, runs, c.map, c.n_ctas, st, wave);
+}
+
+}  // namespace smc
