@@ -892,7 +892,7 @@ __device__ __forceinline__ R beta_ab(Stream& s, R a, R b) {
 // (BTRS, 1993), one block per trial, acceptance in logs with log k!, at most
 // 1000 trials.
 template <typename R>
-__device__ __noinline__ int binomial(Stream& s, int n, R p) {
+__device__ __noinline__ int binomial_exact(Stream& s, int n, R p) {
   if (n <= 0 || !(p > (R)0.0)) return 0;
   if (!(p < (R)1.0)) return n;
   const bool flip = p > (R)0.5;
@@ -941,6 +941,175 @@ __device__ __noinline__ int binomial(Stream& s, int n, R p) {
     }
   }
   return flip ? n - k : k;
+}
+
+
+// ---- the same draw decided in single precision (FP64 particles) ----
+// A binomial draw is an integer: its sampler uses real numbers only in
+// comparisons.  binomial_exact takes 60 to 400 FP64 operations a draw, at a
+// 1/64 of the FP32 rate and with lanes at different terms and trials: the SEIR
+// model's 13 draws a day kept the FP64 pipe 82% busy.  (741 us a day at 65,536
+// particles; 87 with this.)  Here every comparison is made in single precision (integers where
+// a value's whole part is large) with a bound on its error; a draw whose
+// comparisons all clear their bounds is the integer that exact arithmetic gives,
+// any other (about 1 in 1000) is drawn again from its first block by
+// binomial_exact.
+
+// (1 + t) log(1 + t) - t for t > -1, given lt = log(1 + t) (which for |t| >= 0.2
+// it uses): the series t^2 sum (-t)^(j-2) / (j (j - 1)) to t^10 below 0.2.
+__device__ __forceinline__ float deviance(float t, float lt) {
+  if (fabsf(t) >= 0.2f) return fmaf(1.0f + t, lt, -t);
+  float g = fmaf(t, 1.0f / 90.0f, -1.0f / 72.0f);
+  g = fmaf(g, t, 1.0f / 56.0f);
+  g = fmaf(g, t, -1.0f / 42.0f);
+  g = fmaf(g, t, 1.0f / 30.0f);
+  g = fmaf(g, t, -1.0f / 20.0f);
+  g = fmaf(g, t, 1.0f / 12.0f);
+  g = fmaf(g, t, -1.0f / 6.0f);
+  g = fmaf(g, t, 0.5f);
+  return t * t * g;
+}
+// log Gamma(x) - ((x - 1/2) log x - x + log(2 pi) / 2) for whole x >= 1: from 5 on by
+// three terms of Stirling's series (the next is below 1e-8), exactly below.
+__device__ __forceinline__ float stirling(float x) {
+  if (x < 5.0f)
+    return x < 2.0f ? 0.0810614668f : x < 3.0f ? 0.0413406960f : x < 4.0f ? 0.0276779257f : 0.0207906721f;
+  const float ix = __fdividef(1.0f, x), ix2 = ix * ix;
+  return ix * (1.0f / 12.0f - ix2 * (1.0f / 360.0f - ix2 * (1.0f / 1260.0f)));
+}
+
+// binomial_exact's candidate of one rejection trial (-1: below 0)
+__device__ __noinline__ inline int btrs_candidate(int n, double p, Block4 blk) {
+  const double spq = sqrt((double)n * p * (1.0 - p));
+  const double b = 1.15 + 2.53 * spq;
+  const double a = -0.0873 + 0.0248 * b + 0.01 * p;
+  const double u = Unif<double>::first(blk) - 0.5;
+  const double kr = floor((2.0 * a / (0.5 - fabs(u)) + b) * u + ((double)n * p + 0.5));
+  if (kr < 0.0) return -1;
+  return kr > 2147483647.0 ? 2147483647 : (int)kr;
+}
+
+// The draw of Binomial(n, p'), p' = pd = P 2^-64 <= 1/2 (pp: p' as a float, within
+// 2^-23), or -1 where a comparison is too close to call.
+__device__ __forceinline__ int binomial_f32(Stream& s, int n, double pd, unsigned long long P,
+                                            float pp) {
+  const unsigned np = (unsigned)__umul64hi(P, (unsigned long long)n);        // floor(n p')
+  const unsigned nfr = (unsigned)((P * (unsigned long long)n) >> 32);        // its fraction 2^32
+  const float q = 1.0f - pp;
+  if ((np == 9u && nfr > 0xfffff000u) || (np == 10u && nfr < 0x1000u)) return -1;
+  if (np < 10u) {
+    // Inversion.  Errors, relative to the terms: n log q 3e-7 of a value below
+    // 1.39 n p', its exponential 2e-7, 6e-7 a term after it (so 6e-7 n p' on the
+    // average); the additions' 6e-8 of the sum each; u 2^-24:
+    // below 1.1e-6 n p' + 1.5e-6.
+    const float u = (float)(s.next().w1 >> 8) * 0x1p-24f;
+    const float npf = fmaf((float)nfr, 0x1p-32f, (float)np);
+    const float eps = fmaf(1.5e-6f, npf, 3e-6f);
+    const float r = __fdividef(pp, q);
+    float f = f32_exp((float)n * f32_log1p(-pp)), acc = f, c = 1.0f, rest = (float)n;
+    for (int k = 0; k < 60; ++k) {
+      if (u <= acc - eps) return k;
+      if (u < acc + eps || k >= n) return -1;
+      f = f * r * __fdividef(rest, c);
+      rest -= 1.0f;
+      c += 1.0f;
+      acc += f;
+    }
+    return -1;
+  }
+  // Transformed rejection.  With b below within 3e-7 relative, a within 7e-7, the
+  // offset x = (2a/us + b) u is within 1.5e-6 relative, and 2^-31/us of us;
+  // floor(x + n p' + 1/2) adds the whole part of n p' as an integer, and where x
+  // lies too near a whole number it is taken in FP64 (btrs_candidate).
+  const float npf = (float)n * pp;
+  const float spq = sqrtf(npf * q);
+  const float b = fmaf(2.53f, spq, 1.15f);
+  const float a = fmaf(0.01f, pp, fmaf(0.0248f, b, -0.0873f));
+  const float vr = 0.92f - __fdividef(4.2f, b);
+  const float cf = fmaf((float)nfr, 0x1p-32f, 0.5f);
+  for (int trial = 0; trial < 100; ++trial) {
+    const Block4 blk = s.next();
+    const int su = (int)(blk.w1 ^ 0x80000000u);  // u 2^32, u = U - 1/2
+    const unsigned us32 = su >= 0 ? 0x80000000u - (unsigned)su : 0x80000000u + (unsigned)su;
+    if (us32 < (1u << 16) || blk.w3 < (1u << 14)) return -1;
+    const float us = (float)us32 * 0x1p-32f;  // 1/2 - |u|
+    const float v = (float)blk.w3 * 0x1p-32f;
+    const float x = (__fdividef(2.0f * a, us) + b) * ((float)su * 0x1p-32f);
+    const float y = x + cf, fl = floorf(y), dy = y - fl;
+    const float ex = fmaf(fabsf(x), 2.5e-6f + __fdividef(0x1p-31f, us), 2e-6f);
+    int k = (int)np + (int)fl;
+    if (!(dy > ex && dy < 1.0f - ex)) k = btrs_candidate(n, pd, blk);
+    if (k < 0 || k > n) continue;
+    const int d07 = (int)us32 - 300647711;  // 0.07 2^32
+    if (d07 > -8 && d07 < 8) return -1;
+    if (d07 > 0) {
+      if (fabsf(v - vr) < 4e-6f) return -1;
+      if (v < vr) return k;
+    }
+    // log(v alpha / (a/us^2 + b)) against log f(k) - log f(m) at the mode
+    // m = floor((n + 1) p').  With X = k + 1, Y = n - k + 1, M = m + 1, W = n - m + 1,
+    // d = k - m, t = d/M, w = d/W, the difference of Stirling's forms is
+    //   d (log(p'/q) - log(M/W)) - M g(t) - W g(-w) + (log X/M + log Y/W) / 2 + corrections,
+    // g = deviance(): the large terms cancel on paper, not in the arithmetic.  (Where
+    // (n + 1) p' is all but whole, as for p' = 1/7 every seventh n, m may be either
+    // of two modes of the same probability.)
+    const unsigned long long n1 = (unsigned long long)n + 1ull;
+    const int m = (int)__umul64hi(P, n1);
+    const unsigned mfr = (unsigned)((P * n1) >> 32);
+    const float phi = (float)mfr * 0x1p-32f;  // (n + 1) p' - m
+    const float M = (float)(m + 1), W = (float)(n - m + 1), d = (float)(k - m);
+    const float t = __fdividef(d, M), w = -__fdividef(d, W);
+    const float lt = __logf(1.0f + t), lw = __logf(1.0f + w);
+    const float g1 = M * deviance(t, lt), g2 = W * deviance(w, lw);
+    const float mp = (float)n1 * pp, mq = (float)n1 * q;
+    const float slope = f32_log1p_core(__fdividef(phi, mq)) - f32_log1p_core(__fdividef(1.0f - phi, mp));
+    const float L = fmaf(d, slope, -g1 - g2) + 0.5f * (lt + lw) +
+                    ((stirling(M) - stirling((float)(k + 1))) + (stirling(W) - stirling((float)(n - k + 1))));
+    const float alpha = (2.83f + __fdividef(5.1f, b)) * spq;
+    const float lhs = __logf(__fdividef(v * alpha, fmaf(__fdividef(a, us), __fdividef(1.0f, us), b)));
+    // errors: 2e-6 of each deviance from its series; a logarithm's 4e-7 (2^-21.4 ln 2
+    // near 1) times M (1 + t) where it is used; the left side's argument 3e-6 and
+    // its logarithm 5e-6, the rest below 2e-6
+    float eL = fmaf(2e-6f, g1 + g2, 6e-5f) + __fdividef(0x1p-30f, us);
+    if (fabsf(t) >= 0.2f) eL = fmaf(8e-7f * M, 1.0f + t, eL);
+    if (fabsf(w) >= 0.2f) eL = fmaf(8e-7f * W, 1.0f + w, eL);
+    if (!(fabsf(lhs - L) > eL)) return -1;
+    if (lhs < L) return k;
+  }
+  return -1;
+}
+
+template <typename R>
+__device__ __forceinline__ int binomial(Stream& s, int n, R p) {
+  return binomial_exact<R>(s, n, p);
+}
+template <>
+__device__ __noinline__ inline int binomial<double>(Stream& s, int n, double p) {
+  if (n <= 0 || !(p > 0.0)) return 0;
+  if (!(p < 1.0)) return n;
+  const unsigned long long bits = (unsigned long long)__double_as_longlong(p);
+  const unsigned long long mant = (bits & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
+  const int sh = (int)(bits >> 52) - 1011;  // p 2^64 = mant 2^sh, sh <= 11
+  unsigned long long P = sh >= 0 ? mant << sh : shr64(mant, (unsigned)-sh);
+  float pp = trunc_f32((unsigned)(bits >> 32), (unsigned)bits);
+  const bool flip = P > (1ull << 63);
+  if (flip) {
+    P = 0ull - P;
+    pp = __ull2float_rn(P) * 0x1p-64f;
+  }
+  const uint32_t d0 = s.d;
+  const int k = binomial_f32(s, n, flip ? 1.0 - p : p, P, pp);
+  if (k >= 0) return flip ? n - k : k;
+  s.d = d0;
+  return binomial_exact<double>(s, n, p);
+}
+
+// 1 - e^(-i/n) for counts i >= 0, n > 0: FP64 with the exponential on the integer pipes
+__device__ __forceinline__ double one_minus_exp_ratio(int i, int n, const Stream& s, double) {
+  return 1.0 - exp_neg_int((double)i / (double)n, s.tab);
+}
+__device__ __forceinline__ float one_minus_exp_ratio(int i, int n, const Stream& s, float) {
+  return 1.0f - ex(-((float)i / (float)n), s);
 }
 
 // log Binomial(y | z, rho) (-inf for y > z); zero counts contribute nothing.

@@ -295,7 +295,7 @@ struct SeirModel {
       const int mSP = C[4], mEP = C[5], mIP = C[6], mRP = C[7];
       // humans
       const int hN = hSP + hEP + hIP + hRP;
-      const int hTau = binomial<R>(s, hSP, (R)1.0 - ex(-((R)mIP / (R)hN), s));
+      const int hTau = binomial<R>(s, hSP, one_minus_exp_ratio(mIP, hN, s, (R)0));
       const int hDeltaE = binomial<R>(s, hTau, th[0]);
       hDeltaI = binomial<R>(s, hEP, th[1]);
       const int hDeltaR = binomial<R>(s, hIP, th[2]);
@@ -304,7 +304,7 @@ struct SeirModel {
       C[2] = hIP + hDeltaI - hDeltaR;
       C[3] = hRP + hDeltaR;
       // mosquitoes
-      const int mTau = binomial<R>(s, mSP, (R)1.0 - ex(-((R)hIP / (R)hN), s));
+      const int mTau = binomial<R>(s, mSP, one_minus_exp_ratio(hIP, hN, s, (R)0));
       const int mN = mSP + mEP + mIP + mRP;
       const int mDeltaE = binomial<R>(s, mTau, th[3]);
       const int mDeltaI = binomial<R>(s, mEP, th[4]);
