@@ -112,6 +112,8 @@ struct MathTab {
   unsigned long long inv_f_q62[192];        // round((128 / j) 2^62), j = 90..181 used
   unsigned long long exp2_neg64_q63[64];    // round(2^(-j/64) 2^63)
   unsigned long long exp2_neg4096_q63[64];  // round(2^(-j/4096) 2^63)
+  long long log_f_q64[192];  // round(log(j/128) 2^64), j = 90..181 used
+  longlong2 cos_sin_q62[65];  // round(cos, sin of (2 pi j / 512) 2^62)
   double lfact[32];                      // log k!, k < 32 (sums of logs in order)
   double exp2_j[32];    // 2^(j/32)
   double inv_int[256];  // 1 / k (entry 0 unused)
@@ -160,6 +162,16 @@ __device__ __forceinline__ double tang_log(double x, const MathTab* __restrict__
   return tang_log_tail(u, j, e, T);
 }
 
+// q(v) of log1p(v) = v - v^2 q(v) in 2^-62 fixed point, from v 2^64 (|v| < 2^-7.49)
+// and v^2 2^64: q = 1/2 - v/3 + v^2 (1/4 - v/5 + v^2 (1/6 - v/7 + v^2/8)).
+__device__ __forceinline__ long long log1p_q62(long long v64, long long v2) {
+  constexpr long long k2 = 1ll << 61, k3 = 0x1555555555555555ll, k4 = 1ll << 60;
+  constexpr long long k5 = 0x0CCCCCCCCCCCCCCDll, k6 = 0x0AAAAAAAAAAAAAABll, k7 = 0x0924924924924925ll;
+  const long long c = k6 - __mul64hi(v64, k7) + (v2 >> 5);  // 1/6 - v/7 + v^2/8
+  const long long b = k4 - __mul64hi(v64, k5) + __mul64hi(v2, c);
+  return k2 - __mul64hi(v64, k3) + __mul64hi(v2, b);
+}
+
 // log u for the FP64 uniform u = ((x >> 11) | 1) 2^-53 of 64 random bits x,
 // with tang_log's reduction done on the integer pipes: the significand
 // n = (x >> 11) | 1 gives the exponent (leading-zero count), the halving test,
@@ -196,12 +208,7 @@ __device__ __forceinline__ double log_unif53(unsigned long long x, const MathTab
   const long long vm = (long long)__umul64hi(ad << sh, __ldg(&T->inv_f_q62[j]));
   const long long v64 = diff < 0 ? -vm : vm;
   const long long v2 = __mul64hi(v64, v64);  // v^2 2^64
-  // coefficients in 2^-62 fixed point
-  constexpr long long k2 = 1ll << 61, k3 = 0x1555555555555555ll, k4 = 1ll << 60;
-  constexpr long long k5 = 0x0CCCCCCCCCCCCCCDll, k6 = 0x0AAAAAAAAAAAAAABll, k7 = 0x0924924924924925ll;
-  const long long c = k6 - __mul64hi(v64, k7) + (v2 >> 5);  // 1/6 - v/7 + v^2/8
-  const long long b = k4 - __mul64hi(v64, k5) + __mul64hi(v2, c);
-  const long long q = k2 - __mul64hi(v64, k3) + __mul64hi(v2, b);  // in (0.497, 0.503) 2^62
+  const long long q = log1p_q62(v64, v2);  // in (0.497, 0.503) 2^62
   const double qd = __longlong_as_double(__double_as_longlong(__ll2double_rn(q)) - (62ll << 52));
   const double pl = fma(-(v * v), qd, v);
   const double de = (double)e;
@@ -729,11 +736,116 @@ __device__ __forceinline__ float log_first_uniform(const Block4& b, const Stream
 }
 
 template <typename R>
-__device__ __forceinline__ R normal01(Stream& s) {
+__device__ __forceinline__ R normal01(Stream& s);
+template <>
+__device__ __forceinline__ float normal01<float>(Stream& s) {
   const Block4 b = s.next();
-  const R u2 = Unif<R>::second(b);
-  const R rad = m_sqrt((R)-2.0 * log_first_uniform(b, s, (R)0));
+  const float u2 = Unif<float>::second(b);
+  const float rad = m_sqrt(-2.0f * log_first_uniform(b, s, 0.0f));
   return rad * cos_2pi(u2);
+}
+
+// The FP64 normal on the integer pipes.  In FP64 (the form above with the
+// library's sqrt and cos) it takes about 60 operations of 16 issue cycles a warp
+// and a dependent chain of 40 of 64 cycles each.  Here, in 64-bit fixed point:
+//   L = -ln u1 by log_unif53's reduction, in units of 2^-64, 2^-60 or 2^-57 by size;
+//   R = sqrt(2 L 2^..) in [1/2, 1): a single-precision reciprocal root and two
+//     Newton corrections (errors 2^-22, 2^-43, then 2^-63);
+//   cos(2 pi u2): the quadrant from the top bits of u2 (exact), a table of cosine
+//     and sine at multiples of 2 pi / 512, and both series of the remainder
+//     (|phi| < 2^-7.3) to phi^6;
+// and one conversion of the product.  Within 0.13 2^-53 of the exact value below
+// 8 (0.05 typically below 2; the FP64 form rounds 2 pi u2 first, up to 3.5 2^-53
+// from it).  u1 within 2^-12 of 1, where L has few bits in these units, takes the
+// FP64 form.
+__device__ __noinline__ inline double normal_f64(Block4 b, const MathTab* T) {
+  const double rad = sqrt(-2.0 * log_unif53(((unsigned long long)b.w1 << 32) | b.w0, T));
+  return rad * cos_2pi(Unif<double>::second(b));
+}
+
+__device__ __noinline__ inline double normal_of(Block4 b, const MathTab* __restrict__ T) {
+  // L = E ln 2 - log F - log1p(v), as in log_unif53
+  const unsigned long long n = ((((unsigned long long)b.w1 << 32) | b.w0) >> 11) | 1ull;
+  const int p = 63 - __clzll((long long)n);
+  const unsigned long long mb = n << (52 - p);
+  int E = 53 - p, j, sh;
+  long long diff;
+  if (mb >= 0x16A09E667F3BCDull) {
+    E -= 1;
+    j = (int)((mb + (1ull << 45)) >> 46);
+    diff = (long long)mb - ((long long)j << 46);
+    sh = 13;
+  } else {
+    j = (int)((mb + (1ull << 44)) >> 45);
+    diff = (long long)mb - ((long long)j << 45);
+    sh = 14;
+  }
+  const unsigned long long ad = (unsigned long long)(diff < 0 ? -diff : diff);
+  const long long vm = (long long)__umul64hi(ad << sh, __ldg(&T->inv_f_q62[j]));
+  const long long v = diff < 0 ? -vm : vm;  // 2^64
+  const long long v2 = __mul64hi(v, v);
+  const long long t = __ldg(&T->log_f_q64[j]) + v - __mul64hi(v2 << 2, log1p_q62(v, v2));
+  unsigned long long L;
+  int u;  // L in units of 2^(u - 64)
+  if (E == 0) {
+    L = (unsigned long long)-t;
+    u = 0;
+    if (L < (1ull << 52)) return normal_f64(b, T);
+  } else if (E <= 10) {
+    L = (unsigned long long)(E * 0x0B17217F7D1CF79Bll - (t >> 4));  // ln 2 2^60
+    u = 4;
+  } else {
+    L = (unsigned long long)(E * 0x0162E42FEFA39EF3ll - (t >> 7));  // ln 2 2^57
+    u = 7;
+  }
+  // sqrt(2 L) = R 2^h with Y = L 2^c in [2^62, 2^64), c of the parity that makes
+  // the exponent even (L < 2^63, so c >= 0), R = sqrt(Y 2^-64)
+  int c = __clzll((long long)L);
+  c -= (u - 63 - c) & 1;
+  const unsigned long long Y = L << c;
+  const float yf = (float)(unsigned)(Y >> 40) * 0x1p-24f;
+  const float rf = rsqrtf(yf), half = 0.5f * rf;
+  const unsigned g = __float2uint_rz(fminf(yf * rf, 0x1.fffffep-1f) * 0x1p32f);
+  const long long d = (long long)(Y - (unsigned long long)g * g);  // |d| < 2^44
+  const int h1 = __float2int_rz((float)(int)(d >> 14) * half);
+  const unsigned long long G1 =
+      ((unsigned long long)g << 32) + (unsigned long long)((long long)h1 << 14);
+  const int d1 = (int)(long long)(Y - __umul64hi(G1, G1));
+  const unsigned long long G = G1 + (unsigned long long)(long long)__float2int_rz((float)d1 * half);
+  // cos(2 pi u2): 4 u2 = q + 4 t, then t = +-(j / 512 + r)
+  const unsigned long long A = (((((unsigned long long)b.w3 << 32) | b.w2) >> 11) | 1ull) << 11;
+  const unsigned q = (unsigned)((A + (1ull << 61)) >> 62) & 3u;
+  const long long tt = (long long)(A << 2) >> 2;  // A modulo 2^62, in [-2^61, 2^61)
+  const unsigned long long at = (unsigned long long)(tt < 0 ? -tt : tt);
+  const int jj = (int)((at + (1ull << 54)) >> 55);
+  const long long r = (long long)(at - ((unsigned long long)jj << 55));
+  const long long ph = __mul64hi(r << 4, 0x6487ED5110B4611Aull);  // 2 pi 2^60
+  const unsigned long long p2 = (unsigned long long)__mul64hi(ph, ph);  // below 2^50
+  const unsigned p32 = (unsigned)(p2 >> 18);
+  const unsigned long long c1 =
+      0x2AAAAAAAAAAAAAABull - ((unsigned long long)__umulhi(p32, 0x88888888u) << 12);  // 1/6 - p/120
+  const long long sn = ph - __mul64hi(ph, (long long)__umul64hi(p2, c1));             // sin phi
+  const unsigned long long c2 =
+      0x0AAAAAAAAAAAAAABull - ((unsigned long long)__umulhi(p32, 1527099483u) << 10);  // 1/24 - p/720
+  const long long C1 =
+      (long long)__umul64hi(p2, 0x8000000000000000ull - __umul64hi(p2, c2));  // 1 - cos phi
+  const longlong2 cs = __ldg(&T->cos_sin_q62[jj]);
+  const bool odd = (q & 1u) != 0;
+  const long long ca = odd ? cs.y : cs.x, cb = odd ? cs.x : -cs.y;
+  const long long val = ca - __mul64hi(ca, C1) + __mul64hi(cb, sn);  // 2^62, of |t|
+  // cos, -sin, -cos, sin by quadrant, the sines odd in t
+  const bool neg = (q == 2u) != ((q == 1u && tt >= 0) || (q == 3u && tt < 0)) != (val < 0);
+  const unsigned long long av = (unsigned long long)(val < 0 ? -val : val);
+  const unsigned long long P = __umul64hi(G, av << 1);  // R |cos| 2^63
+  if (P == 0) return 0.0;
+  const int h = ((u - 63 - c) >> 1) + 32 - 63;
+  const long long z = __double_as_longlong(__ull2double_rn(P)) + ((long long)h << 52);
+  return __longlong_as_double(neg ? z | (long long)0x8000000000000000ull : z);
+}
+
+template <>
+__device__ __forceinline__ double normal01<double>(Stream& s) {
+  return normal_of(s.next(), s.tab);
 }
 
 // -ln u of the next uniform (FP64: straight from its random bits)

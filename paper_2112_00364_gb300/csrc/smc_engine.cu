@@ -174,6 +174,7 @@ smc_status math_table(const MathTab** out) {
     MathTab h;
     for (int j = 0; j < 192; ++j) {
       h.inv_f_q62[j] = j >= 90 ? (unsigned long long)std::llroundl(std::ldexp(128.0L / j, 62)) : 0ull;
+      h.log_f_q64[j] = j >= 90 ? std::llroundl(std::ldexp(std::log(j / 128.0L), 64)) : 0ll;
       h.log_f[j] = j ? std::log((double)j / 128.0) : 0.0;
       h.inv_f[j] = j ? 128.0 / (double)j : 0.0;
       h.inv_f52[j] = std::ldexp(h.inv_f[j], -52);
@@ -185,6 +186,11 @@ smc_status math_table(const MathTab** out) {
       if (j == 0) return 1ull << 63;
       return (unsigned long long)std::llroundl(std::ldexp(std::exp2l(-(long double)j / m), 63));
     };
+    for (int j = 0; j <= 64; ++j) {
+      const long double th = 6.283185307179586476925286766559L * j / 512.0L;
+      h.cos_sin_q62[j].x = std::llroundl(std::ldexp(std::cos(th), 62));
+      h.cos_sin_q62[j].y = std::llroundl(std::ldexp(std::sin(th), 62));
+    }
     // e^-(j/m) 2^63 rounded; j = 0 is 2^63 itself
     auto e63 = [](int j, int m) -> unsigned long long {
       if (j == 0) return 1ull << 63;
@@ -440,13 +446,14 @@ cudaError_t ChainStreams::join(cudaStream_t main, int chains) {
 namespace {
 cudaError_t launch_chain(const WavePlan& W, const WaveChain& c, int precision, cudaStream_t st,
                          unsigned wave) {
+  const bool alone = W.chains.size() == 1;
   switch (c.kind) {
-    case SMC_MODEL_LG: return launch_kind<SMC_MODEL_LG>(c, W.runs, precision, st, wave);
-    case SMC_MODEL_CRBD: return launch_kind<SMC_MODEL_CRBD>(c, W.runs, precision, st, wave);
-    case SMC_MODEL_RATESHIFT: return launch_kind<SMC_MODEL_RATESHIFT>(c, W.runs, precision, st, wave);
-    case SMC_MODEL_SEIR: return launch_kind<SMC_MODEL_SEIR>(c, W.runs, precision, st, wave);
-    case SMC_MODEL_CRBD_DS: return launch_kind<SMC_MODEL_CRBD_DS>(c, W.runs, precision, st, wave);
-    default: return launch_kind<SMC_MODEL_GEOMETRIC>(c, W.runs, precision, st, wave);
+    case SMC_MODEL_LG: return launch_kind<SMC_MODEL_LG>(c, W.runs, precision, st, wave, alone);
+    case SMC_MODEL_CRBD: return launch_kind<SMC_MODEL_CRBD>(c, W.runs, precision, st, wave, alone);
+    case SMC_MODEL_RATESHIFT: return launch_kind<SMC_MODEL_RATESHIFT>(c, W.runs, precision, st, wave, alone);
+    case SMC_MODEL_SEIR: return launch_kind<SMC_MODEL_SEIR>(c, W.runs, precision, st, wave, alone);
+    case SMC_MODEL_CRBD_DS: return launch_kind<SMC_MODEL_CRBD_DS>(c, W.runs, precision, st, wave, alone);
+    default: return launch_kind<SMC_MODEL_GEOMETRIC>(c, W.runs, precision, st, wave, alone);
   }
 }
 }  // namespace
@@ -887,6 +894,7 @@ extern "C" smc_status smc_model_register(const smc_model_desc* d, smc_model_t* o
   }
   m->n_segments_known = 0;
   if (d->kind == SMC_MODEL_LG) {
+    md.inv_r_sd = d->r_sd > 0x1p-100 && d->r_sd < 0x1p100 ? 1.0 / d->r_sd : 0.0;
     md.lg_lc = std::log(d->r_sd) + 0.91893853320467274178;
     m->n_segments_known = d->T;
   }

@@ -6,6 +6,9 @@
 //                  cross checkpoints plus segment-local scratch);
 //   init/gather/store  PSTATE <-> registers (gather = Section 3.3's particle
 //                  duplication, reading the ancestor's slot of the SoA arrays);
+//   PREDRAW, predraw  (optional) a draw of segment k > 0 that depends on its counter
+//                  alone, taken into the lane before the segment's inputs are there
+//                  (while the checkpoint before it is still being reached);
 //   block(b, ...)  one basic block; sets pc to the successor and `ckpt` when
 //                  the block ends in a checkpoint (Algorithm 1's c_n).
 // Block index PC_STOP (-1) is b_stop: sim(b_stop, s) = (b_stop, s, true).
@@ -45,7 +48,7 @@ struct ModelDev {
   const int* preorder;
   const double* age;
   const double* fixed_mult;
-  double x0_mean, x0_sd, a, b, q_sd, r_sd, lg_lc, corr;
+  double x0_mean, x0_sd, a, b, q_sd, r_sd, inv_r_sd, lg_lc, corr;
   double rho, lambda_fixed, mu_fixed, lambda_scale, mu_scale, sigma, geo_p, geo_logw;
 };
 
@@ -93,13 +96,20 @@ template <typename Real>
 struct LgModel {
   using R = Real;
   static constexpr int NB = 2, N_REAL = 1, N_INT = 1;
-  static constexpr bool HAS_STACK = false;
+  static constexpr bool HAS_STACK = false, PREDRAW = true;
   struct Lane {
     int pc;
     bool ckpt;
     R x, logw;
+    R z;  // the predrawn normal of a segment k > 0, when drawn
+    bool drawn;
     int overflow, limited;
   };
+  // every particle of a segment k > 0 runs block 1, whose one draw is its first
+  __device__ static void predraw(Lane& L, Stream& s) {
+    L.z = normal01<R>(s);
+    L.drawn = true;
+  }
   __device__ static void init(Lane& L) {
     L.pc = 0;
     L.x = (R)0;
@@ -125,6 +135,14 @@ struct LgModel {
     L.ckpt = false;
     L.overflow = L.limited = 0;
   }
+  // x / r_sd; FP64 by the reciprocal and one correction (3 operations, not 12),
+  // where neither can overflow or lose bits (inv_r_sd is 0 for an extreme r_sd)
+  __device__ static double over_r_sd(double x, const ModelDev& md) {
+    const unsigned ex = (unsigned)((unsigned long long)__double_as_longlong(x) >> 52) & 0x7ffu;
+    if (md.inv_r_sd == 0.0 || ex > 1023u + 900u) return x / md.r_sd;
+    return div_by(x, md.r_sd, md.inv_r_sd);
+  }
+  __device__ static float over_r_sd(float x, const ModelDev& md) { return x / (float)md.r_sd; }
   __device__ static void block(int b, Lane& L, Stream& s, const ModelDev& md, const StateView&, int,
                                int k, int) {
     if (b == 0) {
@@ -133,10 +151,10 @@ struct LgModel {
       L.pc = 1;
       return;
     }
-    const R z = normal01<R>(s);
+    const R z = L.drawn ? L.z : normal01<R>(s);
     L.x = m_fma((R)md.a, L.x, m_fma((R)md.q_sd, z, (R)md.b));
     const R y = (R)md.obs[k];
-    const R dz = (y - L.x) / (R)md.r_sd;
+    const R dz = over_r_sd(y - L.x, md);
     const R lp = (R)-0.5 * (dz * dz) - (R)md.lg_lc;
     L.logw = L.logw + lp;
     L.pc = (k + 1 == md.T) ? PC_STOP : 1;
@@ -154,7 +172,7 @@ template <typename Real>
 struct GeoModel {
   using R = Real;
   static constexpr int NB = 1, N_REAL = 0, N_INT = 2;
-  static constexpr bool HAS_STACK = false;
+  static constexpr bool HAS_STACK = false, PREDRAW = false;
   struct Lane {
     int pc, count;
     bool ckpt;
@@ -219,7 +237,7 @@ template <typename Real>
 struct SeirModel {
   using R = Real;
   static constexpr int NB = 2, N_REAL = 6, N_INT = 10;
-  static constexpr bool HAS_STACK = false;
+  static constexpr bool HAS_STACK = false, PREDRAW = false;
   struct Lane {
     int pc;
     bool ckpt;
@@ -436,7 +454,7 @@ struct TreeModel {
   // CRBD keeps log(lambda) as a third, internal real field (computed once at the
   // prior block instead of once per internal-node branch); it is not an output.
   static constexpr int NB = 4, N_REAL = 2, N_INT = RS ? 2 : 1;
-  static constexpr bool HAS_STACK = RS;
+  static constexpr bool HAS_STACK = RS, PREDRAW = false;
   enum { PRIOR = 0, BRANCH = 1, HIDDEN = 2, END = 3 };
   struct Lane {
     int pc, sp, v, n_top, fsp, calls;
@@ -603,7 +621,7 @@ template <typename Real>
 struct TreeDsModel {
   using R = Real;
   static constexpr int NB = 4, N_REAL = 4, N_INT = 1;
-  static constexpr bool HAS_STACK = false;
+  static constexpr bool HAS_STACK = false, PREDRAW = false;
   enum { PRIOR = 0, BRANCH = 1, HIDDEN = 2, END = 3 };
   struct Lane {
     int pc, v, n_top, fsp, calls;

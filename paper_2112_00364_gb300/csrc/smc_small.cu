@@ -190,30 +190,35 @@ __device__ __forceinline__ Combined combine_warp(const TileRec* rec, int nt, con
   return c;
 }
 
-// CL: launched as one cluster of ceil(n_tiles / (TPB / 32)) CTAs (else one CTA).
+// CL: launched as one cluster of ceil(n_tiles / (TPB / 32)) CTAs (else one CTA),
+// each with one warp more than its tiles: that of rank 0 closes the segments (log
+// Z, its records), off every tile's path.
 template <class M, int TPB, bool CL>
-__global__ void __launch_bounds__(TPB, 1) small_run_kernel(const RunDev* __restrict__ runs) {
+__global__ void __launch_bounds__(TPB + (CL ? 32 : 0), 1) small_run_kernel(const RunDev* __restrict__ runs) {
   using R = typename M::R;
   constexpr int WPC = TPB / 32;
   static_assert(CL || WPC >= 16, "one CTA holds the whole run");
   __shared__ __align__(16) RunDev sr;
-  __shared__ long long sh_O[WPC][kSmallMaxTiles + 1];  // each warp's own offsets
-  __shared__ int sh_ks[WPC][kSmallMaxTiles + 1];
+  constexpr int NT = TPB + (CL ? 32 : 0);
+  __shared__ long long sh_O[NT / 32][kSmallMaxTiles + 1];  // each warp's own offsets
+  __shared__ int sh_ks[NT / 32][kSmallMaxTiles + 1];
   {
     const int* src = reinterpret_cast<const int*>(runs);
     int* dst = reinterpret_cast<int*>(&sr);
-    for (int w = threadIdx.x; w < (int)(sizeof(RunDev) / 4); w += TPB) dst[w] = src[w];
+    for (int w = threadIdx.x; w < (int)(sizeof(RunDev) / 4); w += NT) dst[w] = src[w];
   }
   __syncthreads();
   const RunDev& A = sr;
   RunState* rs = A.rs;
   const int N = A.N;
-  const bool lead = !CL || cluster_rank() == 0;  // the CTA that closes each segment
   const int wid = (int)(threadIdx.x >> 5);
+  const bool extra = CL && wid == WPC;  // the warp without a tile
+  // the thread that closes each segment
+  const bool closes = CL ? extra && cluster_rank() == 0 && (threadIdx.x & 31) == 0 : threadIdx.x == 0;
   const int t = (CL ? (int)cluster_rank() * WPC : 0) + wid;
   const int lane = threadIdx.x & 31;
   const int i = t * 32 + lane;  // the tile of this path is 32 particles
-  const bool tile_live = t < A.n_tiles;
+  const bool tile_live = !extra && t < A.n_tiles;
   const bool valid = tile_live && i < N;
   // segment k - 1's closing (log Z, its records) waits for the barrier that
   // ends segment k, where it overlaps the other CTAs' arrival
@@ -222,11 +227,18 @@ __global__ void __launch_bounds__(TPB, 1) small_run_kernel(const RunDev* __restr
   unsigned long long uf = 0;  // the uniform of the next search, drawn in the barrier's shadow
   // the run's counters, summed per lane over the segments and added once
   unsigned long long n_near = 0, n_overflow = 0, n_limit = 0, n_draws = 0, n_blocks = 0;
+  typename M::Lane Ln;  // (what predraw() fills, for the next segment)
   for (int k = 0;; ++k) {
     const int nb = k & 1, cb = nb ^ 1;
     const StateView Sc = A.state[cb];
     const StateView Sn = A.state[nb];
     typename M::Lane L;
+    Stream s{A.k0, A.k1, (uint32_t)i, (uint32_t)k, 0u, 0u, A.md.tab};
+    if constexpr (M::PREDRAW) {
+      L.z = Ln.z;
+      L.drawn = k > 0;
+      s.d = k > 0 ? 1 : 0;
+    }
     bool near = false;
     if (k > 0) {
       const Combined c = combine_warp(A.rec[cb], A.n_tiles, A.ess ? A.tq[cb] : nullptr,
@@ -234,7 +246,7 @@ __global__ void __launch_bounds__(TPB, 1) small_run_kernel(const RunDev* __restr
       const bool go_on = c.kmax != kDeadTile && c.alive && k < A.max_segments;
       const bool resample = decide_resample(A, c);
       if (!go_on) {  // the same c in every thread: a uniform exit
-        if (lead && threadIdx.x == 0) finish_segment(A, k, c, resample);
+        if (closes) finish_segment(A, k, c, resample);
         break;
       }
       c_close = c;
@@ -302,7 +314,6 @@ __global__ void __launch_bounds__(TPB, 1) small_run_kernel(const RunDev* __restr
       L.pc = PC_STOP;
       L.logw = neg_inf<R>();
     }
-    Stream s{A.k0, A.k1, (uint32_t)i, (uint32_t)k, 0u, 0u, A.md.tab};
     const bool active = valid && L.pc != PC_STOP;
     const int n_exec = run_segment<M>(L, s, A.md, Sn, i, k, N, active);
     double lw = -INFINITY;
@@ -348,7 +359,13 @@ __global__ void __launch_bounds__(TPB, 1) small_run_kernel(const RunDev* __restr
     }
     // the segment's records, running sums and states, for the next combine
     if (CL) cluster_arrive();
-    if (k > 0 && lead && threadIdx.x == 0) finish_segment(A, k, c_close, resample_close);
+    if (k > 0 && closes) finish_segment(A, k, c_close, resample_close);
+    if constexpr (M::PREDRAW) {
+      if (valid) {
+        Stream sn{A.k0, A.k1, (uint32_t)i, (uint32_t)(k + 1), 0u, 0u, A.md.tab};
+        M::predraw(Ln, sn);
+      }
+    }
     if (lane == 0) uf = search_uniform(A, k);
     if (CL)
       cluster_wait();
@@ -389,7 +406,7 @@ cudaError_t launch_cluster(const RunDev* runs, int n_tiles, cudaStream_t st) {
   const unsigned ctas = (unsigned)((n_tiles + TPB / 32 - 1) / (TPB / 32));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ctas, 1, 1);
-  cfg.blockDim = dim3(TPB, 1, 1);
+  cfg.blockDim = dim3(TPB + 32, 1, 1);
   cfg.dynamicSmemBytes = 0;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
@@ -415,7 +432,7 @@ bool wide_clusters() {
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(16, 1, 1);
-    cfg.blockDim = dim3(64, 1, 1);
+    cfg.blockDim = dim3(96, 1, 1);
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 16;

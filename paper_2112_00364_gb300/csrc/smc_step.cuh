@@ -349,7 +349,8 @@ struct PublishRun {
 // One tile of one run for segment k (the whole per-CTA body of a wave).
 template <class M, int TPB>
 __device__ __forceinline__ void step_tile(const RunDev& A, const int t, const int k,
-                                          StepShared<TPB>& S) {
+                                          StepShared<TPB>& S, typename M::Lane& L, Stream& s,
+                                          const bool early) {
   using R = typename M::R;
   RunState* rs = A.rs;
   const int N = A.N;
@@ -362,9 +363,7 @@ __device__ __forceinline__ void step_tile(const RunDev& A, const int t, const in
   const bool redundant = A.redundant != 0;
   // resuming a snapshot: segment resume_k - 1 loads the population instead of running it
   const bool load = A.resume_k > 0 && k == A.resume_k - 1;
-  typename M::Lane L;
   bool near = false;
-  Stream s{A.k0, A.k1, (uint32_t)i, (uint32_t)k, 0u, 0u, A.md.tab};
   if (load) {
     if (valid) M::load(L, Sn, SnapView{A.snap_logw, A.snap_real, A.snap_int, A.snap_stack}, i, N, s);
   } else if (k > 0) {
@@ -498,7 +497,7 @@ __device__ __forceinline__ void step_tile(const RunDev& A, const int t, const in
   // start is not hidden.  At the CTA's start / here / at its end: batch of 512
   // 142.9 / 140.3 / 139.9 ms, CRBD 64k 24.2 / 24.0 / 24.5 us a wave, delayed
   // sampling 68.6 / 67.9 / 66.8, linear-Gaussian 23k 9.71 / 9.76 / 9.95.
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (!early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   alive = __syncthreads_or(alive);
   int kt = S.kw[0];
 #pragma unroll
@@ -567,6 +566,8 @@ __device__ __forceinline__ void step_tile(const RunDev& A, const int t, const in
   }
 }
 
+constexpr unsigned kEarlyCtas = 152;  // GB300's SMs
+
 // The block table of a model kind.
 template <int KIND, typename R>
 struct ModelOf;
@@ -590,7 +591,8 @@ struct ModelOf<SMC_MODEL_CRBD_DS, R> { using type = TreeDsModel<R>; };
 // KIND: the model (SMC_MODEL_*) that every run of the launch runs.
 template <typename R, int TPB, int KIND>
 __global__ void __launch_bounds__(TPB, (sizeof(R) == 4 ? 1024 : 768) / TPB) wave_kernel(const RunDev* __restrict__ runs,
-                                                   const int2* __restrict__ cta_map, unsigned wave) {
+                                                   const int2* __restrict__ cta_map, unsigned wave,
+                                                   int alone) {
   __shared__ __align__(16) RunDev sr;
   __shared__ StepShared<TPB> S;
   const int2 rt = cta_map[blockIdx.x];
@@ -604,20 +606,36 @@ __global__ void __launch_bounds__(TPB, (sizeof(R) == 4 ? 1024 : 768) / TPB) wave
   // start (and copy their run table, which no kernel writes) while the last CTAs
   // of the previous one still run; everything below reads what that wave wrote, so
   // it waits for its completion first.
+  // (a lone chain's grid of at most one CTA an SM leaves room for the next wave's
+  // CTAs beside its own: those then start at once, and what they do before the wait
+  // is hidden.  Beside other chains they would take places from them)
+  const bool early = alone && gridDim.x <= kEarlyCtas;
+  if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int k = (int)(wave - sr.start_wave);  // wraps correctly past 2^32 waves
+  using M = typename ModelOf<KIND, R>::type;
+  typename M::Lane L;
+  Stream s{sr.k0, sr.k1, (uint32_t)(rt.y * sr.tile + threadIdx.x), (uint32_t)k, 0u, 0u, sr.md.tab};
+  if constexpr (M::PREDRAW) {
+    // (not for a segment that loads a snapshot.  In larger grids most CTAs start
+    // after the wave before them has ended: nothing to hide the draw behind, and
+    // drawing there took a wave of 2^20 FP32 particles from 78 to 89 us)
+    L.drawn = false;
+    if (early && k > 0 && (int)threadIdx.x < sr.tile && k != sr.resume_k - 1) M::predraw(L, s);
+  }
   // the uniform of the search whose scalars this CTA may form, from the counter
   // alone: in the wait's shadow
   if (threadIdx.x == 0) S.uf = search_uniform(sr, sr.redundant ? k - 1 : k);
   asm volatile("griddepcontrol.wait;" ::: "memory");
   RunState* rs = sr.rs;
   if (*(volatile int32_t*)&rs->done || k < 0) return;
-  step_tile<typename ModelOf<KIND, R>::type, TPB>(sr, rt.y, k, S);
+  step_tile<M, TPB>(sr, rt.y, k, S, L, s, early);
 }
 
 // One bucket of a wave, launched so that it may begin before the kernel ahead
 // of it in the stream has finished (wave_kernel waits for it where it must).
 template <typename R, int TPB, int KIND>
-cudaError_t launch_pdl(const RunDev* runs, const int2* map, int n, cudaStream_t st, unsigned wave) {
+cudaError_t launch_pdl(const RunDev* runs, const int2* map, int n, cudaStream_t st, unsigned wave,
+                       bool alone) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)n);
   cfg.blockDim = dim3(TPB);
@@ -628,17 +646,17 @@ cudaError_t launch_pdl(const RunDev* runs, const int2* map, int n, cudaStream_t 
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, wave_kernel<R, TPB, KIND>, runs, map, wave);
+  return cudaLaunchKernelEx(&cfg, wave_kernel<R, TPB, KIND>, runs, map, wave, alone ? 1 : 0);
 }
 
 template <typename R, int KIND>
 cudaError_t launch_bucket(int b, const RunDev* runs, const int2* map, int n, cudaStream_t st,
-                          unsigned wave) {
+                          unsigned wave, bool alone) {
   switch (b) {
-    case 0: return launch_pdl<R, 32, KIND>(runs, map, n, st, wave);
-    case 1: return launch_pdl<R, 64, KIND>(runs, map, n, st, wave);
-    case 2: return launch_pdl<R, 128, KIND>(runs, map, n, st, wave);
-    default: return launch_pdl<R, 256, KIND>(runs, map, n, st, wave);
+    case 0: return launch_pdl<R, 32, KIND>(runs, map, n, st, wave, alone);
+    case 1: return launch_pdl<R, 64, KIND>(runs, map, n, st, wave, alone);
+    case 2: return launch_pdl<R, 128, KIND>(runs, map, n, st, wave, alone);
+    default: return launch_pdl<R, 256, KIND>(runs, map, n, st, wave, alone);
   }
 }
 

@@ -14,10 +14,10 @@ namespace smc {
 
 template <int KIND>
 cudaError_t launch_kind(const WaveChain& c, const RunDev* runs, int precision, cudaStream_t st,
-                        unsigned wave) {
+                        unsigned wave, bool alone) {
   return precision == SMC_PREC_FP32
-             ? launch_bucket<float, KIND>(c.bucket, runs, c.map, c.n_ctas, st, wave)
-             : launch_bucket<double, KIND>(c.bucket, runs, c.map, c.n_ctas, st, wave);
+             ? launch_bucket<float, KIND>(c.bucket, runs, c.map, c.n_ctas, st, wave, alone)
+             : launch_bucket<double, KIND>(c.bucket, runs, c.map, c.n_ctas, st, wave, alone);
 }
 
 }  // namespace smc

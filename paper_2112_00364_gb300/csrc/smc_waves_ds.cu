@@ -3,6 +3,7 @@
 
 namespace smc {
 
-template cudaError_t launch_kind<SMC_MODEL_CRBD_DS>(const WaveChain&, const RunDev*, int, cudaStream_t, unsigned);
+template cudaError_t launch_kind<SMC_MODEL_CRBD_DS>(const WaveChain&, const RunDev*, int, cudaStream_t, unsigned,
+                                              bool);
 
 }  // namespace smc

@@ -3,7 +3,9 @@
 
 namespace smc {
 
-template cudaError_t launch_kind<SMC_MODEL_RATESHIFT>(const WaveChain&, const RunDev*, int, cudaStream_t, unsigned);
-template cudaError_t launch_kind<SMC_MODEL_GEOMETRIC>(const WaveChain&, const RunDev*, int, cudaStream_t, unsigned);
+template cudaError_t launch_kind<SMC_MODEL_RATESHIFT>(const WaveChain&, const RunDev*, int, cudaStream_t, unsigned,
+                                              bool);
+template cudaError_t launch_kind<SMC_MODEL_GEOMETRIC>(const WaveChain&, const RunDev*, int, cudaStream_t, unsigned,
+                                              bool);
 
 }  // namespace smc
