@@ -83,6 +83,41 @@ __device__ __forceinline__ void load_run(const double* __restrict__ x, int64_t N
   }
 }
 
+// floor(hi 2^64 / d) for hi < d, d >= 2^63: a quotient from the FP64 reciprocal (53
+// bits), then the remainder's quotient from it, then single steps.  (A 128-bit
+// division takes several times as long, in one thread while the others wait.)
+__device__ __forceinline__ unsigned long long div_128_64(unsigned long long hi,
+                                                         unsigned long long d) {
+  const double inv = 1.0 / (double)d;
+  const double q0 = (double)hi * inv * 18446744073709551616.0;
+  unsigned long long q = q0 >= 18446744073709551615.0 ? ~0ull : (unsigned long long)q0;
+  // r = hi 2^64 - q d: |r| below 2^13 d
+  const unsigned long long plo = q * d, phi = __umul64hi(q, d);
+  long long rh = (long long)(hi - phi - (plo != 0 ? 1ull : 0ull));
+  unsigned long long rl = 0ull - plo;
+  const long long dq = (long long)floor(((double)rh * 18446744073709551616.0 + (double)rl) * inv);
+  q += (unsigned long long)dq;
+  // r -= dq d
+  const unsigned long long tl = (unsigned long long)dq * d;
+  const long long th = (long long)__umul64hi((unsigned long long)dq, d) - (dq < 0 ? (long long)d : 0ll);
+  rh = rh - th - (rl < tl ? 1 : 0);
+  rl -= tl;
+#pragma unroll 1
+  for (int k = 0; k < 4 && rh < 0; ++k) {  // r < 0
+    q -= 1;
+    const unsigned long long n = rl + d;
+    rh += n < rl ? 1 : 0;
+    rl = n;
+  }
+#pragma unroll 1
+  for (int k = 0; k < 4 && (rh > 0 || rl >= d); ++k) {
+    q += 1;
+    rh -= rl < d ? 1 : 0;
+    rl -= d;
+  }
+  return q;
+}
+
 // The search scalars of a population, written by rs_combine.
 // Offsets are counted in fixed point with F = 63 - bitlen(N) fraction bits
 // (N 2^F < 2^63): Q = B N / S 2^F for a boundary B in run units.
@@ -95,6 +130,42 @@ struct RsScalars {
 
 // Weights as 2^-50 fixed-point integers: a tile of 4096 sums below 2^62.
 constexpr int kRsBits = 50;
+
+// N / S = rn 2^-(64+L) with rn in [2^63, 2^64): with S and N shifted to 64 bits (sb
+// and nb bits long), s' and n', N / S = n'/s' 2^(nb-sb); n' >= s' takes one bit less.
+__device__ __forceinline__ RsScalars rs_scalars(const Combined& c, int64_t N, double u) {
+  const unsigned long long Su = (unsigned long long)c.S;
+  const int sb = 64 - __clzll((long long)Su), nb = 64 - __clzll((long long)N);
+  const unsigned long long sn = Su << (64 - sb), nn = (unsigned long long)N << (64 - nb);
+  const bool ge = nn >= sn;
+  RsScalars s;
+  // n' >= s': floor(n' 2^63 / s') = floor((n' / 2) 2^64 / s') (n' is even: N < 2^31)
+  s.rn = div_128_64(ge ? nn >> 1 : nn, sn);
+  s.L = sb - nb - (ge ? 1 : 0);
+  s.F = 63 - nb;
+  s.uF = (long long)(frac64(u) >> (64 - s.F));
+  s.tolF = (long long)(kBoundaryEps * (double)N * pow2i(s.F));
+  s.kmax = c.kmax;
+  s.G = c.G;
+  s.degenerate = 0;
+  s.pad_ = 0;
+  return s;
+}
+
+// out3 = {m, S, log-Z increment} of a combined population (one thread)
+__device__ __forceinline__ void rs_out3(const Combined& c, double log_n, const MathTab* tab,
+                                        double* out3) {
+  if (c.kmax == kDeadTile) {
+    out3[0] = -INFINITY;
+    out3[1] = 0.0;
+    out3[2] = -INFINITY;
+    return;
+  }
+  const double Sd = (double)c.S;
+  out3[0] = (double)c.kmax * kLn2;
+  out3[1] = Sd * pow2i(c.G - kRsBits);
+  out3[2] = (double)(c.kmax - kRsBits + c.G) * kLn2 + (tang_log(Sd, tab) - log_n);
+}
 
 // ---- the weight round(e^(x - k_t ln 2) 2^50) on the integer pipes ----
 // The argument X = k_t ln 2 - x >= 0 in units of 2^-52: K52 = k_t ln 2 2^52
@@ -299,19 +370,29 @@ __device__ __forceinline__ void reduce_tile(const double (&v)[RS1_IT], double (&
 // only after that kernel has completed.
 __global__ void __launch_bounds__(RS1_TPB, 2)
     rs_tile_reduce(const double* __restrict__ x, int64_t N, int nt, TileRec* __restrict__ rec,
-                   unsigned* __restrict__ ehi, long long* __restrict__ pref, const MathTab* tab) {
+                   unsigned* __restrict__ ehi, long long* __restrict__ pref,
+                   unsigned long long* n_near, const MathTab* tab) {
   extern __shared__ __align__(16) unsigned long long rs_T[];
   __shared__ int sh_key[2][RS1_WARPS];
   __shared__ long long sh_sum[2][RS1_WARPS];
+  int t = blockIdx.x;
+  double v[RS1_IT];
+  // one tile a CTA: the log-weights' loads first, the table behind them
+  const bool one = nt <= (int)gridDim.x;
+  if (one) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    load_run<RS1_IT>(x, N, (int64_t)t * RS_TILE + threadIdx.x * RS1_IT, v);
+  }
   {
     const ulonglong2* src = reinterpret_cast<const ulonglong2*>(tab->rs_exp_q56);
     ulonglong2* dst = reinterpret_cast<ulonglong2*>(rs_T);
     for (int i = threadIdx.x; i < kRsExpPad / 2; i += RS1_TPB) dst[i] = src[i];
   }
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  int t = blockIdx.x;
-  double v[RS1_IT];
-  if (t < nt) load_run<RS1_IT>(x, N, (int64_t)t * RS_TILE + threadIdx.x * RS1_IT, v);
+  if (!one) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (t < nt) load_run<RS1_IT>(x, N, (int64_t)t * RS_TILE + threadIdx.x * RS1_IT, v);
+  }
+  if (n_near && t == 0 && threadIdx.x == 0) *n_near = 0;  // pass 3 adds to it
   __syncthreads();  // the table
   for (int p = 0; t < nt; t += gridDim.x, p ^= 1) {
     double vn[RS1_IT];
@@ -430,46 +511,16 @@ __global__ void __launch_bounds__(RS_COMBINE_TPB) rs_combine(const TileRec* __re
                          : combine_offsets<RS_COMBINE_TPB>(rec, nt, O, nullptr, sh, nullptr,
                                                            [](const Combined&) {});
   // the log-Z increment (thread 0) and the search scalars (thread 32) in parallel
+  if (threadIdx.x == 0) rs_out3(c, log_n, tab, out3);
+  if (threadIdx.x != 32) return;
   if (c.kmax == kDeadTile) {
-    if (threadIdx.x == 0) {
-      out3[0] = -INFINITY;
-      out3[1] = 0.0;
-      out3[2] = -INFINITY;
-      RsScalars s;
-      std::memset(&s, 0, sizeof(s));
-      s.degenerate = 1;
-      *sc = s;
-    }
+    RsScalars s;
+    std::memset(&s, 0, sizeof(s));
+    s.degenerate = 1;
+    *sc = s;
     return;
   }
-  if (threadIdx.x == 0) {
-    const double Sd = (double)c.S;
-    out3[0] = (double)c.kmax * kLn2;
-    out3[1] = Sd * pow2i(c.G - kRsBits);
-    out3[2] = (double)(c.kmax - kRsBits + c.G) * kLn2 + (tang_log(Sd, tab) - log_n);
-  }
-  if (threadIdx.x != 32) return;
-  RsScalars s;
-  std::memset(&s, 0, sizeof(s));
-  // N / S = rn 2^-(64+L) with rn in [2^63, 2^64): S in [2^61, 2^62] has sb = 62
-  // or 63 bits and N nb bits, so L = sb - nb puts N 2^(64+L) / S in (2^63, 2^65)
-  // (the numerator has 64 + sb <= 127 bits); one step down when it is >= 2^64.
-  const unsigned long long Su = (unsigned long long)c.S;
-  const int sb = 64 - __clzll((long long)Su), nb = 64 - __clzll((long long)N);
-  int L = sb - nb;
-  unsigned __int128 rn = ((unsigned __int128)N << (64 + L)) / Su;
-  if (rn >> 64) {
-    L -= 1;
-    rn = ((unsigned __int128)N << (64 + L)) / Su;
-  }
-  s.rn = (unsigned long long)rn;
-  s.L = L;
-  s.F = 63 - nb;
-  s.uF = (long long)(frac64(u) >> (64 - s.F));
-  s.tolF = (long long)(kBoundaryEps * (double)N * pow2i(s.F));
-  s.kmax = c.kmax;
-  s.G = c.G;
-  *sc = s;
+  *sc = rs_scalars(c, N, u);
 }
 
 // A tile's boundaries in offset units: Q_j = min(Q(O_t) + E_j 2^-sh N / S 2^F,
@@ -611,13 +662,35 @@ __device__ __noinline__ long long rs_exact_running_sum(const double* __restrict_
 // positions (64 bytes apart) fall in different bank groups.
 __device__ __forceinline__ int mark_slot(int k) { return k + ((k >> 5) << 2); }
 
-template <bool FAST>
+// COMB: every CTA combines the tile records itself (at most RS_COMB_TILES of them: no
+// more CTAs than run at once) instead of a launch of rs_combine between passes 1
+// and 3; CTA 0 writes out3.  A 100,003-particle call (25 tiles) is two launches then
+// instead of four with the zeroing of n_near, which pass 1 does.
+constexpr int RS_COMB_TILES = 456;
+struct RsComb {  // the shared memory of a CTA that combines
+  long long O[RS_COMB_TILES + 1];
+  double red[combine_scratch(RS_TPB)];
+  RsScalars sc;
+};
+struct RsPublish {
+  int64_t N;
+  double u, log_n;
+  RsComb* S;
+  double* out3;
+  const MathTab* tab;
+  __device__ __forceinline__ void operator()(const Combined& c) const {
+    if (threadIdx.x == 0) S->sc = rs_scalars(c, N, u);
+    if (threadIdx.x == 32 && blockIdx.x == 0) rs_out3(c, log_n, tab, out3);
+  }
+};
+
+template <bool FAST, bool COMB>
 __global__ void __launch_bounds__(RS_TPB, 3) rs_ancestors(
     const double* __restrict__ x, int64_t n_local, int t0, int64_t N,
-    const TileRec* __restrict__ rec, const long long* __restrict__ O,
+    const TileRec* __restrict__ rec, const long long* __restrict__ Og,
     const RsScalars* __restrict__ scp, const unsigned* __restrict__ ehi,
     const long long* __restrict__ pref, int32_t* __restrict__ anc, unsigned long long* n_near,
-    int64_t* range, const MathTab* tab) {
+    int64_t* range, double u, double log_n, double* out3, const MathTab* tab) {
   __shared__ long long sh[RS_TPB / 32 + 1];
   __shared__ int sh_last[RS_TPB + 1];
   __shared__ int sh_wmax[RS_TPB / 32];
@@ -628,7 +701,23 @@ __global__ void __launch_bounds__(RS_TPB, 3) rs_ancestors(
   const int64_t lbase = (int64_t)tl * RS_TILE, base = (int64_t)t * RS_TILE;
   const int64_t lj0 = lbase + (int64_t)threadIdx.x * RS_IT;
   const int64_t j0 = base + (int64_t)threadIdx.x * RS_IT;
-  const RsScalars sc = *scp;
+  const long long* O = Og;
+  RsScalars sc;
+  if constexpr (COMB) {
+    __shared__ RsComb S;
+    const int nt = (int)gridDim.x;
+    const Combined c = combine_offsets<RS_TPB>(rec, nt, S.O, nullptr, S.red, nullptr,
+                                               RsPublish{N, u, log_n, &S, out3, tab});
+    if (c.kmax == kDeadTile) {
+      sc.degenerate = 1;
+      if (blockIdx.x == 0 && threadIdx.x == 0) rs_out3(c, log_n, tab, out3);
+    } else {
+      sc = S.sc;
+    }
+    O = S.O;
+  } else {
+    sc = *scp;
+  }
   if (sc.degenerate) {  // every weight zero: identity
     for (int q = 0; q < RS_IT; ++q)
       if (lj0 + q < n_local) anc[j0 + q] = (int32_t)(j0 + q);
@@ -779,28 +868,20 @@ __global__ void __launch_bounds__(RS_TPB, 3) rs_ancestors(
 }
 
 // Particle duplication: dst[f][i] = src[f][anc[i]], 16-byte stores of
-// consecutive particles; with sp != NULL row f is copied only if f < sp[anc[i]].
+// consecutive particles.
 template <typename T, int V>
 __global__ void gather_kernel(const T* __restrict__ src, T* __restrict__ dst,
-                              const int32_t* __restrict__ anc, const int32_t* __restrict__ sp,
-                              int64_t N, int n_fields) {
+                              const int32_t* __restrict__ anc, int64_t N, int n_fields) {
   const int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * V;
   if (i0 >= N) return;
   int32_t a[V];
-  int32_t s[V];
 #pragma unroll
-  for (int q = 0; q < V; ++q) {
-    a[q] = (i0 + q < N) ? __ldg(anc + i0 + q) : 0;
-    s[q] = sp ? ((i0 + q < N) ? __ldg(sp + a[q]) : 0) : n_fields;
-  }
+  for (int q = 0; q < V; ++q) a[q] = (i0 + q < N) ? __ldg(anc + i0 + q) : 0;
   const bool full = (i0 + V <= N) && ((reinterpret_cast<uintptr_t>(dst) & 15) == 0) && (N % V == 0);
   for (int f = 0; f < n_fields; ++f) {
     const T* sf = src + (size_t)f * N;
     T* df = dst + (size_t)f * N;
-    bool all = full;
-#pragma unroll
-    for (int q = 0; q < V; ++q) all = all && (f < s[q]);
-    if (all) {
+    if (full) {
       union {
         T e[V];
         uint4 u;
@@ -811,8 +892,51 @@ __global__ void gather_kernel(const T* __restrict__ src, T* __restrict__ dst,
     } else {
 #pragma unroll
       for (int q = 0; q < V; ++q)
-        if (i0 + q < N && f < s[q]) df[i0 + q] = __ldg(sf + a[q]);
+        if (i0 + q < N) df[i0 + q] = __ldg(sf + a[q]);
     }
+  }
+}
+
+// The same with stack pointers: row f only for the particles with f < sp[anc[i]].
+// Bound: HBM (a 32-byte sector of dst with some rows missing is read before it is
+// written).  A CTA takes GA_V * 256 consecutive particles, thread x those at x, x +
+// 256, ..., so that a warp's loads and stores cover whole lines whichever of its
+// particles still have the row and whatever the rows' alignment, and GA_U rows of
+// GA_V particles are loaded before the first store.  12 FP32 rows, the pointers
+// uniform: 2^24 particles 374 -> 308 us, 1.8 M 46.6 -> 37.0, 1 M 18.6 -> 12.7 against
+// four consecutive particles a thread; without stack pointers that form with its
+// 16-byte stores is the faster one (2^24 x 1 FP32 row 39 us against 80).
+constexpr int GA_TPB = 256, GA_V = 4;
+template <typename T, int GA_U>
+__global__ void __launch_bounds__(GA_TPB) gather_stack_kernel(
+    const T* __restrict__ src, T* __restrict__ dst, const int32_t* __restrict__ anc,
+    const int32_t* __restrict__ sp, int64_t N, int n_fields) {
+  const int64_t i0 = (int64_t)blockIdx.x * (GA_TPB * GA_V) + threadIdx.x;
+  const T* from[GA_V];
+  T* to[GA_V];
+  int rows[GA_V];
+  int most = 0;
+#pragma unroll
+  for (int q = 0; q < GA_V; ++q) {
+    const int64_t i = i0 + q * GA_TPB;
+    const int a = i < N ? __ldg(anc + i) : 0;
+    from[q] = src + a;
+    to[q] = dst + i;
+    rows[q] = i < N ? min(__ldg(sp + a), n_fields) : 0;
+    most = max(most, rows[q]);
+  }
+  for (int f = 0; f < most; f += GA_U) {
+    T e[GA_U][GA_V];
+#pragma unroll
+    for (int r = 0; r < GA_U; ++r)
+#pragma unroll
+      for (int q = 0; q < GA_V; ++q)
+        if (f + r < rows[q]) e[r][q] = __ldg(from[q] + (f + r) * N);
+#pragma unroll
+    for (int r = 0; r < GA_U; ++r)
+#pragma unroll
+      for (int q = 0; q < GA_V; ++q)
+        if (f + r < rows[q]) to[q][(f + r) * N] = e[r][q];
   }
 }
 
@@ -995,7 +1119,8 @@ std::mutex g_reduce_mu;
 int g_reduce_ctas[128];
 
 smc_status launch_rs_tile_reduce(const double* logw, int64_t N, TileRec* rec, unsigned* ehi,
-                                 long long* pref, const MathTab* tab, cudaStream_t cs) {
+                                 long long* pref, unsigned long long* n_near, const MathTab* tab,
+                                 cudaStream_t cs) {
   int dev = -1;
   SMC_CUDA_TRY(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 128) return set_error(SMC_EINVAL, "device ordinal %d out of range", dev);
@@ -1015,7 +1140,7 @@ smc_status launch_rs_tile_reduce(const double* logw, int64_t N, TileRec* rec, un
   }
   const int nt = (int)((N + RS_TILE - 1) / RS_TILE);
   SMC_CUDA_TRY(launch_dependent(rs_tile_reduce, (unsigned)std::min(grid, nt), RS1_TPB,
-                                RS1_TABLE_BYTES, cs, logw, N, nt, rec, ehi, pref, tab));
+                                RS1_TABLE_BYTES, cs, logw, N, nt, rec, ehi, pref, n_near, tab));
   return SMC_OK;
 }
 
@@ -1026,23 +1151,18 @@ smc_status rs_launch(const double* logw, int64_t N, double u, int32_t* ancestors
   smc_status ts = math_table(&tab);
   if (ts) return ts;
   const int nt = (int)((N + RS_TILE - 1) / RS_TILE);
-  SMC_CUDA_TRY(cudaMemsetAsync(n_near, 0, sizeof(int64_t), cs));
-  if ((ts = launch_rs_tile_reduce(logw, N, w.rec, w.ehi, w.pref, tab, cs))) return ts;
-  if ((ts = launch_rs_combine(w.rec, nt, N, u, w.O, w.sc, out3, tab, cs))) return ts;
   unsigned long long* nn = reinterpret_cast<unsigned long long*>(n_near);
-  const unsigned* no_ehi = nullptr;
-  const long long* no_pref = nullptr;
+  if ((ts = launch_rs_tile_reduce(logw, N, w.rec, w.ehi, w.pref, nn, tab, cs))) return ts;
+  const bool comb = nt <= RS_COMB_TILES;
+  if (!comb && (ts = launch_rs_combine(w.rec, nt, N, u, w.O, w.sc, out3, tab, cs))) return ts;
   int64_t* no_range = nullptr;
-  if (w.ehi)
-    SMC_CUDA_TRY(launch_dependent(rs_ancestors<true>, (unsigned)nt, RS_TPB, 0, cs, logw, N, 0, N,
-                                  (const TileRec*)w.rec, (const long long*)w.O,
-                                  (const RsScalars*)w.sc, (const unsigned*)w.ehi,
-                                  (const long long*)w.pref, ancestors, nn, no_range, tab));
-  else
-    SMC_CUDA_TRY(launch_dependent(rs_ancestors<false>, (unsigned)nt, RS_TPB, 0, cs, logw, N, 0, N,
-                                  (const TileRec*)w.rec, (const long long*)w.O,
-                                  (const RsScalars*)w.sc, no_ehi, no_pref, ancestors, nn, no_range,
-                                  tab));
+  auto* kern = w.ehi ? (comb ? rs_ancestors<true, true> : rs_ancestors<true, false>)
+                     : (comb ? rs_ancestors<false, true> : rs_ancestors<false, false>);
+  SMC_CUDA_TRY(launch_dependent(kern, (unsigned)nt, RS_TPB, 0, cs, logw, N, 0, N,
+                                (const TileRec*)w.rec, (const long long*)w.O,
+                                (const RsScalars*)w.sc, (const unsigned*)w.ehi,
+                                (const long long*)w.pref, ancestors, nn, no_range, u,
+                                std::log((double)N), out3, tab));
   return SMC_OK;
 }
 
@@ -1152,7 +1272,7 @@ extern "C" smc_status smc_shard_reduce(const double* logw, int64_t n_local, void
   smc_status ts = math_table(&tab);
   if (ts) return ts;
   NvtxRange nv("smc_shard_reduce");
-  return launch_rs_tile_reduce(logw, n_local, (TileRec*)records, nullptr, nullptr, tab,
+  return launch_rs_tile_reduce(logw, n_local, (TileRec*)records, nullptr, nullptr, nullptr, tab,
                                (cudaStream_t)stream);
 }
 
@@ -1191,10 +1311,9 @@ extern "C" smc_status smc_shard_ancestors(const double* logw, int64_t n_local, i
   const TileRec* rec = (const TileRec*)records_all;
   SMC_CUDA_TRY(cudaMemsetAsync(n_near, 0, sizeof(int64_t), cs));
   if ((st = launch_rs_combine(rec, nt_all, n_total, u, O, sc, out3, tab, cs))) return st;
-  rs_ancestors<false><<<nt, RS_TPB, 0, cs>>>(logw, n_local, (int)(first / RS_TILE), n_total, rec,
-                                             O, sc, nullptr, nullptr, ancestors,
-                                             reinterpret_cast<unsigned long long*>(n_near), range,
-                                             tab);
+  rs_ancestors<false, false><<<nt, RS_TPB, 0, cs>>>(
+      logw, n_local, (int)(first / RS_TILE), n_total, rec, O, sc, nullptr, nullptr, ancestors,
+      reinterpret_cast<unsigned long long*>(n_near), range, 0.0, 0.0, nullptr, tab);
   SMC_CUDA_TRY(cudaGetLastError());
   return SMC_OK;
 }
@@ -1204,14 +1323,21 @@ extern "C" smc_status smc_gather(const void* src, void* dst, const int32_t* anc,
   if (!src || !dst || !anc) return set_error(SMC_EINVAL, "NULL pointer");
   if (N < 1 || n_fields < 1) return set_error(SMC_EINVAL, "N and n_fields must be >= 1");
   cudaStream_t cs = (cudaStream_t)stream;
-  if (elem_bytes == 8) {
+  const unsigned grid = (unsigned)((N + GA_TPB * GA_V - 1) / (GA_TPB * GA_V));
+  if (sp && elem_bytes == 8) {
+    gather_stack_kernel<double, 2><<<grid, GA_TPB, 0, cs>>>((const double*)src, (double*)dst, anc,
+                                                            sp, N, n_fields);
+  } else if (sp && elem_bytes == 4) {
+    gather_stack_kernel<float, 4><<<grid, GA_TPB, 0, cs>>>((const float*)src, (float*)dst, anc, sp,
+                                                           N, n_fields);
+  } else if (elem_bytes == 8) {
     const int64_t threads = (N + 1) / 2;
     gather_kernel<double, 2><<<(unsigned)((threads + 255) / 256), 256, 0, cs>>>(
-        (const double*)src, (double*)dst, anc, sp, N, n_fields);
+        (const double*)src, (double*)dst, anc, N, n_fields);
   } else if (elem_bytes == 4) {
     const int64_t threads = (N + 3) / 4;
     gather_kernel<float, 4><<<(unsigned)((threads + 255) / 256), 256, 0, cs>>>(
-        (const float*)src, (float*)dst, anc, sp, N, n_fields);
+        (const float*)src, (float*)dst, anc, N, n_fields);
   } else {
     return set_error(SMC_EINVAL, "elem_bytes must be 4 or 8");
   }
