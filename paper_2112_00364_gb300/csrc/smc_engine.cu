@@ -54,23 +54,54 @@
 
 namespace smc {
 
-// Final outputs: real fields widened to f64, int fields, stack rows with
-// entries at or above the stack pointer zeroed.
+// A run's outputs, all in one launch (one job a grid row): log Z, log-weights, real
+// fields widened to f64, int fields, stack rows with entries at or above the stack
+// pointer zeroed, ancestor rows and resampling decisions.  The run's segment count is
+// read here, so the launch needs no result on the host first.  (A kernel and up to
+// four copies a run before, after a wait for its state: 25 ms of a batch of 512.)
 template <typename R>
-__global__ void finalize_kernel(StateView S, int N, int n_real, int n_int, int cap, double* real_out,
-                                int32_t* int_out, double* stack_out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  if (real_out)
-    for (int f = 0; f < n_real; ++f) real_out[(size_t)f * N + i] = (double)S.rf<R>(f, i, N);
-  if (int_out)
-    for (int f = 0; f < n_int; ++f) int_out[(size_t)f * N + i] = S.inf_(f, i, N);
-  if (stack_out && cap > 0) {
-    const int sp = S.inf_(1, i, N);
-    for (int r = 0; r < cap; ++r)
-      stack_out[(size_t)r * N + i] = r < sp ? (double)S.st<R>(r, i, N) : 0.0;
+__device__ __forceinline__ void collect_fields(const CollectJob& J, int fb, int i) {
+  const StateView& S = J.state[fb];
+  if (J.real)
+    for (int f = 0; f < J.n_real; ++f) J.real[(size_t)f * J.N + i] = (double)S.rf<R>(f, i, J.N);
+  if (J.ints)
+    for (int f = 0; f < J.n_int; ++f) J.ints[(size_t)f * J.N + i] = S.inf_(f, i, J.N);
+  if (J.stack && J.cap > 0) {
+    const int sp = S.inf_(1, i, J.N);
+    for (int r = 0; r < J.cap; ++r)
+      J.stack[(size_t)r * J.N + i] = r < sp ? (double)S.st<R>(r, i, J.N) : 0.0;
   }
 }
+
+__device__ __forceinline__ void collect_job(const CollectJob& J) {
+  const int segs = J.rs->n_segments;
+  const int fb = (segs - 1) & 1, turns = max(0, segs - 1);  // checkpoints the run went on from
+  const int first = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+  for (long long i = first; i < J.N; i += step) {
+    if (J.logw) J.logw[i] = J.src_logw[i];
+    if (segs > 0) {
+      if (J.fp32)
+        collect_fields<float>(J, fb, (int)i);
+      else
+        collect_fields<double>(J, fb, (int)i);
+    }
+  }
+  if (J.anc) {
+    const int rows = J.record_all ? min(turns, J.anc_rows) : min(turns, 1);
+    const long long n = (long long)rows * J.N;
+    for (long long i = first; i < n; i += step) J.anc[i] = J.src_anc[i];
+  }
+  if (J.resampled) {
+    const int t = min(turns, J.max_segments);
+    const int rows = J.record_all ? min(t, J.res_rows) : min(t, 1);
+    const int32_t* src = J.record_all ? J.dec : J.dec + (t - 1);
+    for (int i = first; i < rows; i += step) J.resampled[i] = src[i];
+  }
+  if (J.log_z && first == 0) *J.log_z = J.rs->log_z;
+}
+
+__global__ void collect_one_kernel(const __grid_constant__ CollectJob job) { collect_job(job); }
+__global__ void collect_kernel(const CollectJob* __restrict__ jobs) { collect_job(jobs[blockIdx.y]); }
 
 // ------------------------------------------------------------------------
 // host side
@@ -301,6 +332,114 @@ int real_state_fields(int kind) {
   return kind == SMC_MODEL_CRBD ? 3 : n_real;  // CRBD keeps log(lambda) internally
 }
 
+namespace {
+// The block of a run's outputs (one ancestor row): log Z and the decision in the
+// first 16 bytes, then log-weights, real fields, stack, int fields, ancestors.
+constexpr size_t kStageMax = 1u << 20;
+size_t stage_bytes(const smc_model_s* m, int64_t N) {
+  return 16 + (size_t)N * (8 * (size_t)(1 + m->n_real + m->stack_cap) + 4 * (size_t)(m->n_int + 1));
+}
+
+CollectJob collect_base(const smc_model_s* m, const smc_run_cfg* c, const Layout& Ly,
+                        const RunDev& A) {
+  CollectJob J;
+  std::memset(&J, 0, sizeof(J));
+  J.state[0] = A.state[0];
+  J.state[1] = A.state[1];
+  J.src_logw = A.logw;
+  J.src_anc = A.anc;
+  J.dec = A.dec;
+  J.rs = A.rs;
+  J.N = A.N;
+  J.n_real = m->n_real;
+  J.n_int = m->n_int;
+  J.cap = m->stack_cap;
+  J.fp32 = c->precision == SMC_PREC_FP32;
+  J.record_all = c->record_all_ancestors ? 1 : 0;
+  J.anc_rows = Ly.anc_rows;
+  J.max_segments = Ly.max_segments;
+  return J;
+}
+
+// The job that writes a run's device results.
+CollectJob collect_device(const smc_model_s* m, const smc_run_cfg* c, const Layout& Ly,
+                          const RunDev& A, const smc_result* r) {
+  CollectJob J = collect_base(m, c, Ly, A);
+  J.log_z = r->log_z;
+  J.logw = r->final_logw;
+  J.real = m->n_real ? r->real_fields : nullptr;
+  J.ints = r->int_fields;
+  J.stack = m->stack_cap ? r->stack : nullptr;
+  J.anc = r->ancestors;
+  J.resampled = r->resampled;
+  J.anc_rows = std::max(0, std::min(Ly.anc_rows, r->ancestors_rows));
+  J.res_rows = std::max(0, r->ancestors_rows);
+  return J;
+}
+
+// The job that writes a run's outputs to the block at `at` (one ancestor row).
+CollectJob collect_staged(const smc_model_s* m, const smc_run_cfg* c, const Layout& Ly,
+                          const RunDev& A, char* at) {
+  CollectJob J = collect_base(m, c, Ly, A);
+  const size_t N = (size_t)A.N;
+  J.log_z = (double*)at;
+  J.resampled = (int32_t*)(at + 8);
+  at += 16;
+  J.logw = (double*)at;
+  at += 8 * N;
+  if (m->n_real) J.real = (double*)at;
+  at += 8 * N * (size_t)m->n_real;
+  if (m->stack_cap) J.stack = (double*)at;
+  at += 8 * N * (size_t)m->stack_cap;
+  J.ints = (int32_t*)at;
+  at += 4 * N * (size_t)m->n_int;
+  J.anc = (int32_t*)at;
+  return J;
+}
+
+// From the block's host copy to the caller's arrays.
+void unstage(const smc_model_s* m, int64_t N, int n_segments, const char* at, smc_result* r) {
+  const size_t n = (size_t)N;
+  auto out = [&](void* dst, size_t bytes) {
+    if (dst && bytes) std::memcpy(dst, at, bytes);
+    at += bytes;
+  };
+  if (r->log_z) std::memcpy(r->log_z, at, 8);
+  if (r->resampled && n_segments > 1) std::memcpy(r->resampled, at + 8, 4);
+  at += 16;
+  out(r->final_logw, 8 * n);
+  out(r->real_fields, 8 * n * (size_t)m->n_real);
+  out(r->stack, 8 * n * (size_t)m->stack_cap);
+  out(r->int_fields, 4 * n * (size_t)m->n_int);
+  if (n_segments > 1) out(r->ancestors, 4 * n);
+}
+
+void launch_collect(const CollectJob& J, cudaStream_t cs) {
+  const long long words = std::max<long long>(J.N, J.record_all ? (long long)J.N * J.anc_rows / 8 : 0);
+  const unsigned ctas = (unsigned)std::min<long long>(2432, (words + 255) / 256);
+  collect_one_kernel<<<ctas, 256, 0, cs>>>(J);
+}
+
+void fill_counters(const RunState& hrs, smc_counters& ct) {
+  ct.n_segments = hrs.n_segments;
+  ct.n_resamples = hrs.n_resamples;
+  ct.n_ess_near = hrs.n_ess_near;
+  ct.n_near_boundary = (int64_t)hrs.n_near;
+  ct.n_overflow = (int64_t)hrs.n_overflow;
+  ct.n_limit = (int64_t)hrs.n_limit;
+  ct.n_draws = (int64_t)hrs.n_draws;
+  ct.n_blocks = (int64_t)hrs.n_blocks;
+  ct.log_z_closed = hrs.log_z_closed;
+  ct.debug_code = hrs.dbg_code;
+  ct.debug_index = hrs.dbg_index;
+  ct.debug_count = (int64_t)hrs.dbg_count;
+  int st = hrs.status;
+  if (st == 0 && !hrs.done) st = SMC_ESTEPLIMIT;
+  if (st == 0 && (hrs.n_overflow || hrs.n_limit)) st = SMC_WKILLED;
+  ct.status = st;
+}
+}  // namespace
+
 Layout make_layout(const smc_model_s* m, const smc_run_cfg* c) {
   Layout L{};
   const size_t N = (size_t)c->n_particles;
@@ -343,6 +482,9 @@ Layout make_layout(const smc_model_s* m, const smc_run_cfg* c) {
   L.fin_real = take(8 * N * (size_t)m->n_real);
   L.fin_int = take(4 * N * (size_t)m->n_int);
   L.fin_stack = take(8 * N * (size_t)m->stack_cap);
+  // host results up to kStageMax go out through one block and one copy
+  const size_t stage = stage_bytes(m, (int64_t)N);
+  L.stage = take(!c->record_all_ancestors && stage <= kStageMax ? stage : 0);
   // a host snapshot to resume from is copied here
   L.snap = take(c->resume_k > 0 && c->resume_where == SMC_MEM_HOST
                     ? (8 + 8 * (size_t)m->n_real + 8 * (size_t)m->stack_cap) * N + 4 * N * (size_t)m->n_int
@@ -671,45 +813,36 @@ smc_status check_tree(const smc_model_desc* d) {
 
 }  // namespace
 
-// Copies one finished run's outputs into its smc_result and fills its counters.
+// One finished run's outputs into its smc_result (stream-ordered) and its counters:
+// device results by one launch, host results through the workspace and a copy each.
 smc_status collect_run(const smc_model_s* m, const smc_run_cfg* c, const Layout& Ly, char* ws,
                        const RunDev& A, const RunState& hrs, smc_result* r, cudaStream_t cs) {
-  const int N = A.N;
-  const int fb = (hrs.n_segments - 1) & 1;
-  const bool host = r->where == SMC_MEM_HOST;
-  double* fin_real = host ? (double*)(ws + Ly.fin_real) : r->real_fields;
-  int32_t* fin_int = host ? (int32_t*)(ws + Ly.fin_int) : r->int_fields;
-  double* fin_stack = host ? (double*)(ws + Ly.fin_stack) : r->stack;
-  if (hrs.n_segments > 0 && (r->real_fields || r->int_fields || r->stack)) {
-    const int blocks = (N + 255) / 256;
-    if (c->precision == SMC_PREC_FP32)
-      finalize_kernel<float><<<blocks, 256, 0, cs>>>(A.state[fb], N, m->n_real, m->n_int, m->stack_cap,
-                                                     r->real_fields ? fin_real : nullptr,
-                                                     r->int_fields ? fin_int : nullptr,
-                                                     r->stack ? fin_stack : nullptr);
-    else
-      finalize_kernel<double><<<blocks, 256, 0, cs>>>(A.state[fb], N, m->n_real, m->n_int, m->stack_cap,
-                                                      r->real_fields ? fin_real : nullptr,
-                                                      r->int_fields ? fin_int : nullptr,
-                                                      r->stack ? fin_stack : nullptr);
+  fill_counters(hrs, r->counters);
+  if (r->where != SMC_MEM_HOST) {
+    launch_collect(collect_device(m, c, Ly, A, r), cs);
+    SMC_CUDA_TRY(cudaGetLastError());
+    return SMC_OK;
+  }
+  const size_t N = (size_t)A.N;
+  CollectJob J = collect_base(m, c, Ly, A);
+  if (m->n_real && r->real_fields) J.real = (double*)(ws + Ly.fin_real);
+  if (r->int_fields) J.ints = (int32_t*)(ws + Ly.fin_int);
+  if (m->stack_cap && r->stack) J.stack = (double*)(ws + Ly.fin_stack);
+  if (J.real || J.ints || J.stack) {
+    launch_collect(J, cs);
     SMC_CUDA_TRY(cudaGetLastError());
   }
-  const cudaMemcpyKind kind = host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
+  const cudaMemcpyKind kind = cudaMemcpyDeviceToHost;
   if (r->log_z) SMC_CUDA_TRY(cudaMemcpyAsync(r->log_z, &A.rs->log_z, 8, kind, cs));
-  if (r->final_logw) SMC_CUDA_TRY(cudaMemcpyAsync(r->final_logw, A.logw, 8 * (size_t)N, kind, cs));
-  if (host) {
-    if (r->real_fields && m->n_real)
-      SMC_CUDA_TRY(cudaMemcpyAsync(r->real_fields, fin_real, 8 * (size_t)N * m->n_real, kind, cs));
-    if (r->int_fields && m->n_int)
-      SMC_CUDA_TRY(cudaMemcpyAsync(r->int_fields, fin_int, 4 * (size_t)N * m->n_int, kind, cs));
-    if (r->stack && m->stack_cap)
-      SMC_CUDA_TRY(cudaMemcpyAsync(r->stack, fin_stack, 8 * (size_t)N * m->stack_cap, kind, cs));
-  }
+  if (r->final_logw) SMC_CUDA_TRY(cudaMemcpyAsync(r->final_logw, A.logw, 8 * N, kind, cs));
+  if (J.real) SMC_CUDA_TRY(cudaMemcpyAsync(r->real_fields, J.real, 8 * N * m->n_real, kind, cs));
+  if (J.ints) SMC_CUDA_TRY(cudaMemcpyAsync(r->int_fields, J.ints, 4 * N * m->n_int, kind, cs));
+  if (J.stack) SMC_CUDA_TRY(cudaMemcpyAsync(r->stack, J.stack, 8 * N * m->stack_cap, kind, cs));
   if (r->ancestors) {
     const int n_res = std::max(0, hrs.n_segments - 1);
     const int rows = c->record_all_ancestors ? std::min(std::min(n_res, r->ancestors_rows), Ly.anc_rows)
                                              : (n_res > 0 ? 1 : 0);
-    if (rows > 0) SMC_CUDA_TRY(cudaMemcpyAsync(r->ancestors, A.anc, 4 * (size_t)N * rows, kind, cs));
+    if (rows > 0) SMC_CUDA_TRY(cudaMemcpyAsync(r->ancestors, A.anc, 4 * N * rows, kind, cs));
   }
   if (r->resampled) {  // the decisions (record_all: one per checkpoint; else the last one)
     const int n_tr = std::max(0, std::min(hrs.n_segments - 1, Ly.max_segments));
@@ -717,23 +850,6 @@ smc_status collect_run(const smc_model_s* m, const smc_run_cfg* c, const Layout&
     const int32_t* src = c->record_all_ancestors ? A.dec : A.dec + (n_tr - 1);
     if (rows > 0) SMC_CUDA_TRY(cudaMemcpyAsync(r->resampled, src, 4 * (size_t)rows, kind, cs));
   }
-  smc_counters& ct = r->counters;
-  ct.n_segments = hrs.n_segments;
-  ct.n_resamples = hrs.n_resamples;
-  ct.n_ess_near = hrs.n_ess_near;
-  ct.n_near_boundary = (int64_t)hrs.n_near;
-  ct.n_overflow = (int64_t)hrs.n_overflow;
-  ct.n_limit = (int64_t)hrs.n_limit;
-  ct.n_draws = (int64_t)hrs.n_draws;
-  ct.n_blocks = (int64_t)hrs.n_blocks;
-  ct.log_z_closed = hrs.log_z_closed;
-  ct.debug_code = hrs.dbg_code;
-  ct.debug_index = hrs.dbg_index;
-  ct.debug_count = (int64_t)hrs.dbg_count;
-  int st = hrs.status;
-  if (st == 0 && !hrs.done) st = SMC_ESTEPLIMIT;
-  if (st == 0 && (hrs.n_overflow || hrs.n_limit)) st = SMC_WKILLED;
-  ct.status = st;
   return SMC_OK;
 }
 
@@ -977,6 +1093,7 @@ extern "C" void smc_model_destroy(smc_model_t m) {
     cudaEventDestroy(m->pin_ev);
   }
   if (m->pin) cudaFreeHost(m->pin);
+  if (m->pin_out) cudaFreeHost(m->pin_out);
   delete m;
 }
 
@@ -1051,22 +1168,6 @@ extern "C" smc_status smc_run(smc_model_t m, const smc_run_cfg* c, smc_result* r
       SMC_CUDA_TRY(cudaMemsetAsync(runs[0].dec, 0, 4 * (size_t)skip, cs));
     }
   }
-  // the run table through the handle's pinned buffer (no wait for the copy),
-  // once the previous call's upload from it has run
-  if (m->pin_ev) SMC_CUDA_TRY(cudaEventSynchronize(m->pin_ev));
-  const size_t meta_bytes = wave_meta_bytes(runs);
-  if (m->pin_bytes < meta_bytes) {
-    if (m->pin) cudaFreeHost(m->pin);
-    m->pin = nullptr;
-    m->pin_bytes = 0;
-    if (cudaMallocHost(&m->pin, meta_bytes) == cudaSuccess)
-      m->pin_bytes = meta_bytes;
-    else
-      cudaGetLastError();  // pageable staging instead
-  }
-  if (m->pin && !m->pin_ev) SMC_CUDA_TRY(cudaEventCreateWithFlags(&m->pin_ev, cudaEventDisableTiming));
-  if ((st = upload_wave(runs, ws + meta_off, cs, &W, &m->staging, m->pin))) return st;
-  if (m->pin) SMC_CUDA_TRY(cudaEventRecord(m->pin_ev, cs));
   SMC_CUDA_TRY(cudaEventRecord(m->ev0, cs));
   const bool known = m->n_segments_known > 0 && Ly.max_segments >= m->n_segments_known;
   int launched = 0;
@@ -1074,14 +1175,15 @@ extern "C" smc_status smc_run(smc_model_t m, const smc_run_cfg* c, smc_result* r
   std::vector<RunState*> states{runs[0].rs};
   NvtxRange nv_waves("smc_run/waves");
   // a small run (32-particle tiles, few enough for one CTA or one cluster) runs
-  // every segment in one launch: the same tiles and integers as the waves
+  // every segment in one launch, its table a parameter of it: the same tiles and
+  // integers as the waves
   const int one = c->launch_mode == SMC_LAUNCH_AUTO ? SMC_LAUNCH_CLUSTER : c->launch_mode;
   const bool small = (one == SMC_LAUNCH_ONE_CTA || one == SMC_LAUNCH_CLUSTER) &&
                      c->resume_k == 0 && !c->time_kernels && Ly.tile == 32 &&
                      Ly.n_tiles <= small_run_max_tiles(m->desc.kind, one);
   bool waves = !small;
   if (small) {
-    const cudaError_t e = launch_small_run(m->desc.kind, c->precision, one, W.runs, Ly.n_tiles, cs);
+    const cudaError_t e = launch_small_run(m->desc.kind, c->precision, one, runs[0], Ly.n_tiles, cs);
     if (e != cudaSuccess && c->launch_mode == SMC_LAUNCH_AUTO) {
       cudaGetLastError();  // a cluster the GPU cannot place: the waves instead
       waves = true;
@@ -1091,6 +1193,23 @@ extern "C" smc_status smc_run(smc_model_t m, const smc_run_cfg* c, smc_result* r
     }
   }
   if (waves) {
+    // the run table through the handle's pinned buffer (no wait for the copy),
+    // once the previous call's upload from it has run
+    if (m->pin_ev) SMC_CUDA_TRY(cudaEventSynchronize(m->pin_ev));
+    const size_t meta_bytes = wave_meta_bytes(runs);
+    if (m->pin_bytes < meta_bytes) {
+      if (m->pin) cudaFreeHost(m->pin);
+      m->pin = nullptr;
+      m->pin_bytes = 0;
+      if (cudaMallocHost(&m->pin, meta_bytes) == cudaSuccess)
+        m->pin_bytes = meta_bytes;
+      else
+        cudaGetLastError();  // pageable staging instead
+    }
+    if (m->pin && !m->pin_ev) SMC_CUDA_TRY(cudaEventCreateWithFlags(&m->pin_ev, cudaEventDisableTiming));
+    if ((st = upload_wave(runs, ws + meta_off, cs, &W, &m->staging, m->pin))) return st;
+    if (m->pin) SMC_CUDA_TRY(cudaEventRecord(m->pin_ev, cs));
+    SMC_CUDA_TRY(cudaEventRecord(m->ev0, cs));  // (the run's time begins after the upload)
     st = drive_waves(W, c->precision, states,
                      (known ? m->n_segments_known : Ly.max_segments) + 1 - skip, known, cs,
                      &m->ev_seg, c->time_kernels != 0, &launched, &kms,
@@ -1098,14 +1217,41 @@ extern "C" smc_status smc_run(smc_model_t m, const smc_run_cfg* c, smc_result* r
     if (st) return st;
   }
   SMC_CUDA_TRY(cudaEventRecord(m->ev1, cs));
-  RunState hrs;
-  SMC_CUDA_TRY(cudaMemcpyAsync(&hrs, runs[0].rs, sizeof(RunState), cudaMemcpyDeviceToHost, cs));
-  SMC_CUDA_TRY(cudaStreamSynchronize(cs));
   NvtxRange nv_collect("smc_run/collect");
+  // the outputs and the run's state in one go: device results by the collecting
+  // kernel, host results of up to 1 MB through a block and one copy of it into the
+  // handle's pinned buffer; only larger host results wait for the state first
+  const bool host = r->where == SMC_MEM_HOST;
+  const size_t block = host && !c->record_all_ancestors ? stage_bytes(m, c->n_particles) : 0;
+  const bool staged = block > 0 && block <= kStageMax;
+  const size_t pin_need = align_up(sizeof(RunState), 256) + (staged ? block : 0);
+  if (m->pin_out_bytes < pin_need) {
+    if (m->pin_out) cudaFreeHost(m->pin_out);
+    m->pin_out = nullptr;
+    m->pin_out_bytes = 0;
+    SMC_CUDA_TRY(cudaMallocHost(&m->pin_out, pin_need));
+    m->pin_out_bytes = pin_need;
+  }
+  char* pinned_block = m->pin_out + align_up(sizeof(RunState), 256);
+  if (!host)
+    launch_collect(collect_device(m, c, Ly, runs[0], r), cs);
+  else if (staged)
+    launch_collect(collect_staged(m, c, Ly, runs[0], ws + Ly.stage), cs);
+  SMC_CUDA_TRY(cudaGetLastError());
+  if (staged) SMC_CUDA_TRY(cudaMemcpyAsync(pinned_block, ws + Ly.stage, block, cudaMemcpyDeviceToHost, cs));
+  SMC_CUDA_TRY(cudaMemcpyAsync(m->pin_out, runs[0].rs, sizeof(RunState), cudaMemcpyDeviceToHost, cs));
+  SMC_CUDA_TRY(cudaStreamSynchronize(cs));
+  RunState hrs;
+  std::memcpy(&hrs, m->pin_out, sizeof(RunState));
   float ms = 0.f;
   cudaEventElapsedTime(&ms, m->ev0, m->ev1);
-  if ((st = collect_run(m, c, Ly, ws, runs[0], hrs, r, cs))) return st;
-  SMC_CUDA_TRY(cudaStreamSynchronize(cs));
+  if (host && !staged) {
+    if ((st = collect_run(m, c, Ly, ws, runs[0], hrs, r, cs))) return st;
+    SMC_CUDA_TRY(cudaStreamSynchronize(cs));
+  } else {
+    fill_counters(hrs, r->counters);
+    if (staged) unstage(m, c->n_particles, hrs.n_segments, pinned_block, r);
+  }
   r->counters.device_ms = ms;
   r->counters.kernel_launches = launched;
   r->counters.kernel_ms = kms;
@@ -1144,7 +1290,12 @@ extern "C" smc_status smc_run_batch(const smc_model_t* ms, const smc_run_cfg* cf
     runs[q].n_tiles = lys[q].n_tiles;
   }
   const size_t meta_off = total;
-  total += wave_meta_bytes(runs);
+  total = align_up(total + wave_meta_bytes(runs), 256);
+  // the runs' states side by side (one clear, one copy back) and the collecting jobs
+  const size_t rs_off = total;
+  total = align_up(total + sizeof(RunState) * (size_t)n_runs, 256);
+  const size_t job_off = total;
+  total += sizeof(CollectJob) * (size_t)n_runs;
   void* ws = nullptr;
   {
     cudaError_t e = cudaMallocAsync(&ws, total, cs);
@@ -1162,9 +1313,18 @@ extern "C" smc_status smc_run_batch(const smc_model_t* ms, const smc_run_cfg* cf
   for (int q = 0; q < n_runs; ++q) {
     runs[q] = make_rundev(ms[q], &cfgs[q], lys[q], (char*)ws + offs[q]);
     runs[q].redundant = combine_in_every_cta(lys[q].tile, lys[q].n_tiles, n_runs == 1);
+    runs[q].rs = (RunState*)((char*)ws + rs_off) + q;
     states[q] = runs[q].rs;
-    SMC_CUDA_TRY(cudaMemsetAsync(runs[q].rs, 0, sizeof(RunState), cs));
   }
+  SMC_CUDA_TRY(cudaMemsetAsync((char*)ws + rs_off, 0, sizeof(RunState) * (size_t)n_runs, cs));
+  // the jobs of the runs with device results, and the largest of their outputs
+  std::vector<CollectJob> jobs;
+  for (int q = 0; q < n_runs; ++q)
+    if (res[q].where != SMC_MEM_HOST)
+      jobs.push_back(collect_device(ms[q], &cfgs[q], lys[q], runs[q], &res[q]));
+  if (!jobs.empty())  // (pageable source: copied before the call returns)
+    SMC_CUDA_TRY(cudaMemcpyAsync((char*)ws + job_off, jobs.data(), sizeof(CollectJob) * jobs.size(),
+                                 cudaMemcpyHostToDevice, cs));
   WavePlan W;
   std::vector<char> staging;
   if ((st = upload_wave(runs, (char*)ws + meta_off, cs, &W, &staging))) return st;
@@ -1188,9 +1348,14 @@ extern "C" smc_status smc_run_batch(const smc_model_t* ms, const smc_run_cfg* cf
     return st;
   }
   SMC_CUDA_TRY(cudaEventRecord(e1, cs));
+  for (size_t j0 = 0; j0 < jobs.size(); j0 += 65535) {  // (grid rows)
+    const unsigned rows = (unsigned)std::min<size_t>(65535, jobs.size() - j0);
+    collect_kernel<<<dim3(32, rows), 256, 0, cs>>>((const CollectJob*)((char*)ws + job_off) + j0);
+  }
   std::vector<RunState> h(n_runs);
-  for (int q = 0; q < n_runs; ++q)
-    SMC_CUDA_TRY(cudaMemcpyAsync(&h[q], states[q], sizeof(RunState), cudaMemcpyDeviceToHost, cs));
+  SMC_CUDA_TRY(cudaGetLastError());
+  SMC_CUDA_TRY(cudaMemcpyAsync(h.data(), (char*)ws + rs_off, sizeof(RunState) * (size_t)n_runs,
+                               cudaMemcpyDeviceToHost, cs));
   const cudaError_t se = cudaStreamSynchronize(cs);
   graph_cache_clear(&graph);  // its launch has completed
   if (se != cudaSuccess) return cuda_fail(se, "cudaStreamSynchronize(batch)");
@@ -1199,7 +1364,9 @@ extern "C" smc_status smc_run_batch(const smc_model_t* ms, const smc_run_cfg* cf
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   for (int q = 0; q < n_runs; ++q) {
-    if ((st = collect_run(ms[q], &cfgs[q], lys[q], (char*)ws + offs[q], runs[q], h[q], &res[q], cs)))
+    if (res[q].where != SMC_MEM_HOST)
+      fill_counters(h[q], res[q].counters);
+    else if ((st = collect_run(ms[q], &cfgs[q], lys[q], (char*)ws + offs[q], runs[q], h[q], &res[q], cs)))
       return st;
     res[q].counters.device_ms = msec;
     res[q].counters.kernel_launches = launched;

@@ -73,9 +73,22 @@ struct RunDev {
   const double* snap_stack;
 };
 
+// A run's outputs for the collecting kernel: sources in the run's workspace, and
+// destinations in device memory (NULL: not wanted).
+struct CollectJob {
+  StateView state[2];
+  const double* src_logw;
+  const int32_t* src_anc;
+  const int32_t* dec;
+  const RunState* rs;
+  double *log_z, *logw, *real, *stack;
+  int32_t *ints, *anc, *resampled;
+  int N, n_real, n_int, cap, fp32, record_all, anc_rows, res_rows, max_segments;
+};
+
 struct Layout {
   size_t real[2], ints[2], stack[2], logw, E[2], ends[2], rec[2], tq[2], dec, tO, rs, anc, incr,
-      fin_real, fin_int, fin_stack, snap, total;
+      fin_real, fin_int, fin_stack, stage, snap, total;
   int n_tiles, tile, pad, anc_rows, max_segments;
 };
 
@@ -141,7 +154,7 @@ void block_free(void* p, size_t bytes, int dev);
 // most small_run_max_tiles(kind, launch_mode) of them; launch_mode
 // SMC_LAUNCH_ONE_CTA (grid 1) or SMC_LAUNCH_CLUSTER (one thread-block cluster).
 int small_run_max_tiles(int kind, int launch_mode);
-cudaError_t launch_small_run(int kind, int precision, int launch_mode, const RunDev* runs,
+cudaError_t launch_small_run(int kind, int precision, int launch_mode, const RunDev& run,
                              int n_tiles, cudaStream_t st);
 
 }  // namespace smc
@@ -162,6 +175,8 @@ struct smc_model_s {
   char* pin = nullptr;              // smc_run's pinned copy of it (uploaded without a wait)
   size_t pin_bytes = 0;
   cudaEvent_t pin_ev = nullptr;     // recorded after that upload: the buffer is free again
+  char* pin_out = nullptr;          // smc_run's pinned copy of the run's state and small host results
+  size_t pin_out_bytes = 0;
   smc::GraphCache graph;            // smc_run's captured waves (SMC_LAUNCH_GRAPH)
 };
 

@@ -194,21 +194,13 @@ __device__ __forceinline__ Combined combine_warp(const TileRec* rec, int nt, con
 // each with one warp more than its tiles: that of rank 0 closes the segments (log
 // Z, its records), off every tile's path.
 template <class M, int TPB, bool CL>
-__global__ void __launch_bounds__(TPB + (CL ? 32 : 0), 1) small_run_kernel(const RunDev* __restrict__ runs) {
+__global__ void __launch_bounds__(TPB + (CL ? 32 : 0), 1) small_run_kernel(const __grid_constant__ RunDev A) {
   using R = typename M::R;
   constexpr int WPC = TPB / 32;
   static_assert(CL || WPC >= 16, "one CTA holds the whole run");
-  __shared__ __align__(16) RunDev sr;
   constexpr int NT = TPB + (CL ? 32 : 0);
   __shared__ long long sh_O[NT / 32][kSmallMaxTiles + 1];  // each warp's own offsets
   __shared__ int sh_ks[NT / 32][kSmallMaxTiles + 1];
-  {
-    const int* src = reinterpret_cast<const int*>(runs);
-    int* dst = reinterpret_cast<int*>(&sr);
-    for (int w = threadIdx.x; w < (int)(sizeof(RunDev) / 4); w += NT) dst[w] = src[w];
-  }
-  __syncthreads();
-  const RunDev& A = sr;
   RunState* rs = A.rs;
   const int N = A.N;
   const int wid = (int)(threadIdx.x >> 5);
@@ -394,7 +386,7 @@ int small_run_max_tiles(int kind, int launch_mode) {
 
 namespace {
 template <class M, int TPB>
-cudaError_t launch_cluster(const RunDev* runs, int n_tiles, cudaStream_t st) {
+cudaError_t launch_cluster(const RunDev& run, int n_tiles, cudaStream_t st) {
   auto kern = small_run_kernel<M, TPB, true>;
   static std::once_flag once;
   static cudaError_t attr = cudaSuccess;
@@ -416,7 +408,7 @@ cudaError_t launch_cluster(const RunDev* runs, int n_tiles, cudaStream_t st) {
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, runs);
+  return cudaLaunchKernelEx(&cfg, kern, run);
 }
 
 // Whether the GPU schedules clusters of 16 CTAs of 64 threads (asked once per
@@ -451,38 +443,38 @@ bool wide_clusters() {
 }
 
 template <class M>
-cudaError_t launch_small_m(int launch_mode, int one_cta_tpb, const RunDev* runs, int n_tiles,
+cudaError_t launch_small_m(int launch_mode, int one_cta_tpb, const RunDev& run, int n_tiles,
                            cudaStream_t st) {
   if (launch_mode == SMC_LAUNCH_CLUSTER)
-    return wide_clusters() ? launch_cluster<M, 64>(runs, n_tiles, st)
-                           : launch_cluster<M, 128>(runs, n_tiles, st);
+    return wide_clusters() ? launch_cluster<M, 64>(run, n_tiles, st)
+                           : launch_cluster<M, 128>(run, n_tiles, st);
   if (one_cta_tpb == 1024)
-    small_run_kernel<M, 1024, false><<<1, 1024, 0, st>>>(runs);
+    small_run_kernel<M, 1024, false><<<1, 1024, 0, st>>>(run);
   else
-    small_run_kernel<M, 512, false><<<1, 512, 0, st>>>(runs);
+    small_run_kernel<M, 512, false><<<1, 512, 0, st>>>(run);
   return cudaGetLastError();
 }
 
 template <typename R>
-cudaError_t launch_small_r(int kind, int launch_mode, const RunDev* runs, int n_tiles,
+cudaError_t launch_small_r(int kind, int launch_mode, const RunDev& run, int n_tiles,
                            cudaStream_t st) {
   switch (kind) {
-    case SMC_MODEL_LG: return launch_small_m<LgModel<R>>(launch_mode, 1024, runs, n_tiles, st);
-    case SMC_MODEL_GEOMETRIC: return launch_small_m<GeoModel<R>>(launch_mode, 1024, runs, n_tiles, st);
-    case SMC_MODEL_SEIR: return launch_small_m<SeirModel<R>>(launch_mode, 512, runs, n_tiles, st);
+    case SMC_MODEL_LG: return launch_small_m<LgModel<R>>(launch_mode, 1024, run, n_tiles, st);
+    case SMC_MODEL_GEOMETRIC: return launch_small_m<GeoModel<R>>(launch_mode, 1024, run, n_tiles, st);
+    case SMC_MODEL_SEIR: return launch_small_m<SeirModel<R>>(launch_mode, 512, run, n_tiles, st);
     case SMC_MODEL_CRBD:
-      return launch_small_m<TreeModel<R, false>>(launch_mode, 512, runs, n_tiles, st);
+      return launch_small_m<TreeModel<R, false>>(launch_mode, 512, run, n_tiles, st);
     case SMC_MODEL_RATESHIFT:
-      return launch_small_m<TreeModel<R, true>>(launch_mode, 512, runs, n_tiles, st);
-    default: return launch_small_m<TreeDsModel<R>>(launch_mode, 512, runs, n_tiles, st);
+      return launch_small_m<TreeModel<R, true>>(launch_mode, 512, run, n_tiles, st);
+    default: return launch_small_m<TreeDsModel<R>>(launch_mode, 512, run, n_tiles, st);
   }
 }
 }  // namespace
 
-cudaError_t launch_small_run(int kind, int precision, int launch_mode, const RunDev* runs,
+cudaError_t launch_small_run(int kind, int precision, int launch_mode, const RunDev& run,
                              int n_tiles, cudaStream_t st) {
-  return precision == SMC_PREC_FP32 ? launch_small_r<float>(kind, launch_mode, runs, n_tiles, st)
-                                    : launch_small_r<double>(kind, launch_mode, runs, n_tiles, st);
+  return precision == SMC_PREC_FP32 ? launch_small_r<float>(kind, launch_mode, run, n_tiles, st)
+                                    : launch_small_r<double>(kind, launch_mode, run, n_tiles, st);
 }
 
 }  // namespace smc

@@ -275,8 +275,8 @@ LAUNCH = {"auto": 0, "graph": 1, "one_cta": 2, "cluster": 3, "waves": 4}
 
 
 def _cfg(N, seed, run_id, precision, max_segments, record_all, workspace, time_kernels=False,
-         ess_threshold=0.0, launch="auto"):
-    c = RunCfg()
+         ess_threshold=0.0, launch="auto", c=None):
+    c = RunCfg() if c is None else c
     c.time_kernels = int(time_kernels)
     c.launch_mode = LAUNCH[launch]
     c.ess_threshold = float(ess_threshold)
@@ -288,9 +288,14 @@ def _cfg(N, seed, run_id, precision, max_segments, record_all, workspace, time_k
     return c
 
 
+_OUTPUTS = ("log_z", "final_logw", "ancestors", "real_fields", "int_fields", "stack", "resampled")
+
+
 def _alloc_outputs(model: Model, N: int, rows: int, where: str, outputs: dict | None) -> dict:
-    shapes = _output_shapes(model, N, rows)
     out = dict(outputs or {})
+    if all(k in out or not _wanted(model, k) for k in _OUTPUTS):
+        return out
+    shapes = _output_shapes(model, N, rows)
     if where == "host":
         for k, (shp, dt) in shapes.items():
             if k not in out and _wanted(model, k):
@@ -319,12 +324,11 @@ def _rows(model: Model, max_segments: int, record_all: bool) -> int:
     return max(1, (max_segments or model.n_segments or 4096) - 1) if record_all else 1
 
 
-def _result_struct(out: dict, where: str, rows: int) -> Result:
-    r = Result()
+def _result_struct(out: dict, where: str, rows: int, r: Result | None = None) -> Result:
+    r = Result() if r is None else r
     r.where = MEM_HOST if where == "host" else MEM_DEVICE
     r.ancestors_rows = rows
-    for k in ("log_z", "final_logw", "ancestors", "real_fields", "int_fields", "stack",
-              "resampled"):
+    for k in _OUTPUTS:
         setattr(r, k, _ptr(out.get(k)))
     return r
 
@@ -399,13 +403,12 @@ def run_batch(models: list, specs: list, precision: str = "fp64", where: str = "
     ress = (Result * n)()
     outs, rows_l = [], []
     for q, (m, sp) in enumerate(zip(models, specs)):
-        c = _cfg(sp["N"], sp["seed"], sp.get("run_id", 0), precision, sp.get("max_segments", 0),
-                 record_all_ancestors, None, False, sp.get("ess_threshold", 0.0),
-                 "graph" if launch_graph else "waves")
-        cfgs[q] = c
+        _cfg(sp["N"], sp["seed"], sp.get("run_id", 0), precision, sp.get("max_segments", 0),
+             record_all_ancestors, None, False, sp.get("ess_threshold", 0.0),
+             "graph" if launch_graph else "waves", cfgs[q])
         rows = _rows(m, sp.get("max_segments", 0), record_all_ancestors)
         out = _alloc_outputs(m, sp["N"], rows, where, sp.get("outputs"))
-        ress[q] = _result_struct(out, where, rows)
+        _result_struct(out, where, rows, ress[q])
         outs.append(out)
         rows_l.append(rows)
     handles = (_vp * n)(*[m.handle for m in models])
