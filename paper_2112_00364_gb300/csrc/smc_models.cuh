@@ -461,6 +461,7 @@ struct TreeModel {
     bool ckpt, internal;
     int overflow, limited;
     R lam, mu, logw, loglam, inv_mu;
+    R top;  // RATESHIFT: the pending-rate stack's row sp - 1 as the segment began
     R lam_b, start, stop, lnp1, lnp2, lnp3, cur_t;
     R fr_t[SMC_MAX_DEPTH], fr_bl[SMC_MAX_DEPTH];
     int fr_rem[SMC_MAX_DEPTH];
@@ -479,9 +480,23 @@ struct TreeModel {
     L.pc = Sc.inf_(0, a, N);
     L.logw = (R)0;
     if (RS) {
-      // stack-pointer-bounded copy: only rows [0, sp) of the ancestor's stack
+      // stack-pointer-bounded copy: only rows [0, sp) of the ancestor's stack, eight
+      // loaded before the first is stored (one after another each waited for the load
+      // before it: rows times an L2 round trip); the top row stays in a register for
+      // the branch that reads it
       L.sp = Sc.inf_(1, a, N);
-      for (int r = 0; r < L.sp; ++r) Sn.st<R>(r, i, N) = Sc.st<R>(r, a, N);
+      for (int r0 = 0; r0 < L.sp; r0 += 8) {
+        R e[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+          if (r0 + r < L.sp) e[r] = Sc.st<R>(r0 + r, a, N);
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+          if (r0 + r < L.sp) {
+            Sn.st<R>(r0 + r, i, N) = e[r];
+            L.top = e[r];
+          }
+      }
     }
   }
   __device__ static void store(const Lane& L, const StateView& Sn, int i, int N) {
@@ -549,10 +564,10 @@ struct TreeModel {
           if (L.sp <= 0) {
             lam_p = L.lam;
           } else if (br.flags & 2) {
-            lam_p = S.st<R>(L.sp - 1, i, N);  // left child: parent's rate stays pending
+            lam_p = L.top;  // left child: parent's rate stays pending
           } else {
             L.sp -= 1;  // right child: last use of the parent's rate
-            lam_p = S.st<R>(L.sp, i, N);
+            lam_p = L.top;
           }
           R mult;
           if (md.fixed_mult) {
@@ -748,9 +763,17 @@ __device__ __forceinline__ int run_segment(typename M::Lane& L, Stream& s, const
     if (M::NB == 1) {
       sel = 0;
     } else {
-      const unsigned peers = __match_any_sync(0xffffffffu, active ? L.pc : -2);
-      const unsigned key = active ? ((unsigned)__popc(peers) << 8) | (unsigned)L.pc : 0u;
-      sel = (int)(__reduce_max_sync(0xffffffffu, key) & 0xffu);
+      // (a vote a block index: shorter than matching the lanes' indices, 0.5%)
+      sel = 0;
+      int best = 0;
+#pragma unroll
+      for (int b = 0; b < M::NB; ++b) {
+        const int n = __popc(__ballot_sync(0xffffffffu, active && L.pc == b));
+        if (n > 0 && n >= best) {
+          best = n;
+          sel = b;
+        }
+      }
     }
     if (active && L.pc == sel) {
       M::block(sel, L, s, md, S, i, k, N);
