@@ -7,14 +7,15 @@
 // Warp w of CTA r (its rank in the cluster; 0 without one) is tile
 // r * (TPB / 32) + w of the run.  Each segment is the wave kernel's work with a
 // barrier between the steps that need one:
-//   combine   (k > 0) the previous segment's tile records (in global memory,
-//             written by every CTA of the cluster) combined by each CTA for
+//   combine   (k > 0) the previous segment's tile records (in this CTA's shared
+//             memory, where every CTA of the cluster wrote its own: a load of 30
+//             cycles instead of an L2 round trip) combined by each warp for
 //             itself into exact integer offsets (smc_combine.cuh), the log-Z
 //             increment, the resampling decision and the search scalars: the
 //             same integers in every CTA, so the same decisions;
-//   search    each particle's systematic-resampling ancestor and the fused
-//             gather of its state (step_tile's code, with the offsets and tile
-//             references in shared memory);
+//   search    each particle's systematic-resampling ancestor (the running sums from
+//             the shared memory of the ancestor's CTA) and the fused gather of its
+//             state;
 //   segment   blocks to the next checkpoint with per-warp PC-sorted dispatch;
 //   epilogue  per warp: its power-of-two reference, integer weights, running
 //             sums and tile record (a warp is a tile, so the tile reference is
@@ -23,7 +24,10 @@
 // the records, running sums and states written before it by any CTA of the
 // cluster are visible to every CTA after it); the double-buffered records,
 // sums and states of segment k are not written again before the barrier that
-// ends segment k + 1, which every CTA reaches only after its reads of them.
+// ends segment k + 1, which every CTA reaches only after its reads of them.  No CTA
+// reads another's shared memory after the last barrier, so each may then end.  The
+// first remote store comes after a cluster barrier at the start: every CTA is
+// resident by then.
 // The tiles, their rounding and the combine's integers are those of the wave
 // kernel for the same N, so a run gives the same bits here, alone through the
 // waves, batched and served.  The barriers are the hardware's (every CTA of a
@@ -56,16 +60,38 @@ __device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
+// A store to, and a load from, the shared memory of CTA `rank` of the cluster at
+// the address that `p` has in this CTA's (without a cluster: this CTA's own).
+__device__ __forceinline__ unsigned smem_at(const void* p, unsigned rank) {
+  unsigned a = (unsigned)__cvta_generic_to_shared(p), r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void store_to_cta(longlong2* p, longlong2 v, unsigned rank) {
+  asm volatile("st.shared::cluster.v2.s64 [%0], {%1, %2};"
+               :: "r"(smem_at(p, rank)), "l"(v.x), "l"(v.y) : "memory");
+}
+__device__ __forceinline__ void store_to_cta(long long* p, long long v, unsigned rank) {
+  asm volatile("st.shared::cluster.s64 [%0], %1;" :: "r"(smem_at(p, rank)), "l"(v) : "memory");
+}
+__device__ __forceinline__ long long load_from_cta(const long long* p, unsigned rank) {
+  long long v;
+  asm volatile("ld.shared::cluster.s64 %0, [%1];" : "=l"(v) : "r"(smem_at(p, rank)) : "memory");
+  return v;
+}
+
 // systematic_search for one warp of a small run (tiles of 32 particles): each
 // lane's tile from the offsets as there; then, per distinct tile among the
 // lanes (one or two, the offsets being non-decreasing), the tile's 32 running
-// sums in one load (lane l holds E_{j0+l}) and every lane of that tile finds
+// sums in one load (lane l holds E_{j0+l}, from the shared memory of the tile's CTA)
+// and every lane of that tile finds
 // its first j with E_j > F by a binary search over the shuffled values.  The
 // same ancestors and near-boundary flags as systematic_search; one dependent
 // load of the sums instead of the 8-ary search's two.  Every lane calls it;
 // `want` marks the lanes whose offset is searched.
+template <int WPC, bool CL>
 __device__ __forceinline__ int small_search(int i, bool want, const RunDev& A, const SearchCtx& X,
-                                            const long long* E, bool* near) {
+                                            const long long (*E)[32], bool* near) {
   constexpr unsigned kAll = 0xffffffffu;
   const int N = A.N, T = A.n_tiles, lane = threadIdx.x & 31;
   int a = i, t = -1;
@@ -97,7 +123,8 @@ __device__ __forceinline__ int small_search(int i, bool want, const RunDev& A, c
   while (pending) {
     const int tg = __shfl_sync(kAll, t, __ffs(pending) - 1);
     const int j0 = tg * 32, len = min(32, N - j0);
-    const long long e = lane < len ? __ldcg(E + j0 + lane) : 0x7FFFFFFFFFFFFFFFll;
+    long long e = 0x7FFFFFFFFFFFFFFFll;
+    if (lane < len) e = CL ? load_from_cta(&E[tg % WPC][lane], (unsigned)(tg / WPC)) : E[tg][lane];
     // pos = #{ l < len : E_{j0+l} <= F } (the sums are non-decreasing)
     int pos = 0;
 #pragma unroll
@@ -149,7 +176,7 @@ __device__ __forceinline__ Combined combine_warp(const TileRec* rec, int nt, con
   r.s = 0;
   r.k = kDeadTile;
   r.alive = 0;
-  if (lane < nt) r = load_rec(rec + lane);
+  if (lane < nt) r = rec[lane];
   Combined c;
   c.kmax = __reduce_max_sync(kAll, r.k);
   c.alive = __any_sync(kAll, r.alive) ? 1 : 0;
@@ -179,7 +206,7 @@ __device__ __forceinline__ Combined combine_warp(const TileRec* rec, int nt, con
     double acc = 0.0;
     if (lane < nt && r.k != kDeadTile) {
       const int d2 = 2 * (c.kmax - r.k);
-      if (d2 < 900) acc = acc + (double)__ldcg(q + lane) * pow2i(-54 - d2);
+      if (d2 < 900) acc = acc + (double)q[lane] * pow2i(-54 - d2);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc = acc + __shfl_xor_sync(kAll, acc, o);
@@ -201,6 +228,15 @@ __global__ void __launch_bounds__(TPB + (CL ? 32 : 0), 1) small_run_kernel(const
   constexpr int NT = TPB + (CL ? 32 : 0);
   __shared__ long long sh_O[NT / 32][kSmallMaxTiles + 1];  // each warp's own offsets
   __shared__ int sh_ks[NT / 32][kSmallMaxTiles + 1];
+  // double-buffered by segment parity: every tile's record (and sum of squared
+  // weights), and the running sums of this CTA's tiles
+  __shared__ __align__(16) TileRec sh_rec[2][kSmallMaxTiles];
+  __shared__ long long sh_tq[2][kSmallMaxTiles];
+  __shared__ long long sh_E[2][WPC][32];
+  if (CL) {
+    cluster_arrive();
+    cluster_wait();
+  }
   RunState* rs = A.rs;
   const int N = A.N;
   const int wid = (int)(threadIdx.x >> 5);
@@ -210,6 +246,7 @@ __global__ void __launch_bounds__(TPB + (CL ? 32 : 0), 1) small_run_kernel(const
   const int t = (CL ? (int)cluster_rank() * WPC : 0) + wid;
   const int lane = threadIdx.x & 31;
   const int i = t * 32 + lane;  // the tile of this path is 32 particles
+  const int ctas = (int)gridDim.x;  // (the cluster is the grid)
   const bool tile_live = !extra && t < A.n_tiles;
   const bool valid = tile_live && i < N;
   // segment k - 1's closing (log Z, its records) waits for the barrier that
@@ -233,7 +270,7 @@ __global__ void __launch_bounds__(TPB + (CL ? 32 : 0), 1) small_run_kernel(const
     }
     bool near = false;
     if (k > 0) {
-      const Combined c = combine_warp(A.rec[cb], A.n_tiles, A.ess ? A.tq[cb] : nullptr,
+      const Combined c = combine_warp(sh_rec[cb], A.n_tiles, A.ess ? sh_tq[cb] : nullptr,
                                       sh_O[wid], sh_ks[wid]);
       const bool go_on = c.kmax != kDeadTile && c.alive && k < A.max_segments;
       const bool resample = decide_resample(A, c);
@@ -258,7 +295,7 @@ __global__ void __launch_bounds__(TPB + (CL ? 32 : 0), 1) small_run_kernel(const
 #pragma unroll
       for (int q = 0; q < 5; ++q) q5[q] = __shfl_sync(0xffffffffu, q5[q], 0);
       SearchCtx X;
-      X.rec = A.rec[cb];
+      X.rec = nullptr;
       X.O = sh_O[wid];
       X.ks = sh_ks[wid];
       X.kmax = c.kmax;
@@ -266,7 +303,7 @@ __global__ void __launch_bounds__(TPB + (CL ? 32 : 0), 1) small_run_kernel(const
       X.d = Q64{q5[0], q5[1]};
       X.z0 = Q64{q5[2], q5[3]};
       X.tolZ = (long long)q5[4];
-      const int a_s = resample ? small_search(i, valid, A, X, A.E[cb], &near) : i;
+      const int a_s = resample ? small_search<WPC, CL>(i, valid, A, X, sh_E[cb], &near) : i;
       if (valid) {
         const int row = A.record_all ? k - 1 : 0;
         int a = a_s;
@@ -334,20 +371,26 @@ __global__ void __launch_bounds__(TPB + (CL ? 32 : 0), 1) small_run_kernel(const
       }
     }
     const long long E = block_incl_scan_i64<32>(ef, nullptr);  // a warp scan
-    if (valid) A.E[nb][i] = E;
+    if (tile_live) sh_E[nb][wid][lane] = E;
     if (A.ess) {
       const unsigned long long u = (unsigned long long)ef;
       const long long sq = (long long)((__umul64hi(u, u) << 10) | ((u * u) >> 54));
-      const long long Q = block_incl_scan_i64<32>(sq, nullptr);
-      if (tile_live && lane == 31) A.tq[nb][t] = Q;
+      const long long Q = __shfl_sync(0xffffffffu, block_incl_scan_i64<32>(sq, nullptr), 31);
+      if (CL) {
+        if (tile_live && lane < ctas) store_to_cta(&sh_tq[nb][t], Q, (unsigned)lane);
+      } else if (tile_live && lane == 0) {
+        sh_tq[nb][t] = Q;
+      }
     }
     const int tile_alive = __any_sync(0xffffffffu, alive) ? 1 : 0;
-    if (tile_live && lane == 31) {
-      TileRec r;
-      r.s = E;
-      r.k = kt;
-      r.alive = tile_alive;
-      A.rec[nb][t] = r;
+    // the record to every CTA of the cluster, a lane each
+    longlong2 rec;
+    rec.x = __shfl_sync(0xffffffffu, E, 31);
+    rec.y = (long long)(unsigned)kt | ((long long)tile_alive << 32);
+    if (CL) {
+      if (tile_live && lane < ctas) store_to_cta(reinterpret_cast<longlong2*>(&sh_rec[nb][t]), rec, (unsigned)lane);
+    } else if (tile_live && lane == 0) {
+      *reinterpret_cast<longlong2*>(&sh_rec[nb][t]) = rec;
     }
     // the segment's records, running sums and states, for the next combine
     if (CL) cluster_arrive();
