@@ -42,6 +42,22 @@ __device__ __forceinline__ int tile_exponent(double M) { return (int)ceil(M * kI
 
 __device__ __forceinline__ float trunc_f32(unsigned hi, unsigned lo);
 
+// A float as a double from its bits, but for subnormals and NaN (a conversion runs at
+// the FP64 pipe's rate).
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ double widen(float x) {
+  const unsigned b = __float_as_uint(x), mag = b & 0x7fffffffu, sign = b & 0x80000000u;
+  if (mag - 0x00800000u < 0x7f000000u)
+    return __hiloint2double((int)(sign | ((mag >> 3) + 0x38000000u)), (int)(b << 29));
+  if (mag == 0u) return __hiloint2double((int)sign, 0);
+  if (mag == 0x7f800000u) return __hiloint2double((int)(sign | 0x7ff00000u), 0);
+  return (double)x;
+}
+
+__device__ __forceinline__ bool is_neg_inf(double x) {
+  return (unsigned long long)__double_as_longlong(x) == 0xFFF0000000000000ull;
+}
+
 // tile_exponent off the FP64 pipe (three operations of 16 issue cycles a warp
 // there): in single precision wherever M / ln 2 lies further from an integer than
 // the error of that (below 2.5e-7 relative), else as above.

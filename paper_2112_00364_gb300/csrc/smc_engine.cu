@@ -948,7 +948,7 @@ extern "C" smc_status smc_model_register(const smc_model_desc* d, smc_model_t* o
     if (d->T < 1 || !d->obs) return set_error(SMC_EINVAL, "LG needs T >= 1 observations");
     if (!(d->r_sd > 0.0) || !(d->x0_sd >= 0.0) || !(d->q_sd >= 0.0))
       return set_error(SMC_EINVAL, "LG standard deviations must be >= 0 (r_sd > 0)");
-    blob = 8 * (size_t)d->T;
+    blob = align_up(8 * (size_t)d->T, 256) + 4 * (size_t)d->T;
   } else if (d->kind == SMC_MODEL_SEIR) {
     if (d->T < 1 || !d->obs) return set_error(SMC_EINVAL, "SEIR needs T >= 1 days of reports");
     for (int t = 0; t < d->T; ++t)
@@ -984,21 +984,21 @@ extern "C" smc_status smc_model_register(const smc_model_desc* d, smc_model_t* o
   md.depth_cap = d->depth_cap;
   md.call_limit = d->call_limit;
   md.lam_stack_cap = d->lam_stack_cap;
-  md.x0_mean = d->x0_mean;
-  md.x0_sd = d->x0_sd;
-  md.a = d->a;
-  md.b = d->b;
-  md.q_sd = d->q_sd;
-  md.r_sd = d->r_sd;
-  md.rho = d->rho;
-  md.lambda_fixed = d->lambda_fixed;
-  md.mu_fixed = d->mu_fixed;
-  md.lambda_scale = d->lambda_scale;
-  md.mu_scale = d->mu_scale;
-  md.sigma = d->sigma;
-  md.geo_p = d->geo_p;
-  md.geo_logw = d->geo_logw;
-  md.log_rho = d->rho > 0.0 ? std::log(d->rho) : 0.0;
+  md.d.x0_mean = d->x0_mean;
+  md.d.x0_sd = d->x0_sd;
+  md.d.a = d->a;
+  md.d.b = d->b;
+  md.d.q_sd = d->q_sd;
+  md.d.r_sd = d->r_sd;
+  md.d.rho = d->rho;
+  md.d.lambda_fixed = d->lambda_fixed;
+  md.d.mu_fixed = d->mu_fixed;
+  md.d.lambda_scale = d->lambda_scale;
+  md.d.mu_scale = d->mu_scale;
+  md.d.sigma = d->sigma;
+  md.d.geo_p = d->geo_p;
+  md.d.geo_logw = d->geo_logw;
+  md.d.log_rho = d->rho > 0.0 ? std::log(d->rho) : 0.0;
   {
     const MathTab* tab = nullptr;
     smc_status ts = math_table(&tab);
@@ -1010,8 +1010,8 @@ extern "C" smc_status smc_model_register(const smc_model_desc* d, smc_model_t* o
   }
   m->n_segments_known = 0;
   if (d->kind == SMC_MODEL_LG) {
-    md.inv_r_sd = d->r_sd > 0x1p-100 && d->r_sd < 0x1p100 ? 1.0 / d->r_sd : 0.0;
-    md.lg_lc = std::log(d->r_sd) + 0.91893853320467274178;
+    md.d.inv_r_sd = d->r_sd > 0x1p-100 && d->r_sd < 0x1p100 ? 1.0 / d->r_sd : 0.0;
+    md.d.lg_lc = std::log(d->r_sd) + 0.91893853320467274178;
     m->n_segments_known = d->T;
   }
   if (d->kind == SMC_MODEL_SEIR) m->n_segments_known = d->T;
@@ -1019,9 +1019,10 @@ extern "C" smc_status smc_model_register(const smc_model_desc* d, smc_model_t* o
     const int tips = (d->n_nodes + 1) / 2;
     double lnfact = 0.0;
     for (int i = 2; i <= tips; ++i) lnfact = lnfact + std::log((double)i);
-    md.corr = (double)(tips - 1) * kLn2 - lnfact;
+    md.d.corr = (double)(tips - 1) * kLn2 - lnfact;
     m->n_segments_known = d->n_nodes;
   }
+  md.f.from(md.d);
   cudaGetDevice(&m->dev);
   if (blob) {
     if (d->fixed_mult) blob += align_up(8 * (size_t)d->n_nodes, 256);
@@ -1043,6 +1044,10 @@ extern "C" smc_status smc_model_register(const smc_model_desc* d, smc_model_t* o
     bool ok = true;
     if (d->kind == SMC_MODEL_LG || d->kind == SMC_MODEL_SEIR) {
       ok = (md.obs = (const double*)put(d->obs, 8 * (size_t)d->T)) != nullptr;
+      if (ok && d->kind == SMC_MODEL_LG) {
+        std::vector<float> y(d->obs, d->obs + d->T);
+        ok = (md.obs_f = (const float*)put(y.data(), 4 * (size_t)d->T)) != nullptr;
+      }
     } else {
       const size_t M = d->n_nodes;
       ok = (md.parent = (const int*)put(d->parent, 4 * M)) && (md.left = (const int*)put(d->left, 4 * M)) &&
@@ -1059,6 +1064,8 @@ extern "C" smc_status smc_model_register(const smc_model_desc* d, smc_model_t* o
           r.start = d->age[pa];
           r.flags = (d->left[v] >= 0 ? 1 : 0) | (d->left[pa] == v ? 2 : 0);
         }
+        r.start_f = (float)r.start;
+        r.stop_f = (float)r.stop;
         br[k] = r;
       }
       if (ok) ok = (md.branch = (const BranchRec*)put(br.data(), sizeof(BranchRec) * M)) != nullptr;

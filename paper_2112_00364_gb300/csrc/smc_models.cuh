@@ -28,28 +28,54 @@ namespace smc {
 struct BranchRec {
   double start, stop;
   int v, flags;
-  long long pad_;
+  float start_f, stop_f;  // start and stop rounded to float
+  __host__ __device__ double begin_at(double) const { return start; }
+  __host__ __device__ float begin_at(float) const { return start_f; }
+  __host__ __device__ double end_at(double) const { return stop; }
+  __host__ __device__ float end_at(float) const { return stop_f; }
 };
 
 __device__ __forceinline__ BranchRec load_branch(const BranchRec* __restrict__ b, int k) {
   const double2 a = __ldg(reinterpret_cast<const double2*>(b + k));
   const int4 c = __ldg(reinterpret_cast<const int4*>(b + k) + 1);
-  return BranchRec{a.x, a.y, c.x, c.y, 0};
+  return BranchRec{a.x, a.y, c.x, c.y, __int_as_float(c.z), __int_as_float(c.w)};
 }
+
+// A model's numbers in the particles' precision.
+template <typename R>
+struct ModelConst {
+  R x0_mean, x0_sd, a, b, q_sd, r_sd, inv_r_sd, lg_lc, corr;
+  R log_rho, rho, lambda_fixed, mu_fixed, lambda_scale, mu_scale, sigma, geo_p, geo_logw;
+  template <typename S>
+  __host__ void from(const ModelConst<S>& o) {
+    x0_mean = (R)o.x0_mean, x0_sd = (R)o.x0_sd, a = (R)o.a, b = (R)o.b, q_sd = (R)o.q_sd;
+    r_sd = (R)o.r_sd, inv_r_sd = (R)o.inv_r_sd, lg_lc = (R)o.lg_lc, corr = (R)o.corr;
+    log_rho = (R)o.log_rho, rho = (R)o.rho, lambda_fixed = (R)o.lambda_fixed;
+    mu_fixed = (R)o.mu_fixed, lambda_scale = (R)o.lambda_scale, mu_scale = (R)o.mu_scale;
+    sigma = (R)o.sigma, geo_p = (R)o.geo_p, geo_logw = (R)o.geo_logw;
+  }
+};
 
 struct ModelDev {
   int kind, T, n_nodes, fixed_rates, depth_cap, call_limit, lam_stack_cap, pad_;
   const MathTab* tab;  // this device's log / exp tables
-  double log_rho;      // log(rho), computed on the host
   const double* obs;
+  const float* obs_f;  // the observations rounded to float
   const BranchRec* branch;  // tree models: [n_nodes], entry k for k >= 1
   const int* parent;
   const int* left;
   const int* preorder;
   const double* age;
   const double* fixed_mult;
-  double x0_mean, x0_sd, a, b, q_sd, r_sd, inv_r_sd, lg_lc, corr;
-  double rho, lambda_fixed, mu_fixed, lambda_scale, mu_scale, sigma, geo_p, geo_logw;
+  // the model's numbers, and the same rounded to float: a conversion in the kernel runs
+  // at the FP64 pipe's rate, and those of a linear-Gaussian step with FP32 particles
+  // kept it 31% busy
+  ModelConst<double> d;
+  ModelConst<float> f;
+  __host__ __device__ const ModelConst<double>& c(double) const { return d; }
+  __host__ __device__ const ModelConst<float>& c(float) const { return f; }
+  __device__ double y(int k, double) const { return obs[k]; }
+  __device__ float y(int k, float) const { return obs_f[k]; }
 };
 
 // One buffer of the double-buffered SoA PSTATE (Section 3.3's separate arrays
@@ -139,23 +165,23 @@ struct LgModel {
   // where neither can overflow or lose bits (inv_r_sd is 0 for an extreme r_sd)
   __device__ static double over_r_sd(double x, const ModelDev& md) {
     const unsigned ex = (unsigned)((unsigned long long)__double_as_longlong(x) >> 52) & 0x7ffu;
-    if (md.inv_r_sd == 0.0 || ex > 1023u + 900u) return x / md.r_sd;
-    return div_by(x, md.r_sd, md.inv_r_sd);
+    if (md.d.inv_r_sd == 0.0 || ex > 1023u + 900u) return x / md.d.r_sd;
+    return div_by(x, md.d.r_sd, md.d.inv_r_sd);
   }
-  __device__ static float over_r_sd(float x, const ModelDev& md) { return x / (float)md.r_sd; }
+  __device__ static float over_r_sd(float x, const ModelDev& md) { return x / md.f.r_sd; }
   __device__ static void block(int b, Lane& L, Stream& s, const ModelDev& md, const StateView&, int,
                                int k, int) {
     if (b == 0) {
       const R z0 = normal01<R>(s);
-      L.x = m_fma((R)md.x0_sd, z0, (R)md.x0_mean);
+      L.x = m_fma(md.c((R)0).x0_sd, z0, md.c((R)0).x0_mean);
       L.pc = 1;
       return;
     }
     const R z = L.drawn ? L.z : normal01<R>(s);
-    L.x = m_fma((R)md.a, L.x, m_fma((R)md.q_sd, z, (R)md.b));
-    const R y = (R)md.obs[k];
+    L.x = m_fma(md.c((R)0).a, L.x, m_fma(md.c((R)0).q_sd, z, md.c((R)0).b));
+    const R y = md.y(k, (R)0);
     const R dz = over_r_sd(y - L.x, md);
-    const R lp = (R)-0.5 * (dz * dz) - (R)md.lg_lc;
+    const R lp = (R)-0.5 * (dz * dz) - md.c((R)0).lg_lc;
     L.logw = L.logw + lp;
     L.pc = (k + 1 == md.T) ? PC_STOP : 1;
     L.ckpt = true;
@@ -206,10 +232,10 @@ struct GeoModel {
   }
   __device__ static void block(int, Lane& L, Stream& s, const ModelDev& md, const StateView&, int,
                                int, int) {
-    const bool heads = bernoulli<R>(s, (R)md.geo_p);
+    const bool heads = bernoulli<R>(s, md.c((R)0).geo_p);
     L.count += 1;
     if (heads) {
-      L.logw = L.logw + (R)md.geo_logw;
+      L.logw = L.logw + md.c((R)0).geo_logw;
       L.pc = 0;
     } else {
       L.pc = PC_STOP;
@@ -407,7 +433,7 @@ __device__ __forceinline__ void hidden_event(typename M::Lane& L, Stream& s, con
   const R t = L.cur_t;
   const R dur = M::lifetime(L, s);
   if (gt_nonneg(dur, t)) {  // both >= 0
-    if (bernoulli<R>(s, (R)md.rho)) {
+    if (bernoulli<R>(s, md.c((R)0).rho)) {
       L.lnp3 = neg_inf<R>();
       L.pc = end_block;
       return;
@@ -536,11 +562,11 @@ struct TreeModel {
     switch (b) {
       case PRIOR: {
         if (md.fixed_rates) {
-          L.lam = (R)md.lambda_fixed;
-          L.mu = (R)md.mu_fixed;
+          L.lam = md.c((R)0).lambda_fixed;
+          L.mu = md.c((R)0).mu_fixed;
         } else {
-          L.lam = gamma1<R>(s, (R)md.lambda_scale);
-          L.mu = gamma1<R>(s, (R)md.mu_scale);
+          L.lam = gamma1<R>(s, md.c((R)0).lambda_scale);
+          L.mu = gamma1<R>(s, md.c((R)0).mu_scale);
         }
         if (RS) {
           S.st<R>(0, i, N) = L.lam;  // the root's rate, pending for its children
@@ -548,7 +574,7 @@ struct TreeModel {
         } else {
           L.loglam = lg(L.lam, s);
         }
-        L.logw = L.logw + (R)md.corr;
+        L.logw = L.logw + md.c((R)0).corr;
         L.pc = BRANCH;
         L.ckpt = true;
         return;
@@ -574,16 +600,16 @@ struct TreeModel {
             mult = (R)md.fixed_mult[v];
           } else {
             Stream sm{s.k0, s.k1, s.n, s.k, 0u, 2u, s.tab};
-            mult = lognormal<R>(sm, (R)md.sigma);
+            mult = lognormal<R>(sm, md.c((R)0).sigma);
           }
           lam = lam_p * mult;
         }
         L.lam_b = lam;
-        L.start = (R)br.start;
-        L.stop = (R)br.stop;
+        L.start = br.begin_at((R)0);
+        L.stop = br.end_at((R)0);
         const R dt = L.start - L.stop;
         L.lnp1 = -L.mu * dt;
-        L.lnp2 = L.internal ? (RS ? lg(lam, s) : L.loglam) : (R)md.log_rho;
+        L.lnp2 = L.internal ? (RS ? lg(lam, s) : L.loglam) : md.c((R)0).log_rho;
         L.n_top = poisson<R>(s, lam * dt);
         if (L.n_top > 0 && L.mu > (R)0) L.inv_mu = (R)1 / L.mu;
         L.lnp3 = (R)0;
@@ -701,10 +727,10 @@ struct TreeDsModel {
     switch (b) {
       case PRIOR: {
         L.al = (R)1.0;
-        L.bl = (R)1.0 / (R)md.lambda_scale;
+        L.bl = (R)1.0 / md.c((R)0).lambda_scale;
         L.am = (R)1.0;
-        L.bm = (R)1.0 / (R)md.mu_scale;
-        L.logw = L.logw + (R)md.corr;
+        L.bm = (R)1.0 / md.c((R)0).mu_scale;
+        L.logw = L.logw + md.c((R)0).corr;
         L.pc = BRANCH;
         L.ckpt = true;
         return;
@@ -712,8 +738,8 @@ struct TreeDsModel {
       case BRANCH: {
         const BranchRec br = load_branch(md.branch, k);
         L.v = br.v;
-        L.start = (R)br.start;
-        L.stop = (R)br.stop;
+        L.start = br.begin_at((R)0);
+        L.stop = br.end_at((R)0);
         const R dt = L.start - L.stop;
         L.lnp1 = -L.am * m_log1p(dt / L.bm);
         L.bm = L.bm + dt;
@@ -721,7 +747,7 @@ struct TreeDsModel {
           L.lnp2 = lg(L.al / L.bl, s);
           L.al = L.al + (R)1.0;
         } else {
-          L.lnp2 = (R)md.log_rho;
+          L.lnp2 = md.c((R)0).log_rho;
         }
         L.n_top = neg_binomial<R>(s, L.al, L.bl, dt);
         L.al = L.al + (R)L.n_top;

@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(TPB + (CL ? 32 : 0), 1) small_run_kernel(const
     int alive = 0;
     if (valid) {
       M::store(L, Sn, i, N);
-      lw = (double)L.logw;
+      lw = widen(L.logw);
       A.logw[i] = lw;
       alive = L.pc != PC_STOP;
     }
@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(TPB + (CL ? 32 : 0), 1) small_run_kernel(const
     // the tile's weights: a warp is a tile, so its reference is the warp's
     long long ef = 0;
     const double Mw = warp_max_key(lw);
-    const int kt = Mw == -INFINITY ? kDeadTile : tile_exponent_fast(Mw);
+    const int kt = is_neg_inf(Mw) ? kDeadTile : tile_exponent_fast(Mw);
     if (valid && kt != kDeadTile) {
       if (kt > -2048 && kt < 2048) {
         ef = weight_fix54(lw, kt, ref_q58_lo(kt), A.md.tab);

@@ -452,7 +452,7 @@ __device__ __forceinline__ void step_tile(const RunDev& A, const int t, const in
   int alive = 0;
   if (valid) {
     M::store(L, Sn, i, N);
-    lw = (double)L.logw;
+    lw = widen(L.logw);
     A.logw[i] = lw;
     alive = L.pc != PC_STOP;
   }
@@ -464,7 +464,7 @@ __device__ __forceinline__ void step_tile(const RunDev& A, const int t, const in
   // tile's integer running sum E_j (the next segment's search keys).
   long long ef = 0;
   const double Mw = warp_max_key(lw);
-  const int kw = Mw == -INFINITY ? kDeadTile : tile_exponent_fast(Mw);
+  const int kw = is_neg_inf(Mw) ? kDeadTile : tile_exponent_fast(Mw);
   if (valid && kw != kDeadTile) {
     // (an FP32 log-weight is exact as a double, so both precisions share the
     // normaliser's integer-pipe exponential)
