@@ -107,7 +107,7 @@ PROBE_ITERS = {0: 2000, 1: 100000, 2: 20000, 3: 50000, 4: 5000}
 
 
 # the segment kernel's sources (the standalone resampling kernels are not among them)
-KERNEL_SOURCES = ("smc_engine.cu", "smc_step.cuh", "smc_waves_kind.cu", "smc_engine.h",
+KERNEL_SOURCES = ("smc_engine.cu", "smc_step.cuh", "smc_waves.cuh", "smc_engine.h",
                   "smc_models.cuh", "smc_device.cuh", "smc_combine.cuh")
 # the standalone resampling kernels' sources
 RS_SOURCES = ("smc_prims.cu", "smc_device.cuh", "smc_combine.cuh")

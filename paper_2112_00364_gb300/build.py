@@ -22,8 +22,9 @@ INCLUDE = PKG.parent / "include"
 BUILD = PKG / "_build"
 LIB = PKG / "libsmc.so"
 LIB_DEBUG = PKG / "libsmc_debug.so"
-SOURCES = ["smc_engine.cu", "smc_waves_kind.cu", "smc_waves_tree.cu", "smc_waves_ds.cu",
-           "smc_waves_seir.cu", "smc_small.cu", "smc_prims.cu", "smc_server.cu", "smc_probe.cu"]
+SOURCES = ["smc_waves_kind.cu", "smc_waves_kind_f.cu", "smc_waves_tree.cu", "smc_waves_tree_f.cu",
+           "smc_waves_ds.cu", "smc_waves_ds_f.cu", "smc_waves_seir.cu", "smc_waves_seir_f.cu",
+           "smc_engine.cu", "smc_small.cu", "smc_prims.cu", "smc_server.cu", "smc_probe.cu"]
 GENCODE = "arch=compute_103a,code=sm_103a"
 
 

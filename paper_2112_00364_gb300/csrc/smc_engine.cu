@@ -586,25 +586,34 @@ cudaError_t ChainStreams::join(cudaStream_t main, int chains) {
 }
 
 namespace {
-cudaError_t launch_chain(const WavePlan& W, const WaveChain& c, int precision, cudaStream_t st,
-                         unsigned wave) {
-  const bool alone = W.chains.size() == 1;
+template <typename R>
+cudaError_t launch_chain(const WaveChain& c, const RunDev* runs, cudaStream_t st, unsigned wave,
+                         bool alone, bool dense) {
   switch (c.kind) {
-    case SMC_MODEL_LG: return launch_kind<SMC_MODEL_LG>(c, W.runs, precision, st, wave, alone);
-    case SMC_MODEL_CRBD: return launch_kind<SMC_MODEL_CRBD>(c, W.runs, precision, st, wave, alone);
-    case SMC_MODEL_RATESHIFT: return launch_kind<SMC_MODEL_RATESHIFT>(c, W.runs, precision, st, wave, alone);
-    case SMC_MODEL_SEIR: return launch_kind<SMC_MODEL_SEIR>(c, W.runs, precision, st, wave, alone);
-    case SMC_MODEL_CRBD_DS: return launch_kind<SMC_MODEL_CRBD_DS>(c, W.runs, precision, st, wave, alone);
-    default: return launch_kind<SMC_MODEL_GEOMETRIC>(c, W.runs, precision, st, wave, alone);
+    case SMC_MODEL_LG: return launch_kind<SMC_MODEL_LG, R>(c, runs, st, wave, alone, dense);
+    case SMC_MODEL_CRBD: return launch_kind<SMC_MODEL_CRBD, R>(c, runs, st, wave, alone, dense);
+    case SMC_MODEL_RATESHIFT:
+      return launch_kind<SMC_MODEL_RATESHIFT, R>(c, runs, st, wave, alone, dense);
+    case SMC_MODEL_SEIR: return launch_kind<SMC_MODEL_SEIR, R>(c, runs, st, wave, alone, dense);
+    case SMC_MODEL_CRBD_DS: return launch_kind<SMC_MODEL_CRBD_DS, R>(c, runs, st, wave, alone, dense);
+    default: return launch_kind<SMC_MODEL_GEOMETRIC, R>(c, runs, st, wave, alone, dense);
   }
 }
 }  // namespace
 
 cudaError_t launch_wave(const WavePlan& W, int precision, cudaStream_t st, unsigned wave,
                         const ChainStreams* streams) {
+  const bool alone = W.chains.size() == 1;
+  // whether the wave's CTAs exceed what runs at once at 768 threads an SM
+  long long threads = 0;
+  for (const WaveChain& c : W.chains) threads += (long long)c.n_ctas * (32 << c.bucket);
+  const bool dense = threads > (long long)kSms * 768;
   for (size_t i = 0; i < W.chains.size(); ++i) {
-    const cudaError_t e = launch_chain(W, W.chains[i], precision,
-                                       streams ? streams->at((int)i) : st, wave);
+    const WaveChain& c = W.chains[i];
+    const cudaStream_t s = streams ? streams->at((int)i) : st;
+    const cudaError_t e = precision == SMC_PREC_FP32
+                              ? launch_chain<float>(c, W.runs, s, wave, alone, dense)
+                              : launch_chain<double>(c, W.runs, s, wave, alone, dense);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -203,10 +203,11 @@ size_t fill_plan(const std::vector<RunDev>& runs, char* host, void* dev, WavePla
 // One wave: every chain's launch, on `st`, or each on its own stream with `streams`.
 cudaError_t launch_wave(const WavePlan& W, int precision, cudaStream_t st, unsigned wave,
                         const ChainStreams* streams = nullptr);
-// (alone: no other chain runs beside this one)
-template <int KIND>
-cudaError_t launch_kind(const WaveChain& c, const RunDev* runs, int precision, cudaStream_t st,
-                        unsigned wave, bool alone);
+// (alone: no other chain runs beside this one; dense: the wave's CTAs do not all fit at
+// once, resident_threads())
+template <int KIND, typename R>
+cudaError_t launch_kind(const WaveChain& c, const RunDev* runs, cudaStream_t st, unsigned wave,
+                        bool alone, bool dense);
 smc_status collect_run(const smc_model_s* m, const smc_run_cfg* c, const Layout& Ly, char* ws,
                        const RunDev& A, const RunState& hrs, smc_result* r, cudaStream_t cs);
 smc_status check_cfg(const smc_model_s* m, const smc_run_cfg* c);

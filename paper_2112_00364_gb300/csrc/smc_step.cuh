@@ -566,7 +566,7 @@ __device__ __forceinline__ void step_tile(const RunDev& A, const int t, const in
   }
 }
 
-constexpr unsigned kEarlyCtas = 152;  // GB300's SMs
+constexpr unsigned kSms = 152;  // GB300's
 
 // The block table of a model kind.
 template <int KIND, typename R>
@@ -584,15 +584,31 @@ struct ModelOf<SMC_MODEL_SEIR, R> { using type = SeirModel<R>; };
 template <typename R>
 struct ModelOf<SMC_MODEL_CRBD_DS, R> { using type = TreeDsModel<R>; };
 
+// Resident threads an SM that a wave kernel is bounded to.  A grid that fits at once
+// with 768 (three CTAs of 256, 80 registers) is bound by each CTA's latency and wants
+// the registers; a dense one by how many warps there are to switch between, and
+// takes fewer.  us a wave, sparse / dense form: CRBD FP32 65,536 particles (456 CTAs)
+// 16.4 / 19.8, 2^20 131.5 / 115.6, rate-shift FP32 2^20 145 / 126, CRBD FP64 65,536
+// 20.5 / 23.1, 2^20 184 / 174, linear-Gaussian FP64 2^20 95 / 84, 23,171 7.23 / 7.43; a
+// batch of 512 FP32 runs 152 / 128 ms with its CRBD runs in either form.  (FP32 waves
+// of 2^20 linear-Gaussian particles stay at 1,024: 72 us, 75 with 1,280.)
+template <typename R, int KIND>
+__host__ __device__ constexpr int resident_threads(int tpb, bool dense) {
+  if (!dense) return 768;
+  if (sizeof(R) == 8 || (KIND == SMC_MODEL_LG && tpb == 256)) return 1024;
+  return 1280;
+}
+__host__ __device__ constexpr int min_ctas(int threads, int tpb) {
+  return threads / tpb < 32 ? threads / tpb : 32;
+}
+
 // One wave: CTA b runs tile cta_map[b].y of run cta_map[b].x, segment
 // k = wave - start_wave of that run.
-// 768 resident threads per SM (three 256-thread CTAs: the grid sizing of
-// tile_for) bounds the kernel to 85 registers per thread.
 // KIND: the model (SMC_MODEL_*) that every run of the launch runs.
-template <typename R, int TPB, int KIND>
-__global__ void __launch_bounds__(TPB, (sizeof(R) == 4 ? 1024 : 768) / TPB) wave_kernel(const RunDev* __restrict__ runs,
-                                                   const int2* __restrict__ cta_map, unsigned wave,
-                                                   int alone) {
+template <typename R, int TPB, int KIND, bool DENSE>
+__global__ void __launch_bounds__(TPB, min_ctas(resident_threads<R, KIND>(TPB, DENSE), TPB))
+    wave_kernel(const RunDev* __restrict__ runs, const int2* __restrict__ cta_map, unsigned wave,
+                int alone) {
   __shared__ __align__(16) RunDev sr;
   __shared__ StepShared<TPB> S;
   const int2 rt = cta_map[blockIdx.x];
@@ -609,7 +625,7 @@ __global__ void __launch_bounds__(TPB, (sizeof(R) == 4 ? 1024 : 768) / TPB) wave
   // (a lone chain's grid of at most one CTA an SM leaves room for the next wave's
   // CTAs beside its own: those then start at once, and what they do before the wait
   // is hidden.  Beside other chains they would take places from them)
-  const bool early = alone && gridDim.x <= kEarlyCtas;
+  const bool early = alone && gridDim.x <= kSms;
   if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int k = (int)(wave - sr.start_wave);  // wraps correctly past 2^32 waves
   using M = typename ModelOf<KIND, R>::type;
@@ -633,7 +649,7 @@ __global__ void __launch_bounds__(TPB, (sizeof(R) == 4 ? 1024 : 768) / TPB) wave
 
 // One bucket of a wave, launched so that it may begin before the kernel ahead
 // of it in the stream has finished (wave_kernel waits for it where it must).
-template <typename R, int TPB, int KIND>
+template <typename R, int TPB, int KIND, bool DENSE>
 cudaError_t launch_pdl(const RunDev* runs, const int2* map, int n, cudaStream_t st, unsigned wave,
                        bool alone) {
   cudaLaunchConfig_t cfg = {};
@@ -646,17 +662,17 @@ cudaError_t launch_pdl(const RunDev* runs, const int2* map, int n, cudaStream_t 
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, wave_kernel<R, TPB, KIND>, runs, map, wave, alone ? 1 : 0);
+  return cudaLaunchKernelEx(&cfg, wave_kernel<R, TPB, KIND, DENSE>, runs, map, wave, alone ? 1 : 0);
 }
 
-template <typename R, int KIND>
+template <typename R, int KIND, bool DENSE>
 cudaError_t launch_bucket(int b, const RunDev* runs, const int2* map, int n, cudaStream_t st,
                           unsigned wave, bool alone) {
   switch (b) {
-    case 0: return launch_pdl<R, 32, KIND>(runs, map, n, st, wave, alone);
-    case 1: return launch_pdl<R, 64, KIND>(runs, map, n, st, wave, alone);
-    case 2: return launch_pdl<R, 128, KIND>(runs, map, n, st, wave, alone);
-    default: return launch_pdl<R, 256, KIND>(runs, map, n, st, wave, alone);
+    case 0: return launch_pdl<R, 32, KIND, DENSE>(runs, map, n, st, wave, alone);
+    case 1: return launch_pdl<R, 64, KIND, DENSE>(runs, map, n, st, wave, alone);
+    case 2: return launch_pdl<R, 128, KIND, DENSE>(runs, map, n, st, wave, alone);
+    default: return launch_pdl<R, 256, KIND, DENSE>(runs, map, n, st, wave, alone);
   }
 }
 

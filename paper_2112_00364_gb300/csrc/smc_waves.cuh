@@ -3,7 +3,7 @@
 // wave after wave): each kernel holds one model's block table only, so its code
 // and registers (one kernel dispatching on each run's model spilled 250 bytes a
 // thread at the 64 registers of FP32 particles: 150 us instead of 143 a rate-shift
-// wave of 2^20).  Each model is compiled in a translation unit of its own.
+// wave of 2^20).  Models and precisions have translation units of their own.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -12,12 +12,11 @@
 
 namespace smc {
 
-template <int KIND>
-cudaError_t launch_kind(const WaveChain& c, const RunDev* runs, int precision, cudaStream_t st,
-                        unsigned wave, bool alone) {
-  return precision == SMC_PREC_FP32
-             ? launch_bucket<float, KIND>(c.bucket, runs, c.map, c.n_ctas, st, wave, alone)
-             : launch_bucket<double, KIND>(c.bucket, runs, c.map, c.n_ctas, st, wave, alone);
+template <int KIND, typename R>
+cudaError_t launch_kind(const WaveChain& c, const RunDev* runs, cudaStream_t st, unsigned wave,
+                        bool alone, bool dense) {
+  return dense ? launch_bucket<R, KIND, true>(c.bucket, runs, c.map, c.n_ctas, st, wave, alone)
+               : launch_bucket<R, KIND, false>(c.bucket, runs, c.map, c.n_ctas, st, wave, alone);
 }
 
 }  // namespace smc

@@ -1,9 +1,9 @@
-// smc_waves_ds.cu -- the wave kernels of the delayed-sampling CRBD (smc_waves.cuh).
+// smc_waves_ds.cu -- the wave kernels of the delayed-sampling CRBD, FP64 (smc_waves.cuh).
 #include "smc_waves.cuh"
 
 namespace smc {
 
-template cudaError_t launch_kind<SMC_MODEL_CRBD_DS>(const WaveChain&, const RunDev*, int, cudaStream_t, unsigned,
-                                              bool);
+template cudaError_t launch_kind<SMC_MODEL_CRBD_DS, double>(const WaveChain&, const RunDev*, cudaStream_t, unsigned,
+    bool, bool);
 
 }  // namespace smc

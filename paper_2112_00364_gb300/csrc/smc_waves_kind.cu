@@ -1,11 +1,11 @@
-// smc_waves_kind.cu -- the wave kernels of the linear-Gaussian and CRBD models (smc_waves.cuh).
+// smc_waves_kind.cu -- the wave kernels of the linear-Gaussian and CRBD models, FP64 (smc_waves.cuh).
 #include "smc_waves.cuh"
 
 namespace smc {
 
-template cudaError_t launch_kind<SMC_MODEL_LG>(const WaveChain&, const RunDev*, int, cudaStream_t, unsigned,
-                                              bool);
-template cudaError_t launch_kind<SMC_MODEL_CRBD>(const WaveChain&, const RunDev*, int, cudaStream_t, unsigned,
-                                              bool);
+template cudaError_t launch_kind<SMC_MODEL_LG, double>(const WaveChain&, const RunDev*, cudaStream_t, unsigned,
+    bool, bool);
+template cudaError_t launch_kind<SMC_MODEL_CRBD, double>(const WaveChain&, const RunDev*, cudaStream_t, unsigned,
+    bool, bool);
 
 }  // namespace smc

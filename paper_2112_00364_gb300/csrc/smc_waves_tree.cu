@@ -1,11 +1,13 @@
-// smc_waves_tree.cu -- the wave kernels of the rate-shift model and the geometric program (smc_waves.cuh).
+// smc_waves_tree.cu -- the wave kernels of the rate-shift model, FP64, and the geometric program (smc_waves.cuh).
 #include "smc_waves.cuh"
 
 namespace smc {
 
-template cudaError_t launch_kind<SMC_MODEL_RATESHIFT>(const WaveChain&, const RunDev*, int, cudaStream_t, unsigned,
-                                              bool);
-template cudaError_t launch_kind<SMC_MODEL_GEOMETRIC>(const WaveChain&, const RunDev*, int, cudaStream_t, unsigned,
-                                              bool);
+template cudaError_t launch_kind<SMC_MODEL_RATESHIFT, double>(const WaveChain&, const RunDev*, cudaStream_t, unsigned,
+    bool, bool);
+template cudaError_t launch_kind<SMC_MODEL_GEOMETRIC, double>(const WaveChain&, const RunDev*, cudaStream_t, unsigned,
+    bool, bool);
+template cudaError_t launch_kind<SMC_MODEL_GEOMETRIC, float>(const WaveChain&, const RunDev*, cudaStream_t, unsigned,
+    bool, bool);
 
 }  // namespace smc
