@@ -1245,20 +1245,24 @@ extern "C" smc_status smc_run(smc_model_t m, const smc_run_cfg* c, smc_result* r
     if (m->pin_out) cudaFreeHost(m->pin_out);
     m->pin_out = nullptr;
     m->pin_out_bytes = 0;
-    SMC_CUDA_TRY(cudaMallocHost(&m->pin_out, pin_need));
-    m->pin_out_bytes = pin_need;
+    if (cudaMallocHost(&m->pin_out, pin_need) == cudaSuccess)
+      m->pin_out_bytes = pin_need;
+    else
+      cudaGetLastError();  // pageable memory instead
   }
-  char* pinned_block = m->pin_out + align_up(sizeof(RunState), 256);
+  std::vector<char> pageable(m->pin_out ? 0 : pin_need);
+  char* out_at = m->pin_out ? m->pin_out : pageable.data();
+  char* block_at = out_at + align_up(sizeof(RunState), 256);
   if (!host)
     launch_collect(collect_device(m, c, Ly, runs[0], r), cs);
   else if (staged)
     launch_collect(collect_staged(m, c, Ly, runs[0], ws + Ly.stage), cs);
   SMC_CUDA_TRY(cudaGetLastError());
-  if (staged) SMC_CUDA_TRY(cudaMemcpyAsync(pinned_block, ws + Ly.stage, block, cudaMemcpyDeviceToHost, cs));
-  SMC_CUDA_TRY(cudaMemcpyAsync(m->pin_out, runs[0].rs, sizeof(RunState), cudaMemcpyDeviceToHost, cs));
+  if (staged) SMC_CUDA_TRY(cudaMemcpyAsync(block_at, ws + Ly.stage, block, cudaMemcpyDeviceToHost, cs));
+  SMC_CUDA_TRY(cudaMemcpyAsync(out_at, runs[0].rs, sizeof(RunState), cudaMemcpyDeviceToHost, cs));
   SMC_CUDA_TRY(cudaStreamSynchronize(cs));
   RunState hrs;
-  std::memcpy(&hrs, m->pin_out, sizeof(RunState));
+  std::memcpy(&hrs, out_at, sizeof(RunState));
   float ms = 0.f;
   cudaEventElapsedTime(&ms, m->ev0, m->ev1);
   if (host && !staged) {
@@ -1266,7 +1270,7 @@ extern "C" smc_status smc_run(smc_model_t m, const smc_run_cfg* c, smc_result* r
     SMC_CUDA_TRY(cudaStreamSynchronize(cs));
   } else {
     fill_counters(hrs, r->counters);
-    if (staged) unstage(m, c->n_particles, hrs.n_segments, pinned_block, r);
+    if (staged) unstage(m, c->n_particles, hrs.n_segments, block_at, r);
   }
   r->counters.device_ms = ms;
   r->counters.kernel_launches = launched;
@@ -1344,10 +1348,16 @@ extern "C" smc_status smc_run_batch(const smc_model_t* ms, const smc_run_cfg* cf
   WavePlan W;
   std::vector<char> staging;
   if ((st = upload_wave(runs, (char*)ws + meta_off, cs, &W, &staging))) return st;
-  cudaEvent_t e0, e1;
-  SMC_CUDA_TRY(cudaEventCreate(&e0));
-  SMC_CUDA_TRY(cudaEventCreate(&e1));
-  SMC_CUDA_TRY(cudaEventRecord(e0, cs));
+  struct Events {
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    ~Events() {
+      if (e0) cudaEventDestroy(e0);
+      if (e1) cudaEventDestroy(e1);
+    }
+  } ev;
+  SMC_CUDA_TRY(cudaEventCreate(&ev.e0));
+  SMC_CUDA_TRY(cudaEventCreate(&ev.e1));
+  SMC_CUDA_TRY(cudaEventRecord(ev.e0, cs));
   int launched = 0;
   double kms = 0.0;
   GraphCache graph;
@@ -1359,11 +1369,9 @@ extern "C" smc_status smc_run_batch(const smc_model_t* ms, const smc_run_cfg* cf
                    graphed ? &graph : nullptr, fan ? &streams : nullptr);
   if (st) {
     graph_cache_clear(&graph);
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
     return st;
   }
-  SMC_CUDA_TRY(cudaEventRecord(e1, cs));
+  SMC_CUDA_TRY(cudaEventRecord(ev.e1, cs));
   for (size_t j0 = 0; j0 < jobs.size(); j0 += 65535) {  // (grid rows)
     const unsigned rows = (unsigned)std::min<size_t>(65535, jobs.size() - j0);
     collect_kernel<<<dim3(32, rows), 256, 0, cs>>>((const CollectJob*)((char*)ws + job_off) + j0);
@@ -1376,9 +1384,7 @@ extern "C" smc_status smc_run_batch(const smc_model_t* ms, const smc_run_cfg* cf
   graph_cache_clear(&graph);  // its launch has completed
   if (se != cudaSuccess) return cuda_fail(se, "cudaStreamSynchronize(batch)");
   float msec = 0.f;
-  cudaEventElapsedTime(&msec, e0, e1);
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
+  cudaEventElapsedTime(&msec, ev.e0, ev.e1);
   for (int q = 0; q < n_runs; ++q) {
     if (res[q].where != SMC_MEM_HOST)
       fill_counters(h[q], res[q].counters);
