@@ -196,7 +196,8 @@ typedef struct {
   int64_t n_limit;          /* particle-segments killed by the call limit */
   double device_ms;         /* GPU time of the run (CUDA events) */
   double kernel_ms;         /* time_kernels = 1: summed duration of the segment-kernel launches */
-  int32_t kernel_launches;  /* segment-kernel launches of the run (one per wave and CTA size) */
+  int32_t kernel_launches;  /* segment-kernel launches of the run (one per wave, model and
+                               CTA size) */
   int32_t n_ess_near;       /* ess_threshold > 0: checkpoints whose ESS lay within 1e-9 of tau N */
   smc_status status;        /* this run's own status (0, SMC_WKILLED, SMC_EDEGENERATE,
                                SMC_ESTEPLIMIT) */
@@ -244,8 +245,7 @@ typedef struct {
  * clamp(ceil(N / slots), tile_min, tile_max).  Since the tiling fixes how the
  * weights are rounded to their tile's reference, a run gives the same bits
  * alone, batched and served under one table.  The built-in table is data
- * written by the library's autotuner (sweeps of candidate bands timed on a
- * GB300). */
+ * from sweeps of sizes and tiles timed on a GB300. */
 typedef struct {
   int64_t n_max;     /* the band holds runs of N <= n_max (the last band: >= SMC_MAX_PARTICLES) */
   int32_t slots;     /* >= 1 */
@@ -296,8 +296,8 @@ smc_status smc_workspace_bytes(smc_model_t m, const smc_run_cfg *c, size_t *byte
 smc_status smc_run(smc_model_t m, const smc_run_cfg *c, smc_result *r, void *stream);
 
 /* Run n_runs independent SMC runs (Algorithm 1 each) in one sequence of waves:
- * every wave advances every unfinished run by one segment, all runs' tiles in the
- * same kernel launches, each run resampled by its own last-arriving CTA, so
+ * every wave advances every unfinished run by one segment, the tiles of all runs of
+ * one model and CTA size in one kernel launch, each run resampled on its own, so
  * uneven runs fill the GPU together instead of one after another.  ms[q],
  * cfgs[q], res[q] describe run q exactly as for smc_run (cfg.workspace is
  * ignored: the batch takes stream-ordered device memory for the call and returns

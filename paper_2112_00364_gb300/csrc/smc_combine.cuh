@@ -305,16 +305,6 @@ __device__ __forceinline__ Q64 q_add(Q64 a, Q64 b) {
   return r;
 }
 
-// a - b for a >= b
-__device__ __forceinline__ Q64 q_sub(Q64 a, Q64 b) {
-  Q64 r;
-  r.lo = a.lo - b.lo;
-  r.hi = a.hi - b.hi - (a.lo < b.lo ? 1ull : 0ull);
-  return r;
-}
-
-__device__ __forceinline__ bool q_lt(Q64 a, Q64 b) { return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo); }
-
 // One digit of a long division in base 2^32: floor(num / N) and the remainder
 // for num < N 2^32 and 1 <= N < 2^31, from the per-run reciprocal
 // R = floor((2^64 - 1) / N).  2^64 / N - R < 2, so num R 2^-64 lies within one

@@ -744,20 +744,13 @@ __device__ __forceinline__ R uniform01(Stream& s) {
 }
 
 // Box-Muller, cosine branch: sqrt(-2 ln u1) * cos(2 pi u2)
-__device__ __forceinline__ double log_first_uniform(const Block4& b, const Stream& s, double) {
-  return log_unif53(((unsigned long long)b.w1 << 32) | b.w0, s.tab);
-}
-__device__ __forceinline__ float log_first_uniform(const Block4& b, const Stream&, float) {
-  return f32_log(Unif<float>::first(b));
-}
-
 template <typename R>
 __device__ __forceinline__ R normal01(Stream& s);
 template <>
 __device__ __forceinline__ float normal01<float>(Stream& s) {
   const Block4 b = s.next();
   const float u2 = Unif<float>::second(b);
-  const float rad = m_sqrt(-2.0f * log_first_uniform(b, s, 0.0f));
+  const float rad = m_sqrt(-2.0f * f32_log(Unif<float>::first(b)));
   return rad * cos_2pi(u2);
 }
 
@@ -1379,40 +1372,6 @@ __device__ __forceinline__ int neg_binomial<double>(Stream& s, double alpha, dou
 }
 
 // ---- warp / block primitives (integer, deterministic association order) ----
-// Block max of an int over TPB threads; every thread gets the result.
-template <int TPB>
-__device__ __forceinline__ int block_max_int(int v, int* sh) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  v = __reduce_max_sync(0xffffffffu, v);
-  __syncthreads();
-  if (lane == 0) sh[wid] = v;
-  __syncthreads();
-  int r = sh[0];
-#pragma unroll
-  for (int w = 1; w < TPB / 32; ++w) r = max(r, sh[w]);
-  return r;
-}
-
-// Block inclusive prefix max of int64 keys over TPB threads.  `sh` >= TPB/32
-// long longs.  Non-negative doubles order like their bit patterns, so this is
-// also the prefix max of such doubles, on the integer pipes.
-template <int TPB>
-__device__ __forceinline__ long long block_incl_max_i64(long long v, long long* sh) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const long long t = __shfl_up_sync(0xffffffffu, v, o);
-    if (lane >= o) v = max(v, t);
-  }
-  if (TPB > 32) {
-    __syncthreads();
-    if (lane == 31) sh[wid] = v;
-    __syncthreads();
-    for (int w = 0; w < wid; ++w) v = max(v, sh[w]);
-  }
-  return v;
-}
-
 // Order-preserving int64 key of a double (not NaN): for x >= 0 its bits, for
 // x < 0 its bits with the magnitude bits flipped; max of keys = key of max.
 __device__ __forceinline__ long long order_key(double x) {
@@ -1456,22 +1415,6 @@ __device__ __forceinline__ long long to_fix54(double x) {
   return (m + (1ll << (rs - 1))) >> rs;
 }
 
-// floor(x * 2^54) for any x: -1 below zero, LLONG_MAX from 2^9 up (above every
-// tile sum), integer operations only.
-__device__ __forceinline__ long long floor_fix54(double x) {
-  const long long b = __double_as_longlong(x);
-  if ((b & 0x7FFFFFFFFFFFFFFFll) == 0) return 0;  // +-0
-  if (b < 0) return -1;
-  const int e = (int)(b >> 52);
-  if (e == 0) return 0;
-  if (e >= 1023 + 9) return 0x7FFFFFFFFFFFFFFFll;
-  const long long m = (b & 0x000FFFFFFFFFFFFFll) | 0x0010000000000000ll;
-  const int sh = e - (1075 - kFixBits);
-  if (sh >= 0) return m << sh;
-  const int rs = -sh;
-  return rs >= 63 ? 0 : (m >> rs);
-}
-
 // Block inclusive scan of int64 over TPB threads (exact).  `sh` >= TPB/32 long longs.
 template <int TPB>
 __device__ __forceinline__ long long block_incl_scan_i64(long long v, long long* sh) {
@@ -1497,25 +1440,6 @@ __device__ __forceinline__ long long block_incl_scan_i64(long long v, long long*
   }
   __syncthreads();
   return wid > 0 ? sh[wid] + v : v;
-}
-
-// Block max of doubles (no NaN) through their order keys: integer shuffles
-// and compares only.  Every thread gets the result.  `sh` >= TPB/32 long longs.
-template <int TPB>
-__device__ __forceinline__ double block_max_key(double x, long long* sh) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  long long v = order_key(x);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-  if (TPB > 32) {
-    __syncthreads();
-    if (lane == 0) sh[wid] = v;
-    __syncthreads();
-    v = sh[0];
-#pragma unroll
-    for (int w = 1; w < TPB / 32; ++w) v = max(v, sh[w]);
-  }
-  return from_order_key(v);
 }
 
 }  // namespace smc

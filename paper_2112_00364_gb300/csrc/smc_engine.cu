@@ -2,7 +2,8 @@
 // (SMC over PCFGs) in the RootPPL loop order of Section 3.3.
 //
 // Execution is organised in waves.  One wave advances every resident run by
-// one segment; it is one launch of wave_kernel per block-size bucket.  Each
+// one segment; it is one launch of wave_kernel per model and CTA size (a chain;
+// the chains of a batch run on streams of their own, from wave to wave).  Each
 // CTA of a wave owns one tile (a run and a contiguous slice of its particles,
 // one particle per thread):
 //   prologue  (segment k > 0) the previous segment's tiles combined into exact
@@ -31,11 +32,10 @@
 // sums.  A run stops after the segment in which every particle reached b_stop
 // (no resampling after it); its later CTAs return at once.
 //
-// A run's tile size depends only on its N (tile = ceil(N / 456) clamped to
-// 32..256, 456 = 152 SMs x 3 CTAs), so a run gives the same bits alone and in a
-// batch.  The CTA size of a run is the smallest of 32/64/128/256 threads that
-// holds its tile; runs of different CTA sizes are launched as separate kernels
-// of the same wave.
+// A run's tile size depends only on its N (a table of N bands,
+// smc_tile_table.inc), so a run gives the same bits alone and in a batch.  The CTA
+// size of a run is the smallest of 32/64/128/256 threads that holds its tile.
+// After its last wave one kernel (collect_kernel) writes all of a run's outputs.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -3,7 +3,8 @@
 // parity hooks, and the library's error plumbing.
 //
 // smc_resample (parallel systematic resampling, three launches chained by
-// programmatic dependent launch), in the segment kernel's integer arithmetic
+// programmatic dependent launch; two up to 456 tiles, where every CTA of pass 3
+// combines the records itself), in the segment kernel's integer arithmetic
 // (smc_combine.cuh):
 //   1. rs_tile_reduce (persistent): per tile of 4096 weights, the power-of-two
 //      reference k_t from the largest high word of its log-weights (k_t ln 2 at

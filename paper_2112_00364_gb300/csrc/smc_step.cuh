@@ -1,6 +1,5 @@
 // smc_step.cuh -- one tile of one run for one segment: the body of every
-// segment kernel (the wave kernel of smc_engine.cu and the single-CTA kernel of
-// smc_small.cu).  Algorithm 1 in the RootPPL loop order of Section 3.3: the
+// segment kernel (wave_kernel below and the one-launch kernels of smc_small.cu).  Algorithm 1 in the RootPPL loop order of Section 3.3: the
 // previous segment's tiles combined into exact integer offsets, the log-Z
 // increment and the resampling decision; the systematic search and the
 // particle duplication fused into the load; blocks run to the next checkpoint;
@@ -30,14 +29,14 @@ __device__ __forceinline__ void warp_add_u64(unsigned long long* dst, unsigned l
   if ((threadIdx.x & 31) == 0 && v) atomicAdd(dst, v);
 }
 
-// Finish segment k-1 of the run from its combined offsets (one thread):
-// log Z += k_max ln 2 + (log S - log N) with S = S_units U, the increment
-// record, and the end of the run.  Returns whether segment k runs.
 // Whether to resample after checkpoint k-1 (the same in every CTA: c is).
 __device__ __forceinline__ bool decide_resample(const RunDev& A, const Combined& c) {
   return !A.ess || c.ess < A.ess_target;
 }
 
+// Finish segment k-1 of the run from its combined offsets (one thread):
+// log Z += k_max ln 2 + (log S - log N) with S = S_units U, the increment
+// record, and the end of the run.  Returns whether segment k runs.
 __device__ __forceinline__ bool finish_segment(const RunDev& A, int k, const Combined& c,
                                                bool resample) {
   RunState* rs = A.rs;
