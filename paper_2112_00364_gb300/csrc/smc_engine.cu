@@ -30,7 +30,8 @@
 // common unit with a coarsening G that keeps S in [2^61, 2^62]: the offsets O_t
 // and S are exact integers, so the result does not depend on the order of the
 // sums.  A run stops after the segment in which every particle reached b_stop
-// (no resampling after it); its later CTAs return at once.
+// (no resampling after it); its later CTAs return at once (a batch's waves leave out
+// those that its length or step limit already rules out).
 //
 // A run's tile size depends only on its N (a table of N bands,
 // smc_tile_table.inc), so a run gives the same bits alone and in a batch.  The CTA
@@ -44,6 +45,8 @@
 #include <iterator>
 #include <mutex>
 #include <new>
+#include <numeric>
+#include <utility>
 #include <vector>
 
 #include "smc_device.cuh"
@@ -587,33 +590,36 @@ cudaError_t ChainStreams::join(cudaStream_t main, int chains) {
 
 namespace {
 template <typename R>
-cudaError_t launch_chain(const WaveChain& c, const RunDev* runs, cudaStream_t st, unsigned wave,
-                         bool alone, bool dense) {
+cudaError_t launch_chain(const WaveChain& c, int n, const RunDev* runs, cudaStream_t st,
+                         unsigned wave, bool alone, bool dense) {
   switch (c.kind) {
-    case SMC_MODEL_LG: return launch_kind<SMC_MODEL_LG, R>(c, runs, st, wave, alone, dense);
-    case SMC_MODEL_CRBD: return launch_kind<SMC_MODEL_CRBD, R>(c, runs, st, wave, alone, dense);
+    case SMC_MODEL_LG: return launch_kind<SMC_MODEL_LG, R>(c, n, runs, st, wave, alone, dense);
+    case SMC_MODEL_CRBD: return launch_kind<SMC_MODEL_CRBD, R>(c, n, runs, st, wave, alone, dense);
     case SMC_MODEL_RATESHIFT:
-      return launch_kind<SMC_MODEL_RATESHIFT, R>(c, runs, st, wave, alone, dense);
-    case SMC_MODEL_SEIR: return launch_kind<SMC_MODEL_SEIR, R>(c, runs, st, wave, alone, dense);
-    case SMC_MODEL_CRBD_DS: return launch_kind<SMC_MODEL_CRBD_DS, R>(c, runs, st, wave, alone, dense);
-    default: return launch_kind<SMC_MODEL_GEOMETRIC, R>(c, runs, st, wave, alone, dense);
+      return launch_kind<SMC_MODEL_RATESHIFT, R>(c, n, runs, st, wave, alone, dense);
+    case SMC_MODEL_SEIR: return launch_kind<SMC_MODEL_SEIR, R>(c, n, runs, st, wave, alone, dense);
+    case SMC_MODEL_CRBD_DS: return launch_kind<SMC_MODEL_CRBD_DS, R>(c, n, runs, st, wave, alone, dense);
+    default: return launch_kind<SMC_MODEL_GEOMETRIC, R>(c, n, runs, st, wave, alone, dense);
   }
 }
 }  // namespace
 
 cudaError_t launch_wave(const WavePlan& W, int precision, cudaStream_t st, unsigned wave,
-                        const ChainStreams* streams) {
+                        const ChainStreams* streams, int* launched) {
   const bool alone = W.chains.size() == 1;
   // whether the wave's CTAs exceed what runs at once at 768 threads an SM
   long long threads = 0;
-  for (const WaveChain& c : W.chains) threads += (long long)c.n_ctas * (32 << c.bucket);
+  for (const WaveChain& c : W.chains) threads += (long long)c.ctas_at(wave) * (32 << c.bucket);
   const bool dense = threads > (long long)kSms * 768;
   for (size_t i = 0; i < W.chains.size(); ++i) {
     const WaveChain& c = W.chains[i];
+    const int n = c.ctas_at(wave);
+    if (n == 0) continue;
+    if (launched) ++*launched;
     const cudaStream_t s = streams ? streams->at((int)i) : st;
     const cudaError_t e = precision == SMC_PREC_FP32
-                              ? launch_chain<float>(c, W.runs, s, wave, alone, dense)
-                              : launch_chain<double>(c, W.runs, s, wave, alone, dense);
+                              ? launch_chain<float>(c, n, W.runs, s, wave, alone, dense)
+                              : launch_chain<double>(c, n, W.runs, s, wave, alone, dense);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -626,11 +632,19 @@ size_t wave_meta_bytes(const std::vector<RunDev>& runs) {
          kMaxChains * 256;
 }
 
-size_t fill_plan(const std::vector<RunDev>& runs, char* host, void* dev, WavePlan* W) {
+size_t fill_plan(const std::vector<RunDev>& runs, char* host, void* dev, WavePlan* W,
+                 const std::vector<int>* waves) {
   std::vector<int2> maps[kMaxChains];
-  for (size_t r = 0; r < runs.size(); ++r) {
-    std::vector<int2>& m = maps[(runs[r].md.kind - 1) * 4 + bucket_for(runs[r].tile)];
-    for (int t = 0; t < runs[r].n_tiles; ++t) m.push_back(make_int2((int)r, t));
+  std::vector<std::pair<int, int>> live[kMaxChains];
+  std::vector<int> order(runs.size());
+  std::iota(order.begin(), order.end(), 0);
+  if (waves)
+    std::stable_sort(order.begin(), order.end(),
+                     [&](int a, int b) { return (*waves)[a] > (*waves)[b]; });
+  for (const int r : order) {
+    const int c = (runs[r].md.kind - 1) * 4 + bucket_for(runs[r].tile);
+    for (int t = 0; t < runs[r].n_tiles; ++t) maps[c].push_back(make_int2(r, t));
+    if (waves) live[c].emplace_back((*waves)[r], (int)maps[c].size());
   }
   std::memcpy(host, runs.data(), sizeof(RunDev) * runs.size());
   size_t off = align_up(sizeof(RunDev) * runs.size(), 256);
@@ -643,6 +657,7 @@ size_t fill_plan(const std::vector<RunDev>& runs, char* host, void* dev, WavePla
     w.bucket = c % 4;
     w.n_ctas = (int)maps[c].size();
     w.map = (const int2*)((char*)dev + off);
+    w.live = std::move(live[c]);
     W->chains.push_back(w);
     std::memcpy(host + off, maps[c].data(), sizeof(int2) * maps[c].size());
     off = align_up(off + sizeof(int2) * maps[c].size(), 256);
@@ -654,9 +669,9 @@ size_t fill_plan(const std::vector<RunDev>& runs, char* host, void* dev, WavePla
 // staging the call waits for the copy; from `pinned` (at least
 // wave_meta_bytes(runs), not rewritten before the copy has run) it does not.
 smc_status upload_wave(const std::vector<RunDev>& runs, void* meta, cudaStream_t st, WavePlan* W,
-                       std::vector<char>* staging, char* pinned) {
+                       std::vector<char>* staging, char* pinned, const std::vector<int>* waves) {
   if (!pinned) staging->assign(wave_meta_bytes(runs), 0);
-  const size_t off = fill_plan(runs, pinned ? pinned : staging->data(), meta, W);
+  const size_t off = fill_plan(runs, pinned ? pinned : staging->data(), meta, W, waves);
   if (pinned) {
     SMC_CUDA_TRY(cudaMemcpyAsync(meta, pinned, off, cudaMemcpyHostToDevice, st));
     return SMC_OK;
@@ -684,7 +699,9 @@ smc_status capture_waves(GraphCache* g, const WavePlan& W, int precision, int ma
   graph_cache_clear(g);
   SMC_CUDA_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
   cudaError_t e = cudaSuccess;
-  for (int k = 0; k < max_waves && e == cudaSuccess; ++k) e = launch_wave(W, precision, st, (unsigned)k);
+  int launched = 0;
+  for (int k = 0; k < max_waves && e == cudaSuccess; ++k)
+    e = launch_wave(W, precision, st, (unsigned)k, nullptr, &launched);
   cudaGraph_t graph = nullptr;
   const cudaError_t e2 = cudaStreamEndCapture(st, &graph);
   if (e != cudaSuccess || e2 != cudaSuccess) {
@@ -700,6 +717,7 @@ smc_status capture_waves(GraphCache* g, const WavePlan& W, int precision, int ma
   g->plan = W;
   g->precision = precision;
   g->waves = max_waves;
+  g->launches = launched;
   return SMC_OK;
 }
 
@@ -716,14 +734,14 @@ smc_status drive_waves(const WavePlan& W, int precision, const std::vector<RunSt
   *launched = 0;
   *kernel_ms = 0.0;
   timed = timed && evs;
-  const int kernels_per_wave = (int)W.chains.size();
+  const int n_chains = (int)W.chains.size();
   if (known && graph && !timed && st != nullptr && st != cudaStreamLegacy) {
     if (!graph_matches(graph, W, precision, max_waves)) {
       smc_status s = capture_waves(graph, W, precision, max_waves, st);
       if (s) return s;
     }
     SMC_CUDA_TRY(cudaGraphLaunch(graph->exec, st));
-    *launched = kernels_per_wave * max_waves;
+    *launched = graph->launches;
     return SMC_OK;
   }
   int waves = 0;
@@ -736,18 +754,17 @@ smc_status drive_waves(const WavePlan& W, int precision, const std::vector<RunSt
       }
       SMC_CUDA_TRY(cudaEventRecord((*evs)[2 * waves], st));
     }
-    SMC_CUDA_TRY(launch_wave(W, precision, st, (unsigned)waves, streams));
+    SMC_CUDA_TRY(launch_wave(W, precision, st, (unsigned)waves, streams, launched));
     if (timed) SMC_CUDA_TRY(cudaEventRecord((*evs)[2 * waves + 1], st));
     ++waves;
-    *launched += kernels_per_wave;
     return SMC_OK;
   };
   if (known) {
     smc_status s = SMC_OK;
-    if (streams) SMC_CUDA_TRY(streams->fork(st, kernels_per_wave));
+    if (streams) SMC_CUDA_TRY(streams->fork(st, n_chains));
     for (int k = 0; k < max_waves && !s; ++k) s = one();
     if (streams) {  // after an error too: what was launched still uses the workspace
-      const cudaError_t e = streams->join(st, kernels_per_wave);
+      const cudaError_t e = streams->join(st, n_chains);
       if (!s && e != cudaSuccess) s = cuda_fail(e, "joining the chains' streams");
     }
     if (s) return s;
@@ -1297,6 +1314,7 @@ extern "C" smc_status smc_run_batch(const smc_model_t* ms, const smc_run_cfg* cf
   std::vector<Layout> lys(n_runs);
   std::vector<size_t> offs(n_runs);
   std::vector<RunDev> runs(n_runs);
+  std::vector<int> run_waves(n_runs);
   size_t total = 0;
   int max_waves = 0;
   bool known = true;
@@ -1306,7 +1324,9 @@ extern "C" smc_status smc_run_batch(const smc_model_t* ms, const smc_run_cfg* cf
     total = align_up(total + lys[q].total, 256);
     const bool kq = ms[q]->n_segments_known > 0 && lys[q].max_segments >= ms[q]->n_segments_known;
     known = known && kq;
-    max_waves = std::max(max_waves, kq ? ms[q]->n_segments_known : lys[q].max_segments);
+    run_waves[q] =  // the last one closes
+        std::min(kq ? ms[q]->n_segments_known : lys[q].max_segments, 0x7FFFFFFE) + 1;
+    max_waves = std::max(max_waves, run_waves[q]);
     runs[q].n_tiles = lys[q].n_tiles;
   }
   const size_t meta_off = total;
@@ -1347,7 +1367,8 @@ extern "C" smc_status smc_run_batch(const smc_model_t* ms, const smc_run_cfg* cf
                                  cudaMemcpyHostToDevice, cs));
   WavePlan W;
   std::vector<char> staging;
-  if ((st = upload_wave(runs, (char*)ws + meta_off, cs, &W, &staging))) return st;
+  if ((st = upload_wave(runs, (char*)ws + meta_off, cs, &W, &staging, nullptr, &run_waves)))
+    return st;
   struct Events {
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     ~Events() {
@@ -1365,7 +1386,7 @@ extern "C" smc_status smc_run_batch(const smc_model_t* ms, const smc_run_cfg* cf
   ChainStreams streams;
   const bool fan = known && !graphed && W.chains.size() > 1;
   if (fan) SMC_CUDA_TRY(streams.init(std::min((int)W.chains.size(), kChainStreams)));
-  st = drive_waves(W, prec, states, max_waves + 1, known, cs, nullptr, false, &launched, &kms,
+  st = drive_waves(W, prec, states, max_waves, known, cs, nullptr, false, &launched, &kms,
                    graphed ? &graph : nullptr, fan ? &streams : nullptr);
   if (st) {
     graph_cache_clear(&graph);

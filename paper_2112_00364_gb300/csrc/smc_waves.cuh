@@ -13,10 +13,10 @@
 namespace smc {
 
 template <int KIND, typename R>
-cudaError_t launch_kind(const WaveChain& c, const RunDev* runs, cudaStream_t st, unsigned wave,
-                        bool alone, bool dense) {
-  return dense ? launch_bucket<R, KIND, true>(c.bucket, runs, c.map, c.n_ctas, st, wave, alone)
-               : launch_bucket<R, KIND, false>(c.bucket, runs, c.map, c.n_ctas, st, wave, alone);
+cudaError_t launch_kind(const WaveChain& c, int n_ctas, const RunDev* runs, cudaStream_t st,
+                        unsigned wave, bool alone, bool dense) {
+  return dense ? launch_bucket<R, KIND, true>(c.bucket, runs, c.map, n_ctas, st, wave, alone)
+               : launch_bucket<R, KIND, false>(c.bucket, runs, c.map, n_ctas, st, wave, alone);
 }
 
 }  // namespace smc

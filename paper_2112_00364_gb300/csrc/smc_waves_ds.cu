@@ -3,7 +3,7 @@
 
 namespace smc {
 
-template cudaError_t launch_kind<SMC_MODEL_CRBD_DS, double>(const WaveChain&, const RunDev*, cudaStream_t, unsigned,
+template cudaError_t launch_kind<SMC_MODEL_CRBD_DS, double>(const WaveChain&, int, const RunDev*, cudaStream_t, unsigned,
     bool, bool);
 
 }  // namespace smc

@@ -3,9 +3,9 @@
 
 namespace smc {
 
-template cudaError_t launch_kind<SMC_MODEL_LG, float>(const WaveChain&, const RunDev*, cudaStream_t, unsigned,
+template cudaError_t launch_kind<SMC_MODEL_LG, float>(const WaveChain&, int, const RunDev*, cudaStream_t, unsigned,
     bool, bool);
-template cudaError_t launch_kind<SMC_MODEL_CRBD, float>(const WaveChain&, const RunDev*, cudaStream_t, unsigned,
+template cudaError_t launch_kind<SMC_MODEL_CRBD, float>(const WaveChain&, int, const RunDev*, cudaStream_t, unsigned,
     bool, bool);
 
 }  // namespace smc

@@ -3,11 +3,11 @@
 
 namespace smc {
 
-template cudaError_t launch_kind<SMC_MODEL_RATESHIFT, double>(const WaveChain&, const RunDev*, cudaStream_t, unsigned,
+template cudaError_t launch_kind<SMC_MODEL_RATESHIFT, double>(const WaveChain&, int, const RunDev*, cudaStream_t, unsigned,
     bool, bool);
-template cudaError_t launch_kind<SMC_MODEL_GEOMETRIC, double>(const WaveChain&, const RunDev*, cudaStream_t, unsigned,
+template cudaError_t launch_kind<SMC_MODEL_GEOMETRIC, double>(const WaveChain&, int, const RunDev*, cudaStream_t, unsigned,
     bool, bool);
-template cudaError_t launch_kind<SMC_MODEL_GEOMETRIC, float>(const WaveChain&, const RunDev*, cudaStream_t, unsigned,
+template cudaError_t launch_kind<SMC_MODEL_GEOMETRIC, float>(const WaveChain&, int, const RunDev*, cudaStream_t, unsigned,
     bool, bool);
 
 }  // namespace smc
