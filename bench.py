@@ -85,18 +85,18 @@ RS_BYTES = 20          # logw read twice (normaliser, scan) + ancestor written, 
 # DADD + DMUL), DRAM traffic per launch and the FP64 pipe's busy fraction.  The
 # roofline basis is the unit that bounds the kernel: instruction issue for the
 # plain CRBD (latency-bound, most arithmetic on the integer pipes), the FP64
-# rate for the delayed-sampling CRBD (FP64 pipe busy 36-44% of a launch).  The
+# rate for the delayed-sampling CRBD (FP64 pipe busy 26-40% of a launch).  The
 # traffic holds only for the kernel sources with the recorded digest.
-NCU = {"crbd64": dict(basis="issue", warp_inst_per_pstep=113.9, fp64_flop_per_pstep=18.8,
-                      bytes_per_launch=2.963e6, fp64_pipe_elapsed=0.185,
-                      src_digest="fc844398542168c5"),
-       "crbd_ds128": dict(basis="fp64", warp_inst_per_pstep=110.2, fp64_flop_per_pstep=169.1,
-                          bytes_per_launch=4.953e6, fp64_pipe_elapsed=0.353,
-                          src_digest="fc844398542168c5"),
+NCU = {"crbd64": dict(basis="issue", warp_inst_per_pstep=99.6, fp64_flop_per_pstep=16.9,
+                      bytes_per_launch=3.778e6, fp64_pipe_elapsed=0.146,
+                      src_digest="697fcdc932dbb4c1"),
+       "crbd_ds128": dict(basis="fp64", warp_inst_per_pstep=75.3, fp64_flop_per_pstep=91.7,
+                          bytes_per_launch=5.401e6, fp64_pipe_elapsed=0.316,
+                          src_digest="697fcdc932dbb4c1"),
        # FP32 waves of 2^20 particles: bound by memory latency (long-scoreboard
-       # stalls), reported against HBM; 72-75 warp instructions per particle-step
-       "rateshift256": dict(basis="hbm", warp_inst_per_pstep=73.5, bytes_per_launch=1.182e8,
-                            src_digest="fc844398542168c5")}
+       # stalls), reported against HBM; 61-85 warp instructions per particle-step
+       "rateshift256": dict(basis="hbm", warp_inst_per_pstep=69.3, bytes_per_launch=1.112e8,
+                            src_digest="697fcdc932dbb4c1")}
 
 # 152 SMs x 2070 MHz x 4 FP64 flop/clk/SM (2 DFMA/clk/SM) = GB300's FP64 rate
 FP64_PEAK_FLOPS = 152 * 2070e6 * 4
@@ -115,7 +115,7 @@ RS_SOURCES = ("smc_prims.cu", "smc_device.cuh", "smc_combine.cuh")
 # DRAM traffic of one smc_resample call at 2^24 (the three kernels' dram__bytes
 # read + write in one ncu capture, profiles folder), valid for the sources with
 # the recorded digest.
-RS_NCU = dict(bytes_per_call=2.353e8, src_digest="84e4a804f220f1c5")
+RS_NCU = dict(bytes_per_call=2.353e8, src_digest="abef18a496ac9b77")
 
 
 def code_text(src: str) -> str:
@@ -1122,7 +1122,7 @@ def main() -> int:
                          "per particle-step, from the run's device counters"},
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": d2h},
-        "gpu_launches": args.steps * (meas["launches_per_step"] + len(work.runs)),
+        "gpu_launches": args.steps * (meas["launches_per_step"] + 1),  # + the collecting kernel
         "roofline": roof,
         "cpu_baseline": cpu,
         "clocks": meas["clocks"],
