@@ -869,20 +869,32 @@ __global__ void __launch_bounds__(RS_TPB, 3) rs_ancestors(
 }
 
 // Particle duplication: dst[f][i] = src[f][anc[i]], 16-byte stores of
-// consecutive particles.
-template <typename T, int V>
+// consecutive particles; with stack pointers (STACK) row f only for the particles
+// with f < sp[anc[i]].  Rows of whole 16-byte groups without stack pointers, and one
+// or two FP32 rows with them (4.2 M x 1: 10.5 us against 12.4 in the other form).
+template <typename T, int V, bool STACK>
 __global__ void gather_kernel(const T* __restrict__ src, T* __restrict__ dst,
-                              const int32_t* __restrict__ anc, int64_t N, int n_fields) {
+                              const int32_t* __restrict__ anc, const int32_t* __restrict__ sp,
+                              int64_t N, int n_fields) {
   const int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * V;
   if (i0 >= N) return;
   int32_t a[V];
+  int32_t s[V];
 #pragma unroll
-  for (int q = 0; q < V; ++q) a[q] = (i0 + q < N) ? __ldg(anc + i0 + q) : 0;
+  for (int q = 0; q < V; ++q) {
+    a[q] = (i0 + q < N) ? __ldg(anc + i0 + q) : 0;
+    s[q] = STACK ? ((i0 + q < N) ? __ldg(sp + a[q]) : 0) : n_fields;
+  }
   const bool full = (i0 + V <= N) && ((reinterpret_cast<uintptr_t>(dst) & 15) == 0) && (N % V == 0);
   for (int f = 0; f < n_fields; ++f) {
     const T* sf = src + (size_t)f * N;
     T* df = dst + (size_t)f * N;
-    if (full) {
+    bool all = full;
+    if (STACK) {
+#pragma unroll
+      for (int q = 0; q < V; ++q) all = all && (f < s[q]);
+    }
+    if (all) {
       union {
         T e[V];
         uint4 u;
@@ -893,52 +905,69 @@ __global__ void gather_kernel(const T* __restrict__ src, T* __restrict__ dst,
     } else {
 #pragma unroll
       for (int q = 0; q < V; ++q)
-        if (i0 + q < N) df[i0 + q] = __ldg(sf + a[q]);
+        if (i0 + q < N && f < s[q]) df[i0 + q] = __ldg(sf + a[q]);
     }
   }
 }
 
-// The same with stack pointers: row f only for the particles with f < sp[anc[i]].
+// The same in whole lines whatever the rows' length, alignment and stack pointers.
 // Bound: HBM (a 32-byte sector of dst with some rows missing is read before it is
-// written).  A CTA takes GA_V * 256 consecutive particles, thread x those at x, x +
-// 256, ..., so that a warp's loads and stores cover whole lines whichever of its
-// particles still have the row and whatever the rows' alignment, and GA_U rows of
-// GA_V particles are loaded before the first store.  12 FP32 rows, the pointers
-// uniform: 2^24 particles 374 -> 308 us, 1.8 M 46.6 -> 37.0, 1 M 18.6 -> 12.7 against
-// four consecutive particles a thread; without stack pointers that form with its
-// 16-byte stores is the faster one (2^24 x 1 FP32 row 39 us against 80).
-constexpr int GA_TPB = 256, GA_V = 4;
-template <typename T, int GA_U>
-__global__ void __launch_bounds__(GA_TPB) gather_stack_kernel(
+// written); below a million particles the latency of the loads.  A CTA takes V * 256
+// consecutive particles, thread x those at x, x + 256, ..., so that a warp's loads and
+// stores cover whole lines, and U rows of V particles are loaded before the first
+// store.  us a copy, four consecutive particles a thread / this form: 12 FP32 rows with
+// pointers 2^24 particles 374 / 308, 1.8 M 46.6 / 37.0, 1 M 18.6 / 12.7; 12 ragged FP32
+// rows without them 4.2 M 77.7 / 72.0, 1 M 22.8 / 14.5, 10,001 8.3 / 4.3; 8 ragged FP64
+// rows 4.2 M 103 / 84, 1 M 30.9 / 22.7.  Rows of whole 16-byte groups without pointers
+// stay with their 16-byte stores (2^24 x 1 FP32 row 39 against 80).  V, U: 4, 4 for
+// FP32; 2, 4 for FP64 (8 x 4.2 M 84, with 4, 4 96), but 4, 2 for one or two rows with
+// pointers (1 x 4.2 M 16.6 against 20.6).
+constexpr int GA_TPB = 256;
+template <typename T, int V, int U, bool STACK>
+__global__ void __launch_bounds__(GA_TPB) gather_lines_kernel(
     const T* __restrict__ src, T* __restrict__ dst, const int32_t* __restrict__ anc,
     const int32_t* __restrict__ sp, int64_t N, int n_fields) {
-  const int64_t i0 = (int64_t)blockIdx.x * (GA_TPB * GA_V) + threadIdx.x;
-  const T* from[GA_V];
-  T* to[GA_V];
-  int rows[GA_V];
+  const int64_t i0 = (int64_t)blockIdx.x * (GA_TPB * V) + threadIdx.x;
+  const T* from[V];
+  T* to[V];
+  int rows[V];
   int most = 0;
 #pragma unroll
-  for (int q = 0; q < GA_V; ++q) {
+  for (int q = 0; q < V; ++q) {
     const int64_t i = i0 + q * GA_TPB;
     const int a = i < N ? __ldg(anc + i) : 0;
     from[q] = src + a;
     to[q] = dst + i;
-    rows[q] = i < N ? min(__ldg(sp + a), n_fields) : 0;
+    rows[q] = i >= N ? 0 : STACK ? min(__ldg(sp + a), n_fields) : n_fields;
     most = max(most, rows[q]);
   }
-  for (int f = 0; f < most; f += GA_U) {
-    T e[GA_U][GA_V];
+  for (int f = 0; f < most; f += U) {
+    T e[U][V];
 #pragma unroll
-    for (int r = 0; r < GA_U; ++r)
+    for (int r = 0; r < U; ++r)
 #pragma unroll
-      for (int q = 0; q < GA_V; ++q)
+      for (int q = 0; q < V; ++q)
         if (f + r < rows[q]) e[r][q] = __ldg(from[q] + (f + r) * N);
 #pragma unroll
-    for (int r = 0; r < GA_U; ++r)
+    for (int r = 0; r < U; ++r)
 #pragma unroll
-      for (int q = 0; q < GA_V; ++q)
+      for (int q = 0; q < V; ++q)
         if (f + r < rows[q]) to[q][(f + r) * N] = e[r][q];
   }
+}
+
+template <typename T, int V, bool STACK>
+void launch_gather(const void* src, void* dst, const int32_t* anc, const int32_t* sp, int64_t N,
+                   int n_fields, cudaStream_t cs) {
+  gather_kernel<T, V, STACK><<<(unsigned)((N + 256 * V - 1) / (256 * V)), 256, 0, cs>>>(
+      (const T*)src, (T*)dst, anc, sp, N, n_fields);
+}
+template <typename T, int V, int U, bool STACK>
+void launch_gather_lines(const void* src, void* dst, const int32_t* anc, const int32_t* sp, int64_t N,
+                         int n_fields, cudaStream_t cs) {
+  gather_lines_kernel<T, V, U, STACK>
+      <<<(unsigned)((N + GA_TPB * V - 1) / (GA_TPB * V)), GA_TPB, 0, cs>>>((const T*)src, (T*)dst, anc,
+                                                                         sp, N, n_fields);
 }
 
 __global__ void philox_kernel(const uint32_t* __restrict__ ctr, const uint32_t* __restrict__ key,
@@ -1324,23 +1353,18 @@ extern "C" smc_status smc_gather(const void* src, void* dst, const int32_t* anc,
   if (!src || !dst || !anc) return set_error(SMC_EINVAL, "NULL pointer");
   if (N < 1 || n_fields < 1) return set_error(SMC_EINVAL, "N and n_fields must be >= 1");
   cudaStream_t cs = (cudaStream_t)stream;
-  const unsigned grid = (unsigned)((N + GA_TPB * GA_V - 1) / (GA_TPB * GA_V));
-  if (sp && elem_bytes == 8) {
-    gather_stack_kernel<double, 2><<<grid, GA_TPB, 0, cs>>>((const double*)src, (double*)dst, anc,
-                                                            sp, N, n_fields);
-  } else if (sp && elem_bytes == 4) {
-    gather_stack_kernel<float, 4><<<grid, GA_TPB, 0, cs>>>((const float*)src, (float*)dst, anc, sp,
-                                                           N, n_fields);
-  } else if (elem_bytes == 8) {
-    const int64_t threads = (N + 1) / 2;
-    gather_kernel<double, 2><<<(unsigned)((threads + 255) / 256), 256, 0, cs>>>(
-        (const double*)src, (double*)dst, anc, N, n_fields);
-  } else if (elem_bytes == 4) {
-    const int64_t threads = (N + 3) / 4;
-    gather_kernel<float, 4><<<(unsigned)((threads + 255) / 256), 256, 0, cs>>>(
-        (const float*)src, (float*)dst, anc, N, n_fields);
+  if (elem_bytes != 4 && elem_bytes != 8) return set_error(SMC_EINVAL, "elem_bytes must be 4 or 8");
+  const bool whole = N % (16 / elem_bytes) == 0 && (reinterpret_cast<uintptr_t>(dst) & 15) == 0;
+  if (elem_bytes == 4) {
+    if (sp && n_fields > 2) launch_gather_lines<float, 4, 4, true>(src, dst, anc, sp, N, n_fields, cs);
+    else if (sp) launch_gather<float, 4, true>(src, dst, anc, sp, N, n_fields, cs);
+    else if (whole) launch_gather<float, 4, false>(src, dst, anc, sp, N, n_fields, cs);
+    else launch_gather_lines<float, 4, 4, false>(src, dst, anc, sp, N, n_fields, cs);
   } else {
-    return set_error(SMC_EINVAL, "elem_bytes must be 4 or 8");
+    if (sp && n_fields > 2) launch_gather_lines<double, 2, 4, true>(src, dst, anc, sp, N, n_fields, cs);
+    else if (sp) launch_gather_lines<double, 4, 2, true>(src, dst, anc, sp, N, n_fields, cs);
+    else if (whole) launch_gather<double, 2, false>(src, dst, anc, sp, N, n_fields, cs);
+    else launch_gather_lines<double, 2, 4, false>(src, dst, anc, sp, N, n_fields, cs);
   }
   SMC_CUDA_TRY(cudaGetLastError());
   return SMC_OK;
