@@ -208,7 +208,7 @@ int tile_for(int64_t N);
 int bucket_for(int tile);
 // The combine placement of a run (the same results either way): in every CTA
 // of the next wave when latency matters (`single`: a run alone, up to
-// redundant_cap tiles), else only for runs of at most one tile per thread.
+// redundant_cap tiles), else only for runs of at most 32 tiles.
 int combine_in_every_cta(int tile, int n_tiles, bool single);
 Layout make_layout(const smc_model_s* m, const smc_run_cfg* c);
 RunDev make_rundev(const smc_model_s* m, const smc_run_cfg* c, const Layout& Ly, char* ws);
