@@ -621,13 +621,19 @@ __global__ void __launch_bounds__(TPB, min_ctas(resident_threads<R, KIND>(TPB, D
   // start (and copy their run table, which no kernel writes) while the last CTAs
   // of the previous one still run; everything below reads what that wave wrote, so
   // it waits for its completion first.
+  using M = typename ModelOf<KIND, R>::type;
   // (a lone chain's grid of at most one CTA an SM leaves room for the next wave's
   // CTAs beside its own: those then start at once, and what they do before the wait
   // is hidden.  Beside other chains they would take places from them)
   const bool early = alone && gridDim.x <= kSms;
-  if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // (Triggered before the wait, several waves gather on the SMs, and the later ones take
+  // the places that happen to come free, two CTAs of a wave on one SM beside idle ones:
+  // SEIR FP32 with 122 CTAs of 128 195 us a day, after the wait 114; CRBD with delayed
+  // sampling 30.7 / 24.3.  Only the models that draw ahead, whose blocks are short, are
+  // faster so in CTAs of 256: 23,171 FP64 7.26 us a wave, 7.68 after the wait.)
+  const bool ahead = early && M::PREDRAW && TPB == 256;
+  if (ahead) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int k = (int)(wave - sr.start_wave);  // wraps correctly past 2^32 waves
-  using M = typename ModelOf<KIND, R>::type;
   typename M::Lane L;
   Stream s{sr.k0, sr.k1, (uint32_t)(rt.y * sr.tile + threadIdx.x), (uint32_t)k, 0u, 0u, sr.md.tab};
   if constexpr (M::PREDRAW) {
@@ -641,6 +647,7 @@ __global__ void __launch_bounds__(TPB, min_ctas(resident_threads<R, KIND>(TPB, D
   // alone: in the wait's shadow
   if (threadIdx.x == 0) S.uf = search_uniform(sr, sr.redundant ? k - 1 : k);
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (early && !ahead) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   RunState* rs = sr.rs;
   if (*(volatile int32_t*)&rs->done || k < 0) return;
   step_tile<M, TPB>(sr, rt.y, k, S, L, s, early);
