@@ -375,9 +375,9 @@ __device__ __forceinline__ long long exp_fix2(double d, const unsigned long long
 
 // ---- the argument k ln 2 - x in 2^-58 fixed point, on the integer pipes ----
 // For a power-of-two reference 2^k (|k| < 2^11) and a log-weight x <= k ln 2
-// (up to rounding): K = k ln 2 2^58 from ln 2 to 2^-116, and x 2^58 from the
-// bits of x, so X = K - x 2^58 is within two units of (k ln 2 - x) 2^58
-// whatever the magnitudes of k and x.
+// (but for the rounding of k = ceil(x / ln 2)): K = k ln 2 2^58 from ln 2 to 2^-116,
+// and x 2^58 from the bits of x, so X = K - x 2^58 is within two units of
+// (k ln 2 - x) 2^58 whatever the magnitudes of k and x.
 constexpr unsigned long long kLn2Q116Hi = 0xb17217f7d1cf7ull;               // round(ln 2 2^116) >> 64
 constexpr unsigned long long kLn2Q116Lo = 0x9abc9e3b39803f2full;           // its low 64 bits
 constexpr unsigned long long kExpCutQ58 = 0x9a00000000000000ull;           // 38.5 2^58
@@ -434,7 +434,11 @@ __device__ __forceinline__ long long weight_fix54(double x, int k, unsigned long
   const int sh = e - 1017;  // x 2^58 = m 2^sh
   const unsigned long long v = sh >= 0 ? shl64(m, (unsigned)sh) : shr64(m, (unsigned)-sh);
   unsigned long long X = b < 0 ? K + v : K - v;
-  if (X > ~15ull) X = 0;  // x above the reference by rounding: weight 1
+  // x above the reference by rounding: weight 1.  The product behind k = ceil(x / ln 2)
+  // may round down to the integer k by up to 2^-52 of it, so X may wrap from as far as
+  // 2^17 units below zero (it does for x = log(2^j) with 4 in 10 of the j); what has
+  // not wrapped lies below 2^64 - 2^59, by the comparison above
+  if ((unsigned)(X >> 32) == 0xffffffffu) X = 0;
   if (X >= kExpCutQ58) return 0;
   return exp_fix_x<54>(X, T);
 }
