@@ -1356,8 +1356,12 @@ __device__ __forceinline__ int neg_binomial<double>(Stream& s, double alpha, dou
   const float be = trunc_f32((unsigned)(bb >> 32), (unsigned)bb);
   const float t = trunc_f32((unsigned)(tb >> 32), (unsigned)tb);
   const float r = __fdividef(t, be), mean = a * r;
-  // (magnitudes that single precision holds with all its bits)
-  if (a < 1e6f && be > 1e-12f && be < 1e12f && (t > 1e-12f || t == 0.0f) && mean < 9.99f) {
+  // (magnitudes that single precision holds with all its bits, by the doubles' exponents:
+  // a float's would wrap from 2^128 on, a rate of 2^512 counting as 1)
+  auto in_range = [](unsigned long long b) {  // 2^-40 <= x < 2^40, x > 0
+    return (unsigned)(b >> 32) - 0x3d700000u < 0x05000000u;
+  };
+  if (in_range(ab) && in_range(bb) && (in_range(tb) || tb == 0) && a < 1e6f && mean < 9.99f) {
     const uint32_t d0 = s.d;
     const float u = (float)(s.next().w1 >> 8) * 0x1p-24f;
     const float eps = fmaf(4e-6f, mean, 6e-6f);
