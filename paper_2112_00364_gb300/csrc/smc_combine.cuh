@@ -105,16 +105,27 @@ __host__ __device__ constexpr int ess_thread(int tpb) { return tpb > 32 ? 32 : 0
 // 64-bit words of shared scratch that combine_offsets uses.
 __host__ __device__ constexpr int combine_scratch(int tpb) { return 6 * (tpb / 32); }
 
-// q 2^-d for a tile's sum of squared weights q and d >= 0, in 32.32-bit pieces
-// (bits below 2^-32 dropped), added to f (fraction), l and h (the value's halves).
-__device__ __forceinline__ void add_scaled(unsigned long long q, int d, unsigned long long* f,
-                                           unsigned long long* l, unsigned long long* h) {
-  const unsigned long long v = d < 64 ? q >> d : 0ull;
-  const unsigned long long frac =
-      d < 32 ? (q << (32 - d)) & 0xffffffffull : d < 96 ? (q >> (d - 32)) & 0xffffffffull : 0ull;
-  *f += frac;
+// A tile's sum of squared weights q brought from its reference 2^k_t to the run's
+// 2^(k_t + d), d >= 0: q 2^-2d in 32.32-bit pieces (bits below 2^-32 dropped), added
+// to f (fraction), l and h (the value's halves); each piece is below 2^32.
+__device__ __forceinline__ void add_squares(unsigned long long q, int d, unsigned long long* f,
+                                            unsigned long long* l, unsigned long long* h) {
+  if (d >= 48) return;  // q <= 2^62: nothing left
+  const int sh = 2 * d;
+  const unsigned long long v = sh < 64 ? q >> sh : 0ull;
+  *f += (sh < 32 ? q << (32 - sh) : q >> (sh - 32)) & 0xffffffffull;
   *l += v & 0xffffffffull;
   *h += v >> 32;
+}
+
+// (sum w)^2 / sum w^2 from the pieces' sums and the total S in units U.  The sums are
+// integers, so every combine of the same records forms the same number.
+__device__ __forceinline__ double ess_of(unsigned long long f, unsigned long long l,
+                                         unsigned long long h, long long S, int G) {
+  const double acc =
+      ((double)h * 4294967296.0 + ((double)l + (double)f * 0x1p-32)) * pow2i(-54);
+  const double sd = (double)S * pow2i(G - 54);
+  return acc > 0.0 ? (sd * sd) / acc : 0.0;
 }
 
 // Combine n_tiles tile records into the offsets O[0..nt] (O[nt] = S); ks non-NULL
@@ -203,10 +214,8 @@ __device__ __forceinline__ Combined combine_offsets(const TileRec* rec, int nt, 
   unsigned long long qf = 0, ql = 0, qh = 0;
   each([&](int t, const TileRec& x) {
     bl += magnitude(x.s, x.k, c.kmax);
-    if (q && x.k != kDeadTile) {  // sum w^2 relative to 2^(2 k_max)
-      const int d = c.kmax - x.k;
-      if (d < 48) add_scaled((unsigned long long)__ldcg(q + t), 2 * d, &qf, &ql, &qh);
-    }
+    if (q && x.k != kDeadTile)
+      add_squares((unsigned long long)__ldcg(q + t), c.kmax - x.k, &qf, &ql, &qh);
   });
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) bl += __shfl_xor_sync(kAll, bl, o);
@@ -279,10 +288,7 @@ __device__ __forceinline__ Combined combine_offsets(const TileRec* rec, int nt, 
       l += es[3 * w + 1];
       h += es[3 * w + 2];
     }
-    const double acc =
-        ((double)h * 4294967296.0 + ((double)l + (double)f * 0x1p-32)) * pow2i(-54);
-    const double sd = (double)c.S * pow2i(c.G - 54);
-    c.ess = acc > 0.0 ? (sd * sd) / acc : 0.0;
+    c.ess = ess_of(f, l, h, c.S, c.G);
   }
   after(c);
   __syncthreads();  // the offsets and after()'s results for every thread

@@ -163,11 +163,18 @@ __device__ __forceinline__ void warp_add_u64_wide(unsigned long long* dst, unsig
   if ((threadIdx.x & 31) == 0 && v) atomicAdd(dst, v);
 }
 
+// The warp's sum of a 32-bit value per lane, exactly, to every lane.
+__device__ __forceinline__ unsigned long long warp_sum_u32(unsigned v) {
+  const unsigned lo = __reduce_add_sync(0xffffffffu, v & 0xffffu);
+  const unsigned hi = __reduce_add_sync(0xffffffffu, v >> 16);
+  return lo + ((unsigned long long)hi << 16);
+}
+
 // The combine of at most 32 tiles by one warp, lane t holding tile t: the
 // integers of combine_offsets (the same k_max, coarsening G, unit totals,
-// exact offsets and S, and the effective sample size summed in the same
-// order) from warp shuffles, with no CTA barrier.  Writes O[0..nt] (O[nt] = S)
-// and ks[0..nt) to the warp's own shared arrays.
+// exact offsets and S, and pieces of the sum of squared weights, so the same
+// effective sample size) from warp shuffles, with no CTA barrier.  Writes
+// O[0..nt] (O[nt] = S) and ks[0..nt) to the warp's own shared arrays.
 __device__ __forceinline__ Combined combine_warp(const TileRec* rec, int nt, const long long* q,
                                                  long long* O, int* ks) {
   constexpr unsigned kAll = 0xffffffffu;
@@ -203,15 +210,11 @@ __device__ __forceinline__ Combined combine_warp(const TileRec* rec, int nt, con
   if (lane < nt) O[lane] = inc - v;
   if (lane == 0) O[nt] = c.S;
   if (q) {
-    double acc = 0.0;
-    if (lane < nt && r.k != kDeadTile) {
-      const int d2 = 2 * (c.kmax - r.k);
-      if (d2 < 900) acc = acc + (double)q[lane] * pow2i(-54 - d2);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc = acc + __shfl_xor_sync(kAll, acc, o);
-    const double sd = (double)c.S * pow2i(c.G - 54);
-    c.ess = acc > 0.0 ? (sd * sd) / acc : 0.0;
+    unsigned long long f = 0, l = 0, h = 0;
+    if (lane < nt && r.k != kDeadTile)
+      add_squares((unsigned long long)q[lane], c.kmax - r.k, &f, &l, &h);
+    c.ess = ess_of(warp_sum_u32((unsigned)f), warp_sum_u32((unsigned)l), warp_sum_u32((unsigned)h),
+                   c.S, c.G);
   }
   __syncwarp();
   return c;
