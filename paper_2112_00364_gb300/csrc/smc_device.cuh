@@ -1175,7 +1175,9 @@ __device__ __forceinline__ int binomial_f32(Stream& s, int n, double pd, unsigne
     return -1;
   }
   // Transformed rejection.  With b below within 3e-7 relative, a within 7e-7, the
-  // offset x = (2a/us + b) u is within 1.5e-6 relative, and 2^-31/us of us;
+  // offset x = (2a/us + b) u is within 1.5e-6 relative.  The 2^-32 of u's dropped
+  // bits move it by (a/us^2 + b) 2^-32 (dx/du), which 2^-31/us of x and (4a + b) 2^-32
+  // cover together: with r = us the sum less that is a (2 - 1/r)^2 2^-32 and more.
   // floor(x + n p' + 1/2) adds the whole part of n p' as an integer, and where x
   // lies too near a whole number it is taken in FP64 (btrs_candidate).
   const float npf = (float)n * pp;
@@ -1184,6 +1186,7 @@ __device__ __forceinline__ int binomial_f32(Stream& s, int n, double pd, unsigne
   const float a = fmaf(0.01f, pp, fmaf(0.0248f, b, -0.0873f));
   const float vr = 0.92f - __fdividef(4.2f, b);
   const float cf = fmaf((float)nfr, 0x1p-32f, 0.5f);
+  const float e0 = fmaf(fmaf(4.0f, a, b), 0x1p-32f, 2e-6f);
   for (int trial = 0; trial < 100; ++trial) {
     const Block4 blk = s.next();
     const int su = (int)(blk.w1 ^ 0x80000000u);  // u 2^32, u = U - 1/2
@@ -1193,7 +1196,7 @@ __device__ __forceinline__ int binomial_f32(Stream& s, int n, double pd, unsigne
     const float v = (float)blk.w3 * 0x1p-32f;
     const float x = (__fdividef(2.0f * a, us) + b) * ((float)su * 0x1p-32f);
     const float y = x + cf, fl = floorf(y), dy = y - fl;
-    const float ex = fmaf(fabsf(x), 2.5e-6f + __fdividef(0x1p-31f, us), 2e-6f);
+    const float ex = fmaf(fabsf(x), 2.5e-6f + __fdividef(0x1p-31f, us), e0);
     int k = (int)np + (int)fl;
     if (!(dy > ex && dy < 1.0f - ex)) k = btrs_candidate(n, pd, blk);
     if (k < 0 || k > n) continue;
