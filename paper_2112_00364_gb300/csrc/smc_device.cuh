@@ -1229,8 +1229,8 @@ __device__ __forceinline__ int binomial_f32(Stream& s, int n, double pd, unsigne
     const float lhs = __logf(__fdividef(v * alpha, fmaf(__fdividef(a, us), __fdividef(1.0f, us), b)));
     // errors: 2e-6 of each deviance from its series; a logarithm's 4e-7 (2^-21.4 ln 2
     // near 1) times M (1 + t) where it is used; the left side's argument 3e-6 and
-    // its logarithm 5e-6, the rest below 2e-6
-    float eL = fmaf(2e-6f, g1 + g2, 6e-5f) + __fdividef(0x1p-30f, us);
+    // its logarithm 5e-6, v's dropped bits 2^-32 / v and us's 2^-31 / us, the rest below 2e-6
+    float eL = fmaf(2e-6f, g1 + g2, 6e-5f) + __fdividef(0x1p-30f, us) + __fdividef(0x1p-32f, v);
     if (fabsf(t) >= 0.2f) eL = fmaf(8e-7f * M, 1.0f + t, eL);
     if (fabsf(w) >= 0.2f) eL = fmaf(8e-7f * W, 1.0f + w, eL);
     if (!(fabsf(lhs - L) > eL)) return -1;
