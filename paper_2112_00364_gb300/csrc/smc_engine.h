@@ -85,7 +85,9 @@ struct CollectJob {
   double *log_z, *logw, *real, *stack;
   int32_t *ints, *anc, *resampled;
   int N, n_real, n_int, cap, fp32, record_all, anc_rows, res_rows, max_segments;
+  int parts;  // a batch's job: its CTAs
 };
+static_assert(sizeof(CollectJob) % 8 == 0, "the CTA map follows the jobs");
 
 struct Layout {
   size_t real[2], ints[2], stack[2], logw, E[2], ends[2], rec[2], tq[2], dec, tO, rs, anc, incr,
