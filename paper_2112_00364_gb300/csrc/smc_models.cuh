@@ -131,8 +131,8 @@ struct LgModel {
     bool drawn;
     int overflow, limited;
   };
-  // a segment's first draw, whichever block takes it: block 1 has one, and a snapshot
-  // may hold particles at block 0, which draws before it
+  // every particle of a segment k > 0 runs block 1, whose one draw is its first, but
+  // those that a snapshot holds at block 0 (a segment that wave_kernel does not draw for)
   __device__ static void predraw(Lane& L, Stream& s) {
     L.z = normal01<R>(s);
     L.drawn = true;
@@ -173,8 +173,7 @@ struct LgModel {
   __device__ static void block(int b, Lane& L, Stream& s, const ModelDev& md, const StateView&, int,
                                int k, int) {
     if (b == 0) {
-      const R z0 = L.drawn ? L.z : normal01<R>(s);
-      L.drawn = false;
+      const R z0 = normal01<R>(s);
       L.x = m_fma(md.c((R)0).x0_sd, z0, md.c((R)0).x0_mean);
       L.pc = 1;
       return;

@@ -637,11 +637,12 @@ __global__ void __launch_bounds__(TPB, min_ctas(resident_threads<R, KIND>(TPB, D
   typename M::Lane L;
   Stream s{sr.k0, sr.k1, (uint32_t)(rt.y * sr.tile + threadIdx.x), (uint32_t)k, 0u, 0u, sr.md.tab};
   if constexpr (M::PREDRAW) {
-    // (not for a segment that loads a snapshot.  In larger grids most CTAs start
+    // (not for a segment that loads a snapshot, nor the one after it, which runs the
+    // blocks that the snapshot names.  In larger grids most CTAs start
     // after the wave before them has ended: nothing to hide the draw behind, and
     // drawing there took a wave of 2^20 FP32 particles from 78 to 89 us)
     L.drawn = false;
-    if (early && k > 0 && (int)threadIdx.x < sr.tile && k != sr.resume_k - 1) M::predraw(L, s);
+    if (early && k > sr.resume_k && (int)threadIdx.x < sr.tile) M::predraw(L, s);
   }
   // the uniform of the search whose scalars this CTA may form, from the counter
   // alone: in the wait's shadow
