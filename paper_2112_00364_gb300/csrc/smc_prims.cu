@@ -870,8 +870,10 @@ __global__ void __launch_bounds__(RS_TPB, 3) rs_ancestors(
 
 // Particle duplication: dst[f][i] = src[f][anc[i]], 16-byte stores of
 // consecutive particles; with stack pointers (STACK) row f only for the particles
-// with f < sp[anc[i]].  Rows of whole 16-byte groups without stack pointers, and one
-// or two FP32 rows with them (4.2 M x 1: 10.5 us against 12.4 in the other form).
+// with f < sp[anc[i]].  Rows of whole 16-byte groups without stack pointers, one FP32
+// row of any length without them (4.2 M + 5: 12.3 us against 14.3 in the other form,
+// 2^24 - 1: 37.0 against 53.2), and one or two FP32 rows with them (4.2 M x 1: 10.5
+// against 12.4).
 template <typename T, int V, bool STACK>
 __global__ void gather_kernel(const T* __restrict__ src, T* __restrict__ dst,
                               const int32_t* __restrict__ anc, const int32_t* __restrict__ sp,
@@ -920,8 +922,9 @@ __global__ void gather_kernel(const T* __restrict__ src, T* __restrict__ dst,
 // rows without them 4.2 M 77.7 / 72.0, 1 M 22.8 / 14.5, 10,001 8.3 / 4.3; 8 ragged FP64
 // rows 4.2 M 103 / 84, 1 M 30.9 / 22.7.  Rows of whole 16-byte groups without pointers
 // stay with their 16-byte stores (2^24 x 1 FP32 row 39 against 80).  V, U: 4, 4 for
-// FP32; 2, 4 for FP64 (8 x 4.2 M 84, with 4, 4 96), but 4, 2 for one or two rows with
-// pointers (1 x 4.2 M 16.6 against 20.6).
+// FP32; 2, 4 for FP64 (8 x 4.2 M 84, with 4, 4 96), but for one or two rows 2, 2 without
+// pointers (4.2 M + 5 x 1 16.4 against 20.5, x 2 25.1 / 28.8, x 3 37.1 / 36.8) and 4, 2
+// with them (1 x 4.2 M 16.6 against 20.6).
 constexpr int GA_TPB = 256;
 template <typename T, int V, int U, bool STACK>
 __global__ void __launch_bounds__(GA_TPB) gather_lines_kernel(
@@ -1358,12 +1361,13 @@ extern "C" smc_status smc_gather(const void* src, void* dst, const int32_t* anc,
   if (elem_bytes == 4) {
     if (sp && n_fields > 2) launch_gather_lines<float, 4, 4, true>(src, dst, anc, sp, N, n_fields, cs);
     else if (sp) launch_gather<float, 4, true>(src, dst, anc, sp, N, n_fields, cs);
-    else if (whole) launch_gather<float, 4, false>(src, dst, anc, sp, N, n_fields, cs);
+    else if (whole || n_fields == 1) launch_gather<float, 4, false>(src, dst, anc, sp, N, n_fields, cs);
     else launch_gather_lines<float, 4, 4, false>(src, dst, anc, sp, N, n_fields, cs);
   } else {
     if (sp && n_fields > 2) launch_gather_lines<double, 2, 4, true>(src, dst, anc, sp, N, n_fields, cs);
     else if (sp) launch_gather_lines<double, 4, 2, true>(src, dst, anc, sp, N, n_fields, cs);
     else if (whole) launch_gather<double, 2, false>(src, dst, anc, sp, N, n_fields, cs);
+    else if (n_fields <= 2) launch_gather_lines<double, 2, 2, false>(src, dst, anc, sp, N, n_fields, cs);
     else launch_gather_lines<double, 2, 4, false>(src, dst, anc, sp, N, n_fields, cs);
   }
   SMC_CUDA_TRY(cudaGetLastError());
