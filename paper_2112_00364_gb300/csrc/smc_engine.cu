@@ -731,15 +731,23 @@ bool graph_matches(const GraphCache* g, const WavePlan& W, int precision, int ma
          g->plan.chains == W.chains;
 }
 
-// Capture max_waves waves on `st` into a graph and instantiate it into g.
+// Capture max_waves waves on `st` into a graph and instantiate it into g; with `streams`
+// the chains are branches of the graph.  (One after another in a single branch, a
+// batch of four models with 300 particles and 7 or 8 segments each took 833 us
+// instead of 625, four of 5,000 with 50 segments 4,496 instead of 2,140.)
 smc_status capture_waves(GraphCache* g, const WavePlan& W, int precision, int max_waves,
-                         cudaStream_t st) {
+                         cudaStream_t st, ChainStreams* streams) {
   graph_cache_clear(g);
   SMC_CUDA_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-  cudaError_t e = cudaSuccess;
+  const int n_chains = (int)W.chains.size();
+  cudaError_t e = streams ? streams->fork(st, n_chains) : cudaSuccess;
   int launched = 0;
   for (int k = 0; k < max_waves && e == cudaSuccess; ++k)
-    e = launch_wave(W, precision, st, (unsigned)k, nullptr, &launched);
+    e = launch_wave(W, precision, st, (unsigned)k, streams, &launched);
+  if (streams) {  // after an error too: the branches end with the capture
+    const cudaError_t je = streams->join(st, n_chains);
+    if (e == cudaSuccess) e = je;
+  }
   cudaGraph_t graph = nullptr;
   const cudaError_t e2 = cudaStreamEndCapture(st, &graph);
   if (e != cudaSuccess || e2 != cudaSuccess) {
@@ -775,7 +783,7 @@ smc_status drive_waves(const WavePlan& W, int precision, const std::vector<RunSt
   const int n_chains = (int)W.chains.size();
   if (known && graph && !timed && st != nullptr && st != cudaStreamLegacy) {
     if (!graph_matches(graph, W, precision, max_waves)) {
-      smc_status s = capture_waves(graph, W, precision, max_waves, st);
+      smc_status s = capture_waves(graph, W, precision, max_waves, st, streams);
       if (s) return s;
     }
     SMC_CUDA_TRY(cudaGraphLaunch(graph->exec, st));
@@ -1441,7 +1449,7 @@ extern "C" smc_status smc_run_batch(const smc_model_t* ms, const smc_run_cfg* cf
   GraphCache graph;
   const bool graphed = cfgs[0].launch_mode == SMC_LAUNCH_GRAPH;
   ChainStreams streams;
-  const bool fan = known && !graphed && W.chains.size() > 1;
+  const bool fan = known && W.chains.size() > 1;
   if (fan) SMC_CUDA_TRY(streams.init(std::min((int)W.chains.size(), kChainStreams)));
   st = drive_waves(W, prec, states, max_waves, known, cs, nullptr, false, &launched, &kms,
                    graphed ? &graph : nullptr, fan ? &streams : nullptr);
