@@ -136,16 +136,16 @@ struct WavePlan {
 // chain's waves need not wait for the slowest CTAs of the others' (on one stream
 // every launch waits for the launch before it).  fork(): the chains' work waits for
 // what `main` holds so far; join(): `main` waits for the chains' work so far.
-// Chain i runs on stream i modulo the number of streams.  Owned by one batch call
-// or one server; its streams are idle when it is destroyed (after a join that the
-// owner has waited for).
+// Chain i runs on stream i modulo the number of streams.  Used by one batch call
+// or one server at a time; its streams are idle when it is destroyed (after a join
+// that the owner has waited for).
 class ChainStreams {
  public:
   ChainStreams() = default;
   ChainStreams(const ChainStreams&) = delete;
   ChainStreams& operator=(const ChainStreams&) = delete;
   ~ChainStreams();
-  cudaError_t init(int n);
+  cudaError_t init(int n);  // at least n streams
   cudaError_t fork(cudaStream_t main, int chains);
   cudaError_t join(cudaStream_t main, int chains);
   cudaStream_t at(int chain) const { return s_[(size_t)chain % s_.size()]; }
@@ -155,6 +155,24 @@ class ChainStreams {
   std::vector<cudaStream_t> s_;
   std::vector<cudaEvent_t> done_;
   cudaEvent_t ready_ = nullptr;
+};
+
+// The streams of one batch call: a set that an earlier call left idle, or a new one; left
+// for later calls once idle() was called, destroyed otherwise (after an error).
+class BorrowedStreams {
+ public:
+  BorrowedStreams() = default;
+  BorrowedStreams(const BorrowedStreams&) = delete;
+  BorrowedStreams& operator=(const BorrowedStreams&) = delete;
+  ~BorrowedStreams();
+  cudaError_t take(int n);
+  void idle() { idle_ = true; }
+  ChainStreams* get() const { return set_; }
+
+ private:
+  ChainStreams* set_ = nullptr;
+  int dev_ = 0;
+  bool idle_ = false;
 };
 
 // An instantiated CUDA graph of a known-length sequence of waves and the wave
