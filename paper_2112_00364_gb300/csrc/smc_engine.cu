@@ -507,10 +507,6 @@ Layout make_layout(const smc_model_s* m, const smc_run_cfg* c) {
     L.stack[b] = take(rb * N * (size_t)m->stack_cap);
   }
   L.logw = take(8 * N);
-  for (int b = 0; b < 2; ++b) {
-    L.E[b] = take(8 * (size_t)L.n_tiles * (size_t)L.pad);
-    L.ends[b] = take(L.pad > 32 ? 64 * (size_t)L.n_tiles : 0);
-  }
   L.rec[0] = take(sizeof(TileRec) * (size_t)L.n_tiles);
   L.rec[1] = take(sizeof(TileRec) * (size_t)L.n_tiles);
   L.tq[0] = take(8 * (size_t)L.n_tiles);
@@ -520,12 +516,22 @@ Layout make_layout(const smc_model_s* m, const smc_run_cfg* c) {
   L.rs = take(sizeof(RunState));
   L.anc = take(4 * N * (size_t)L.anc_rows);
   L.incr = take(8 * (size_t)L.max_segments);
+  // the running sums, and in their place, once the run has ended, its outputs for the
+  // host: in arrays of their own, or (up to kStageMax) in one block that takes one copy
+  const size_t sums = off;
+  for (int b = 0; b < 2; ++b) {
+    L.E[b] = take(8 * (size_t)L.n_tiles * (size_t)L.pad);
+    L.ends[b] = take(L.pad > 32 ? 64 * (size_t)L.n_tiles : 0);
+  }
+  const size_t sums_end = off;
+  off = sums;
   L.fin_real = take(8 * N * (size_t)m->n_real);
   L.fin_int = take(4 * N * (size_t)m->n_int);
   L.fin_stack = take(8 * N * (size_t)m->stack_cap);
-  // host results up to kStageMax go out through one block and one copy
   const size_t stage = stage_bytes(m, (int64_t)N);
-  L.stage = take(!c->record_all_ancestors && stage <= kStageMax ? stage : 0);
+  L.stage = sums;
+  if (!c->record_all_ancestors && stage <= kStageMax) off = std::max(off, align_up(sums + stage, 256));
+  off = std::max(off, sums_end);
   // a host snapshot to resume from is copied here
   L.snap = take(c->resume_k > 0 && c->resume_where == SMC_MEM_HOST
                     ? (8 + 8 * (size_t)m->n_real + 8 * (size_t)m->stack_cap) * N + 4 * N * (size_t)m->n_int
@@ -705,8 +711,9 @@ cudaError_t launch_wave(const WavePlan& W, int precision, cudaStream_t st, unsig
 size_t wave_meta_bytes(const std::vector<RunDev>& runs) {
   size_t n_ctas = 0;
   for (const RunDev& r : runs) n_ctas += (size_t)r.n_tiles;
+  // (each chain's map starts on a boundary; every run belongs to one chain)
   return align_up(sizeof(RunDev) * runs.size(), 256) + align_up(sizeof(int2) * n_ctas, 256) +
-         kMaxChains * 256;
+         std::min(runs.size(), (size_t)kMaxChains) * 256;
 }
 
 size_t fill_plan(const std::vector<RunDev>& runs, char* host, void* dev, WavePlan* W,
