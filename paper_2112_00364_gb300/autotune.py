@@ -4,7 +4,9 @@ A run of N particles is cut into tiles, one CTA per tile and wave; the tile
 size must be a function of N alone (it fixes how the weights are rounded, so a
 run gives the same bits alone, batched and served).  The library reads it from
 a table of N bands (csrc/smc_tile_table.inc): the band with the smallest
-n_max >= N gives tiles of clamp(ceil(N / slots), tile_min, tile_max).
+n_max >= N gives tiles of clamp(ceil(N / slots), tile_min, tile_max).  The
+built-in table is not this sweep's: its bands were chosen by hand from sweeps of
+single runs at 27 sizes and of mixed batches, so that no single run lost time.
 
 For every band this script times each candidate rule on a representative N:
   - a batch of 48 runs of that N (half linear-Gaussian with T = 50, half CRBD
@@ -13,14 +15,15 @@ For every band this script times each candidate rule on a representative N:
     single run),
 each the median of repeated CUDA-event timings, and scores a candidate by the
 mean of log(throughput / best throughput) over the three.  The best candidate
-of each band is written to csrc/smc_tile_table.inc (adjacent bands with the
-same choice merged), and the whole sweep to the file given by --report.
+of each band is written to smc_tile_table.inc in the working folder, or the file
+given by --table (adjacent bands with the same choice merged), and the whole sweep
+to the file given by --report.
 
     python -m paper_2112_00364_gb300.autotune [--report FILE] [--table FILE] [--dry-run]
 
 It needs a CUDA device; the library must be built (python -c "import
-__graft_entry__ as g; g.build()").  Rebuild the library afterwards to compile
-the new table in.
+__graft_entry__ as g; g.build()").  To use a table, name the built-in file with
+--table and rebuild the library.
 """
 from __future__ import annotations
 
@@ -33,7 +36,7 @@ from pathlib import Path
 
 PKG = Path(__file__).resolve().parent
 ROOT = PKG.parent
-TABLE = PKG / "csrc" / "smc_tile_table.inc"
+TABLE = Path("smc_tile_table.inc")
 
 # band upper edges (particles); the last band reaches the largest run
 EDGES = [256, 512, 1024, 2048, 4096, 8192, 16384, 32768, 65536, 131072, 0x7FFFFFFF]
