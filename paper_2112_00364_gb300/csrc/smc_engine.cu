@@ -301,8 +301,9 @@ int model_fields(int kind, int* n_real, int* n_int) {
 }
 
 // ---- tiling: a function of N alone, from a table of N bands ----
-// The built-in table is data written by the autotuner (autotune.py sweeps the
-// candidate rules per band on a GB300 and writes smc_tile_table.inc); a band
+// The built-in table (smc_tile_table.inc) is data from sweeps of single runs and mixed
+// batches on a GB300, with the lines chosen by hand (autotune.py sweeps batches of equal
+// runs, weighs batches and single runs alike and would choose other bands); a band
 // {n_max, slots, tile_min, tile_max} gives a run of N <= n_max particles tiles
 // of clamp(ceil(N / slots), tile_min, tile_max) particles.  Because the tile of
 // a run depends on its N alone, a run gives the same bits alone, batched and

@@ -86,8 +86,8 @@ __device__ __forceinline__ long long load_from_cta(const long long* p, unsigned 
 // sums in one load (lane l holds E_{j0+l}, from the shared memory of the tile's CTA)
 // and every lane of that tile finds
 // its first j with E_j > F by a binary search over the shuffled values.  The
-// same ancestors and near-boundary flags as systematic_search; one dependent
-// load of the sums instead of the 8-ary search's two.  Every lane calls it;
+// same ancestors and near-boundary flags as systematic_search, which reads a tile's
+// sums in two rounds; a tile here is one warp.  Every lane calls it;
 // `want` marks the lanes whose offset is searched.
 template <int WPC, bool CL>
 __device__ __forceinline__ int small_search(int i, bool want, const RunDev& A, const SearchCtx& X,

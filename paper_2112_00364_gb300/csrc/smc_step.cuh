@@ -630,7 +630,9 @@ __global__ void __launch_bounds__(TPB, min_ctas(resident_threads<R, KIND>(TPB, D
   // the places that happen to come free, two CTAs of a wave on one SM beside idle ones:
   // SEIR FP32 with 122 CTAs of 128 195 us a day, after the wait 114; CRBD with delayed
   // sampling 30.7 / 24.3.  Only the models that draw ahead, whose blocks are short, are
-  // faster so in CTAs of 256: 23,171 FP64 7.26 us a wave, 7.68 after the wait.)
+  // faster so in CTAs of 256: nine sizes from 20,000 to 38,912 linear-Gaussian particles,
+  // us a wave so / after the wait: FP64 all faster, 7.24 / 7.50 to 7.61 / 8.19; FP32 seven
+  // faster, 6.80 / 6.86 to 7.01 / 7.17, two not (20,000 6.79 / 6.71, 31,000 6.75 / 6.66).)
   const bool ahead = early && M::PREDRAW && TPB == 256;
   if (ahead) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int k = (int)(wave - sr.start_wave);  // wraps correctly past 2^32 waves
