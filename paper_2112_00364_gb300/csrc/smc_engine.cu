@@ -508,15 +508,6 @@ Layout make_layout(const smc_model_s* m, const smc_run_cfg* c) {
     L.stack[b] = take(rb * N * (size_t)m->stack_cap);
   }
   L.logw = take(8 * N);
-  L.rec[0] = take(sizeof(TileRec) * (size_t)L.n_tiles);
-  L.rec[1] = take(sizeof(TileRec) * (size_t)L.n_tiles);
-  L.tq[0] = take(8 * (size_t)L.n_tiles);
-  L.tq[1] = take(8 * (size_t)L.n_tiles);
-  L.dec = take(4 * (size_t)L.max_segments);
-  L.tO = take(8 * (size_t)(L.n_tiles + 1));
-  L.rs = take(sizeof(RunState));
-  L.anc = take(4 * N * (size_t)L.anc_rows);
-  L.incr = take(8 * (size_t)L.max_segments);
   // the running sums, and in their place, once the run has ended, its outputs for the
   // host: in arrays of their own, or (up to kStageMax) in one block that takes one copy
   const size_t sums = off;
@@ -533,6 +524,15 @@ Layout make_layout(const smc_model_s* m, const smc_run_cfg* c) {
   L.stage = sums;
   if (!c->record_all_ancestors && stage <= kStageMax) off = std::max(off, align_up(sums + stage, 256));
   off = std::max(off, sums_end);
+  L.rec[0] = take(sizeof(TileRec) * (size_t)L.n_tiles);
+  L.rec[1] = take(sizeof(TileRec) * (size_t)L.n_tiles);
+  L.tq[0] = take(8 * (size_t)L.n_tiles);
+  L.tq[1] = take(8 * (size_t)L.n_tiles);
+  L.dec = take(4 * (size_t)L.max_segments);
+  L.tO = take(8 * (size_t)(L.n_tiles + 1));
+  L.rs = take(sizeof(RunState));
+  L.anc = take(4 * N * (size_t)L.anc_rows);
+  L.incr = take(8 * (size_t)L.max_segments);
   // a host snapshot to resume from is copied here
   L.snap = take(c->resume_k > 0 && c->resume_where == SMC_MEM_HOST
                     ? (8 + 8 * (size_t)m->n_real + 8 * (size_t)m->stack_cap) * N + 4 * N * (size_t)m->n_int
