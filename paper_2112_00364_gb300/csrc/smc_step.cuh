@@ -480,7 +480,9 @@ __device__ __forceinline__ void step_tile(const RunDev& A, const int t, const in
   // of them fell on two words in a wave of 2^20 particles; that, a fence by every
   // thread and two more barriers took 20 of the rate-shift model's 178 us a wave.)
   // Kills are rare.
-  const unsigned draws = __reduce_add_sync(0xffffffffu, active ? s.d : 0u);
+  // (a stopped particle's stream has moved only where a draw was taken ahead)
+  const unsigned draws =
+      __reduce_add_sync(0xffffffffu, (M::PREDRAW && early ? active : valid) ? s.d : 0u);
   const unsigned execs = __reduce_add_sync(0xffffffffu, (unsigned)n_exec);
   const unsigned kills = __reduce_add_sync(
       0xffffffffu, active ? (unsigned)L.overflow | ((unsigned)L.limited << 16) : 0u);
