@@ -619,11 +619,13 @@ cudaError_t ChainStreams::init(int n) {
 }
 
 namespace {
-// Idle sets of batch calls that have ended, at most kIdleSets of them (a set is in one
-// call's hands or here; calls beyond that destroy theirs).  With its streams and events
+// Idle sets of batch calls that have ended, at most kIdleSets of kIdleStreams each (a set
+// is in one call's hands or here; other sets are destroyed).  With its streams and events
 // made and destroyed in each call, a batch of two small runs took 374 us instead of 334,
-// one of four models 584 instead of 531.
-constexpr size_t kIdleSets = 4;
+// one of four models 584 instead of 531.  Batches of more chains are larger and would not
+// notice; their streams, kept, slowed a server's bursts by 0.7% (25.87 -> 26.06 ms).
+constexpr size_t kIdleSets = 2;
+constexpr int kIdleStreams = 4;
 std::mutex g_idle_mu;
 std::vector<std::pair<int, ChainStreams*>> g_idle;  // device, set
 }  // namespace
@@ -632,7 +634,7 @@ BorrowedStreams::~BorrowedStreams() {
   if (!set_) return;
   {
     std::lock_guard<std::mutex> lock(g_idle_mu);
-    if (idle_ && g_idle.size() < kIdleSets) {
+    if (idle_ && set_->size() <= kIdleStreams && g_idle.size() < kIdleSets) {
       g_idle.emplace_back(dev_, set_);
       return;
     }
@@ -647,7 +649,7 @@ cudaError_t BorrowedStreams::take(int n) {
     std::lock_guard<std::mutex> lock(g_idle_mu);
     g_idle.reserve(kIdleSets);
     for (size_t q = 0; q < g_idle.size() && !set_; ++q)
-      if (g_idle[q].first == dev_) {
+      if (n <= kIdleStreams && g_idle[q].first == dev_) {
         set_ = g_idle[q].second;
         g_idle.erase(g_idle.begin() + (long)q);
       }
