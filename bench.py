@@ -88,15 +88,15 @@ RS_BYTES = 20          # logw read twice (normaliser, scan) + ancestor written, 
 # rate for the delayed-sampling CRBD (FP64 pipe busy 25-40% of a launch).  The
 # traffic holds only for the kernel sources with the recorded digest.
 NCU = {"crbd64": dict(basis="issue", warp_inst_per_pstep=99.4, fp64_flop_per_pstep=16.9,
-                      bytes_per_launch=3.779e6, fp64_pipe_elapsed=0.147,
-                      src_digest="b221f7c0c8e901e4"),
+                      bytes_per_launch=3.776e6, fp64_pipe_elapsed=0.147,
+                      src_digest="a45363317455a27f"),
        "crbd_ds128": dict(basis="fp64", warp_inst_per_pstep=75.3, fp64_flop_per_pstep=91.7,
-                          bytes_per_launch=5.398e6, fp64_pipe_elapsed=0.315,
-                          src_digest="b221f7c0c8e901e4"),
+                          bytes_per_launch=5.404e6, fp64_pipe_elapsed=0.314,
+                          src_digest="a45363317455a27f"),
        # FP32 waves of 2^20 particles: bound by memory latency (long-scoreboard
        # stalls), reported against HBM; 61-85 warp instructions per particle-step
        "rateshift256": dict(basis="hbm", warp_inst_per_pstep=69.2, bytes_per_launch=1.114e8,
-                            src_digest="b221f7c0c8e901e4")}
+                            src_digest="a45363317455a27f")}
 
 # 152 SMs x 2070 MHz x 4 FP64 flop/clk/SM (2 DFMA/clk/SM) = GB300's FP64 rate
 FP64_PEAK_FLOPS = 152 * 2070e6 * 4
@@ -115,7 +115,7 @@ RS_SOURCES = ("smc_prims.cu", "smc_device.cuh", "smc_combine.cuh")
 # DRAM traffic of one smc_resample call at 2^24 (the three kernels' dram__bytes
 # read + write in one ncu capture, profiles folder), valid for the sources with
 # the recorded digest.
-RS_NCU = dict(bytes_per_call=2.350e8, src_digest="46cea9ab26127de1")
+RS_NCU = dict(bytes_per_call=2.348e8, src_digest="46cea9ab26127de1")
 
 
 def code_text(src: str) -> str:
